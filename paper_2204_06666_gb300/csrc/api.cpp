@@ -152,6 +152,44 @@ ehyb_status_t device_query(int* dev, int* sms, int* smem_optin) {
 ehyb_status_t device_alloc(void** p, size_t bytes) { return dev_alloc(p, bytes); }
 
 // device view of a plan for entry points defined in other translation units
+WideLists wide_lists(int32_t nparts, const std::vector<int32_t>& slice_ptr, const std::vector<int64_t>& slice_pos,
+                     const std::vector<int64_t>& er_slice_pos) {
+  WideLists L;
+  const size_t ns = slice_ptr.empty() ? 0 : (size_t)slice_ptr.back();
+  auto width = [](const std::vector<int64_t>& pos, size_t s) { return (int32_t)((pos[s + 1] - pos[s]) >> 5); };
+  bool any = false;
+  for (size_t s = 0; s < ns && !any; ++s)
+    any = width(slice_pos, s) > kWideCap || width(er_slice_pos, s) > kWideCap;
+  if (!any) return L;
+  L.slice_wide.assign(ns, -1);
+  L.unit_ptr.assign((size_t)nparts + 1, 0);
+  L.wide_ptr.assign((size_t)nparts + 1, 0);
+  for (int32_t p = 0; p < nparts; ++p) {
+    const size_t u0 = L.units.size();
+    for (int32_t s = slice_ptr[(size_t)p]; s < slice_ptr[(size_t)p + 1]; ++s) {
+      const int32_t w[2] = {width(slice_pos, (size_t)s), width(er_slice_pos, (size_t)s)};
+      if (w[0] <= kWideCap && w[1] <= kWideCap) continue;
+      L.slice_wide[(size_t)s] = L.parts;
+      WideSlice ws{s, L.parts++, 0, 0};
+      for (int er = 0; er < 2; ++er)
+        for (int32_t k = kWideCap; k < w[er]; k += kWideCap) {
+          const int64_t pos = (er ? er_slice_pos : slice_pos)[(size_t)s] + 32 * (int64_t)k;
+          L.units.push_back({pos, std::min(w[er] - k, kWideCap), er, L.parts++, 0});
+          ++ws.count;
+        }
+      L.wides.push_back(ws);
+    }
+    // longest first; an extra-row slot gathers x from global memory and counts twice, as in the slice order
+    std::stable_sort(L.units.begin() + (long)u0, L.units.end(), [](const WideUnit& a, const WideUnit& b) {
+      return a.w * (1 + a.er) > b.w * (1 + b.er);
+    });
+    L.unit_ptr[(size_t)p + 1] = (int32_t)L.units.size();
+    L.wide_ptr[(size_t)p + 1] = (int32_t)L.wides.size();
+    L.max_items = std::max(L.max_items, slice_ptr[(size_t)p + 1] - slice_ptr[(size_t)p] + (int32_t)(L.units.size() - u0));
+  }
+  return L;
+}
+
 const DevPlan* plan_device_view(ehyb_plan_t plan, int* device) {
   if (!plan || plan->host_only) return nullptr;
   if (device) *device = plan->device;
@@ -365,8 +403,31 @@ ehyb_status_t plan_finalize(std::unique_ptr<ehyb_plan_s>& P, const ehyb_options_
   D.nparts = H.nparts;
   D.tpr = H.tpr;
   D.er_tpr = P->er_tpr;
+  WideLists W;
+  try {
+    if (H.er_layout == 0) {
+      W = wide_lists(H.nparts, H.slice_ptr, H.slice_pos, H.er_slice_pos);
+    } else if (H.er_layout == 2 && H.tpr == 1) {  // flags only: these slices hold both parts of a row in one
+      for (int64_t r = 0; r < n; ++r)
+        if (H.row_ell_count[(size_t)r] > kWideCap || H.row_er_count[(size_t)r] > kWideCap) W.parts = 1;
+      if (W.parts) {
+        W.slice_wide.assign((size_t)H.nslices, -1);
+        for (int32_t p = 0; p < H.nparts; ++p)
+          for (int32_t r = H.part_ptr[(size_t)p]; r < H.part_ptr[(size_t)p + 1]; ++r)
+            if (H.row_ell_count[(size_t)r] > kWideCap || H.row_er_count[(size_t)r] > kWideCap)
+              W.slice_wide[(size_t)(H.slice_ptr[(size_t)p] + (r - H.part_ptr[(size_t)p]) / 32)] = 0;
+        W.unit_ptr.assign((size_t)H.nparts + 1, 0);
+        W.wide_ptr.assign((size_t)H.nparts + 1, 0);
+      }
+    }
+  } catch (const std::bad_alloc&) {
+    return EHYB_ERR_OOM;
+  }
+  D.wide_parts = W.parts;
   if (opt.block_threads == 0) {  // enough warps for the average partition's slices
-    const int64_t per_part = H.nparts ? ((int64_t)H.nslices + H.nparts - 1) / H.nparts : 1;
+    int64_t per_part = H.nparts ? ((int64_t)H.nslices + H.nparts - 1) / H.nparts : 1;
+    // ... and, when every partition has an SM to itself, for the units of the one with the most
+    if (W.max_items > per_part && H.nparts <= d.sms) per_part = W.max_items;
     opt.block_threads = (int32_t)std::min<int64_t>(1024, std::max<int64_t>(128, 32 * per_part));
   }
   D.threads = opt.block_threads;
@@ -416,6 +477,15 @@ ehyb_status_t plan_finalize(std::unique_ptr<ehyb_plan_s>& P, const ehyb_options_
     const size_t o_hp = A.add<int64_t>(H.halo_ptr.size());
     const size_t o_hn = A.add<int32_t>(H.halo_new.size());
     const size_t o_ho = A.add<int32_t>(H.halo_old.size());
+    const bool halo_wide = W.parts > 0 && H.er_layout == 2;
+    const size_t o_sw = A.add<int32_t>(W.slice_wide.size());
+    const size_t o_up = A.add<int32_t>(W.unit_ptr.size());
+    const size_t o_un = A.add<WideUnit>(W.units.size());
+    const size_t o_wp = A.add<int32_t>(W.wide_ptr.size());
+    const size_t o_ws = A.add<WideSlice>(W.wides.size());
+    const size_t o_ww = A.add<double>(32 * (size_t)W.parts);
+    const size_t o_rc = A.add<int32_t>(halo_wide ? (size_t)n : 0);
+    const size_t o_re = A.add<int32_t>(halo_wide ? (size_t)n : 0);
     const size_t o_xp = A.add<double>((size_t)n + 2);
     const size_t o_xp32 = A.add<float>((size_t)n + 4);
     const size_t o_st = A.add<int32_t>(4);
@@ -436,6 +506,10 @@ ehyb_status_t plan_finalize(std::unique_ptr<ehyb_plan_s>& P, const ehyb_options_
     UP(o_erv16, H.er_val_bf16) UP(o_esp, H.er_slice_pos) UP(o_so, H.slice_order) UP(o_esc, H.er_scol) UP(o_eso, H.er_scol_old) UP(o_esv, H.er_sval)
     UP(o_esv32, H.er_sval_f32) UP(o_esv16, H.er_sval_bf16) UP(o_ecl, H.ell_col_low) UP(o_escl, H.er_scol_low)
     UP(o_esol, H.er_scol_old_low) UP(o_hp, H.halo_ptr) UP(o_hn, H.halo_new) UP(o_ho, H.halo_old)
+    UP(o_sw, W.slice_wide) UP(o_up, W.unit_ptr) UP(o_un, W.units) UP(o_wp, W.wide_ptr) UP(o_ws, W.wides)
+    if (halo_wide) {
+      UP(o_rc, H.row_ell_count) UP(o_re, H.row_er_count)
+    }
 #undef UP
     if (e == cudaSuccess) e = cudaMemsetAsync(base + o_st, 0, 16, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(base + o_xp, 0, ((size_t)n + 2) * 8, s);
@@ -471,6 +545,16 @@ ehyb_status_t plan_finalize(std::unique_ptr<ehyb_plan_s>& P, const ehyb_options_
     D.halo_ptr = (const int64_t*)(base + o_hp);
     D.halo_new = (const int32_t*)(base + o_hn);
     D.halo_old = (const int32_t*)(base + o_ho);
+    if (W.parts > 0) {
+      D.slice_wide = (const int32_t*)(base + o_sw);
+      D.unit_ptr = (const int32_t*)(base + o_up);
+      D.units = (const WideUnit*)(base + o_un);
+      D.wide_ptr = (const int32_t*)(base + o_wp);
+      D.wides = (const WideSlice*)(base + o_ws);
+      D.wide_ws = (double*)(base + o_ww);
+      D.row_cin = halo_wide ? (const int32_t*)(base + o_rc) : nullptr;
+      D.row_cer = halo_wide ? (const int32_t*)(base + o_re) : nullptr;
+    }
     D.lowp_group = H.lowp_group;
     D.ell_col_low = H.lowp_group == 1 ? D.ell_col : (const uint16_t*)(base + o_ecl);
     D.er_scol_low = H.lowp_group == 1 ? D.er_scol : (const int32_t*)(base + o_escl);

@@ -56,7 +56,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1) batch_kernel(const BatchPlan* 
     const BatchPlan& bp = plans[tl.x];
     double* xs = reinterpret_cast<double*>(smem_raw);
     const bool ok =
-        bp.kbatch == 6
+        bp.a.wide_parts > 0
+            ? partition_spmv<double, double, true, true, false, true, kBatch, false, false, false, true>(
+                  bp.a, bp.ell_val, bp.er_val, bp.x, bp.y, tl.y, xs, bs)
+        : bp.kbatch == 6
             ? partition_spmv<double, double, true, true, false, true, 6>(bp.a, bp.ell_val, bp.er_val, bp.x, bp.y,
                                                                          tl.y, xs, bs)
             : partition_spmv<double, double, true, true, false, true>(bp.a, bp.ell_val, bp.er_val, bp.x, bp.y, tl.y,
@@ -174,11 +177,19 @@ extern "C" ehyb_status_t ehyb_batch_create(int32_t count, const ehyb_plan_t* pla
 
   const size_t t_bytes = ((size_t)count * sizeof(BatchPlan) + 255) & ~(size_t)255;
   const size_t l_bytes = ((size_t)std::max(b->ntiles, 1) * sizeof(int2) + 255) & ~(size_t)255;
-  ehyb_status_t st = device_alloc(&b->arena, t_bytes + l_bytes + 256);
+  // partial sums of the plans' wide slices: the batch's own, since a plan may be in it more than once
+  size_t wide = 0;
+  for (BatchPlan& bp : b->table) wide += (size_t)bp.a.wide_parts * 32 * sizeof(double);
+  ehyb_status_t st = device_alloc(&b->arena, t_bytes + l_bytes + 256 + wide);
   if (st != EHYB_OK) { batch_free(b); return st; }
   b->d_table = (BatchPlan*)b->arena;
   b->d_tiles = (int2*)((char*)b->arena + t_bytes);
   b->d_counters = (int*)((char*)b->arena + t_bytes + l_bytes);
+  double* ww = (double*)((char*)b->arena + t_bytes + l_bytes + 256);
+  for (BatchPlan& bp : b->table) {
+    bp.a.wide_ws = ww;
+    ww += (size_t)bp.a.wide_parts * 32;
+  }
   e = cudaMemcpy(b->d_table, b->table.data(), (size_t)count * sizeof(BatchPlan), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && b->ntiles)
     e = cudaMemcpy(b->d_tiles, sorted.data(), sorted.size() * sizeof(int2), cudaMemcpyHostToDevice);

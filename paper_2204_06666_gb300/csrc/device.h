@@ -5,6 +5,20 @@
 
 namespace ehyb {
 
+// Chunk of a lane's slots that one chain of FMAs sums, in the slab and in the extra rows of a slice alike
+// (ehyb_core.cuh, wide slices).  A multiple of 4, so that a chunk of the copies in runs of four starts on a run;
+// above 81, so that the rows of 3D elasticity stay one chain.
+constexpr int kWideCap = 96;
+struct WideUnit {  // one later chunk of a wide slice
+  int64_t pos;     // its first slot in the slab (er 0) or extra-row (er 1) arrays
+  int32_t w, er;   // slots per lane
+  int32_t part;    // where its sums go in the workspace
+  int32_t pad;
+};
+struct WideSlice {  // parts part .. part + count of slice s: the first chunks, then `count` later ones in order
+  int32_t s, part, count, pad;
+};
+
 // Plan arrays on the device (names after the paper: part_ptr = partBoundary, slice_pos =
 // PositionELL, ell_col = ColELL, ell_val = ValELL, er_row = yIdxER).
 struct DevPlan {
@@ -48,6 +62,17 @@ struct DevPlan {
   const uint16_t* ell_col_low = nullptr;
   const int32_t* er_scol_low = nullptr;
   const int32_t* er_scol_old_low = nullptr;
+  // wide slices (wide_parts > 0; wide_lists in plan.h): part of each slice or -1, units and wide slices by
+  // partition, workspace of the partial sums.  er_layout 2: a flag per slice and the entry counts of each row
+  int32_t wide_parts = 0;
+  const int32_t* slice_wide = nullptr;
+  const int32_t* unit_ptr = nullptr;
+  const WideUnit* units = nullptr;
+  const int32_t* wide_ptr = nullptr;
+  const WideSlice* wides = nullptr;
+  double* wide_ws = nullptr;
+  const int32_t* row_cin = nullptr;
+  const int32_t* row_cer = nullptr;
   int32_t* status = nullptr;  // device status word (first fault wins)
   uint64_t wait_timeout_ns = 1000000000ull;
   int32_t inject_wait_fault = 0;

@@ -419,6 +419,17 @@ __device__ __forceinline__ X er_dot_runs(const V* __restrict__ vb, const int32_t
   return acc;
 }
 
+// ---- wide slices.  A lane sums its slots one after the other, so a slice with a row of thousands of entries was
+// one chain of dependent loads and FMAs thousands of slots long while the other warps had nothing left to do
+// (power-law matrix, 200k rows, longest slice 3,299 slots a lane: 442 us for 2 M entries, 100 us now; what is left is
+// the block with the most padded slots, 7,706 a warp lane at about 20 cycles each).  The slots of a slice
+// are therefore summed in chunks of kWideCap a lane: acc0 = the first kWideCap slab slots, then the first
+// kWideCap extra-row slots, as one chain; every later chunk of the slab, then of the extra rows, is a chain of
+// its own (one unit of work, taken by any warp of the block); the row is acc0 + ((c1 + c2) + c3 ...).  A slice of
+// at most kWideCap slots in each part has no later chunk and keeps its single chain, so 81-entry elasticity
+// rows and narrower ones are summed as before.  Every path sums in this order (the products, the batch, SpMM,
+// the shards and er_layout 2), so their results stay equal bit for bit.
+
 struct KArgs {
   int32_t tpr_log2, er_tpr_log2;
   int64_t n;              // rows of the matrix (of y)
@@ -448,9 +459,46 @@ struct KArgs {
   int32_t* dot_arrive;    // optional (with dot_part, one block per partition): arrival counter; the last
   double* dot_result;     //   block reduces the partials into *dot_result and resets the counter
   const int32_t* skip;    // optional: the launch does nothing while *skip != 0 (converged solver)
+  // wide slices (WIDE kernels; see wide_cap): a wide slice's part index or -1, the units and the wide slices of
+  // each partition, and the workspace of the parts' partial sums (32 lanes each, 8 bytes apart)
+  const int32_t* slice_wide;
+  const int32_t* unit_ptr;
+  const WideUnit* units;
+  const int32_t* wide_ptr;
+  const WideSlice* wides;
+  double* wide_ws;
+  int32_t wide_parts;     // parts in the workspace (checked build only)
+  const int32_t* row_cin;   // er_layout 2 with one lane per row: slab / extra entries of each row (else null)
+  const int32_t* row_cer;
   int32_t meta_off;       // byte offset of the partition's slice table in dynamic shared memory (0: none)
   int32_t meta_cap;       //   ... and its capacity in entries (checked build only)
 };
+
+// er_layout 2 (one lane per row): a lane's slots hold its cin slab entries and then its cer extra entries; the
+// same chunks as above, each lane at its own boundaries (w slots, the slice's widest row)
+template <typename V, typename X, bool RUNS>
+__device__ __forceinline__ X halo_wide_dot(const V* __restrict__ vb, const uint16_t* __restrict__ cb, int lane, int w,
+                                           int cin, int cer, const X* xs, int lim, int32_t* status) {
+  X acc0 = X(0), t = X(0), cur = X(0);
+  const int wg = RUNS ? (w & ~3) : 0;
+#pragma unroll 4
+  for (int k = 0; k < w; ++k) {
+    const int64_t o = k < wg ? 128 * (int64_t)(k >> 2) + 4 * lane + (k & 3) : 32 * (int64_t)k + lane;
+    const X v = load_val<V, X>(vb + o);
+    const X xv = xs[checked((int)__ldcs(reinterpret_cast<const unsigned short*>(cb + o)), lim, status)];
+    const int e = k < cin ? k : k - cin;  // entry of the slab part, then of the extra part
+    if (e < kWideCap) {
+      acc0 = fma_t(v, xv, acc0);
+    } else {
+      cur = fma_t(v, xv, cur);
+      if (e % kWideCap == kWideCap - 1 || k == cin - 1 || k == cin + cer - 1) {
+        t += cur;
+        cur = X(0);
+      }
+    }
+  }
+  return acc0 + t;
+}
 
 // One slice of a partition in its processing order, as the block keeps it in shared memory: where its slab
 // and extra-row slots start and how many slots a lane has in each.  Staged once per partition, so a warp
@@ -504,14 +552,18 @@ struct BlockState {
 // out of time.
 // TABLE: the launch may provide the partition's slice table (a.meta_off); without it only the global path is
 // compiled (the persistent batch kernel, whose blocks run many partitions one after the other).
+// WIDE: the plan has wide slices.
+// sub, nsub: the block takes every nsub-th slice of the processing order, from the sub-th on (nsub > 1: several
+// blocks share a partition of a batch; not with WIDE, whose partial sums are combined by one block).
 // PDL: the kernel was launched with programmatic stream serialization and has not yet waited for the previous
 // grid: the slice table, which reads plan arrays only, is filled first, then griddepcontrol.wait, then every
 // read of x (and of the solver's skip flag) and every write of y.
 template <typename V, typename X, bool SCATTER, bool ER_SLICED, bool DOT = false, bool GATHER = false,
-          int KB = kBatch, bool RUNS = false, bool TABLE = false, bool PDL = false>
+          int KB = kBatch, bool RUNS = false, bool TABLE = false, bool PDL = false, bool WIDE = false>
 __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restrict__ ell_val,
                                                const V* __restrict__ er_val, const X* __restrict__ xp,
-                                               X* __restrict__ y, const int p, X* xs, BlockState& bs) {
+                                               X* __restrict__ y, const int p, X* xs, BlockState& bs,
+                                               const int sub = 0, const int nsub = 1) {
   constexpr int EPV = 16 / (int)sizeof(X);  // elements per 16 bytes
   const int tid = threadIdx.x;
   const int lane = tid & 31;
@@ -626,17 +678,35 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
 
   const X* xsl = xs + (pb - a0);  // xsl[local column] = x_p[pb + local column]
   const int tpr = 1 << a.tpr_log2;
-  const int sub = lane & (tpr - 1);
+  const int sub_lane = lane & (tpr - 1);
   const int rows_per_slice = 32 >> a.tpr_log2;
 
   // ---- 2. slab: warp per 32-lane slice, dynamic slice balancing inside the partition
   // (static round-robin when the fused dot product is requested, so its order is fixed)
   constexpr bool dot = DOT;  // a.dot_part is set
   double dacc = 0.0;
-  // metadata of the slice at position j of the processing order (j < s1): from the table, else from global
-  auto slice_meta = [&](int j, int& sj, int64_t& posj, int& wj, int64_t& eposj, int& wej) {
+  // work items of the block: with WIDE the partition's units first, then its slices in processing order
+  const int u0 = WIDE ? a.unit_ptr[p] : 0;
+  const int nu = WIDE ? a.unit_ptr[p + 1] - u0 : 0;
+  const int items = s0 + (nu + ns - sub + nsub - 1) / nsub;
+  // item j < items: the slice at its position of the processing order (from the table, else from global), or a
+  // unit (sj = -1 - its part index): a chunk of either a slab or an extra-row part
+  auto item_meta = [&](int j, int& sj, int64_t& posj, int& wj, int64_t& eposj, int& wej) {
+    int t = sub + nsub * (j - s0);
+    if (WIDE) {
+      if (t < nu) {
+        const WideUnit u = a.units[u0 + t];
+        sj = -1 - u.part;
+        posj = u.pos;
+        eposj = u.pos;
+        wj = u.er ? 0 : u.w;
+        wej = u.er ? u.w : 0;
+        return;
+      }
+      t -= nu;
+    }
     if (tbl) {
-      const SliceMeta m = tbl[checked(j - s0, a.meta_cap, a.status)];
+      const SliceMeta m = tbl[checked(t, a.meta_cap, a.status)];
       sj = m.s;
       posj = m.pos;
       wj = m.w;
@@ -644,7 +714,7 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
       wej = m.we;
       return;
     }
-    sj = a.slice_order[j];
+    sj = a.slice_order[s0 + t];
     posj = a.slice_pos[sj];
     wj = (int)((a.slice_pos[sj + 1] - posj) >> 5);
     if (ER_SLICED) {
@@ -652,13 +722,23 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
       wej = (int)((a.er_slice_pos[sj + 1] - eposj) >> 5);
     }
   };
-  int i = s0 + warp;  // position in the partition's processing order
+  // store the rows of slice sl from their lanes' sums (and add them to the fused dot product)
+  auto store_rows = [&](int sl, X acc) {
+    for (int off = tpr >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(FULL, acc, off);
+    const int row = pb + (sl - s0) * rows_per_slice + (lane >> a.tpr_log2);
+    if (sub_lane == 0 && row < pe) {
+      if (SCATTER) y[checked(a.new_to_old[row], a.n, a.status)] = acc;
+      else y[checked(row, a.n, a.status)] = acc;
+      if (dot) dacc = fma((double)acc, a.dot_self ? (double)acc : (double)xsl[row - pb], dacc);
+    }
+  };
+  int i = s0 + warp;
   int s = s1;
   int64_t pos = 0, epos = 0;
   int w = 0, we = 0;
-  if (i < s1) slice_meta(i, s, pos, w, epos, we);
-  while (i < s1) {
-    // reserve the next slice and start its metadata loads before working on this one
+  if (i < items) item_meta(i, s, pos, w, epos, we);
+  while (i < items) {
+    // reserve the next item and start its metadata loads before working on this one
     int inxt;
     if (dot) {
       inxt = i + nwarps;
@@ -670,9 +750,24 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
     int nxt = s1;
     int64_t npos = 0, nepos = 0;
     int nw = 0, nwe = 0;
-    if (inxt < s1) slice_meta(inxt, nxt, npos, nw, nepos, nwe);
+    if (inxt < items) item_meta(inxt, nxt, npos, nw, nepos, nwe);
+    int part = -1;  // WIDE: the part of the workspace this item's sums go to (-1: a whole slice)
+    bool halo_wide = false;
+    if (WIDE) {
+      part = s < 0 ? -1 - s : a.slice_wide[s];
+      halo_wide = part >= 0 && a.row_cin;
+      if (!halo_wide) {  // a slice's first chunks (a unit holds at most one chunk)
+        w = min(w, kWideCap);
+        we = min(we, kWideCap);
+      }
+    }
     X acc;
-    if constexpr (RUNS) {  // the copy in runs of four slots (its own column arrays are in a.ell_col / a.er_scol*)
+    if (WIDE && halo_wide) {
+      const int row = pb + (s - s0) * 32 + lane;
+      const int cin = row < pe ? a.row_cin[row] : 0, cer = row < pe ? a.row_cer[row] : 0;
+      acc = halo_wide_dot<V, X, RUNS>(ell_val + pos, a.ell_col + pos, lane, w, cin, cer, xsl, pe - pb + nh, a.status);
+      part = -1;
+    } else if constexpr (RUNS) {  // the copy in runs of four slots (its own column arrays are in a.ell_col / a.er_scol*)
       acc = slab_dot_runs<V, X, KB>(ell_val + pos, a.ell_col + pos, lane, w, xsl, X(0), pe - pb + nh, a.status);
       if (ER_SLICED)
         acc = er_dot_runs<V, X>(er_val + epos, (GATHER ? a.er_scol_old : a.er_scol) + epos, lane, we, xp, acc, a.n_x,
@@ -683,19 +778,31 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
         acc = er_dot<V, X, KB>(er_val + epos + lane, (GATHER ? a.er_scol_old : a.er_scol) + epos + lane, we, xp, acc,
                                a.n_x, a.status);
     }
-    for (int off = tpr >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(FULL, acc, off);
-    const int row = pb + (s - s0) * rows_per_slice + (lane >> a.tpr_log2);
-    if (sub == 0 && row < pe) {
-      if (SCATTER) y[checked(a.new_to_old[row], a.n, a.status)] = acc;
-      else y[checked(row, a.n, a.status)] = acc;
-      if (dot) dacc = fma((double)acc, a.dot_self ? (double)acc : (double)xsl[row - pb], dacc);
-    }
+    if (WIDE && part >= 0)
+      *reinterpret_cast<X*>(a.wide_ws + 32 * (int64_t)checked(part, a.wide_parts, a.status) + lane) = acc;
+    else
+      store_rows(s, acc);
     i = inxt;
     s = nxt;
     pos = npos;
     w = nw;
     epos = nepos;
     we = nwe;
+  }
+  if (WIDE) {  // combine the wide slices' parts (all written by this block), in order
+    const int w0 = a.wide_ptr[p], w1 = a.wide_ptr[p + 1];
+    if (w0 < w1) {
+      __syncthreads();
+      for (int k = w0 + warp; k < w1; k += nwarps) {
+        const WideSlice ws = a.wides[k];
+        const double* q = a.wide_ws + 32 * (int64_t)checked(ws.part, a.wide_parts - ws.count, a.status) + lane;
+        const X acc0 = *reinterpret_cast<const X*>(q);
+        X t = X(0);
+#pragma unroll 4
+        for (int c = 1; c <= ws.count; ++c) t += *reinterpret_cast<const X*>(q + 32 * c);
+        store_rows(ws.s, acc0 + t);
+      }
+    }
   }
   if (dot) {  // only offered for the sliced ER layout, where a slice's rows are final here
     const double t = block_sum_fixed(dacc, bs.ws);
@@ -798,6 +905,15 @@ inline KArgs make_kargs(const DevPlan& P) {
   a.dot_arrive = nullptr;
   a.dot_result = nullptr;
   a.skip = nullptr;
+  a.slice_wide = P.slice_wide;
+  a.unit_ptr = P.unit_ptr;
+  a.units = P.units;
+  a.wide_ptr = P.wide_ptr;
+  a.wides = P.wides;
+  a.wide_ws = P.wide_ws;
+  a.wide_parts = P.wide_parts;
+  a.row_cin = P.row_cin;
+  a.row_cer = P.row_cer;
   a.meta_off = 0;
   a.meta_cap = 0;
   return a;

@@ -26,6 +26,20 @@ ehyb_status_t cuda_error_status(cudaError_t e, const char* what);
 ehyb_status_t device_alloc(void** p, size_t bytes);
 }  // namespace ehyb
 
+namespace ehyb {
+// Wide slices of a sliced layout (er_layout 0): slices with more than kWideCap slab or extra-row slots per lane,
+// their later chunks as units by partition (longest first), and the numbering of the parts' partial sums.
+struct WideLists {
+  int32_t parts = 0;
+  std::vector<int32_t> slice_wide, unit_ptr, wide_ptr;
+  std::vector<WideUnit> units;
+  std::vector<WideSlice> wides;
+  int32_t max_items = 0;  // most slices + units of one partition
+};
+WideLists wide_lists(int32_t nparts, const std::vector<int32_t>& slice_ptr, const std::vector<int64_t>& slice_pos,
+                     const std::vector<int64_t>& er_slice_pos);
+}  // namespace ehyb
+
 struct ehyb_plan_s {
   ehyb::HostPlan host;        // arrays kept only when requested (or host-only); metadata always
   bool host_kept = false;

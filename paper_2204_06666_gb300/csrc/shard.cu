@@ -282,6 +282,13 @@ ehyb_status_t ehyb_shard_create(ehyb_plan_t plan, int32_t nranks, int32_t rank, 
     D.max_part_rows = std::max(D.max_part_rows, S->part_ptr[(size_t)p + 1] - S->part_ptr[(size_t)p]);
     D.max_part_slices = std::max(D.max_part_slices, S->slice_ptr[(size_t)p + 1] - S->slice_ptr[(size_t)p]);
   }
+  WideLists W;
+  try {
+    W = wide_lists(D.nparts, S->slice_ptr, S->slice_pos, S->er_slice_pos);
+  } catch (const std::bad_alloc&) {
+    return EHYB_ERR_OOM;
+  }
+  D.wide_parts = W.parts;
   if (!S->host_only) {
     cudaStream_t s = (cudaStream_t)stream;
     CKS(cudaGetDevice(&S->device));
@@ -294,7 +301,9 @@ ehyb_status_t ehyb_shard_create(ehyb_plan_t plan, int32_t nranks, int32_t rank, 
                  o_ev = add(S->ell_val.size() * 8), o_esp = add(S->er_slice_pos.size() * 8),
                  o_esc = add(S->er_scol.size() * 4), o_esv = add(S->er_sval.size() * 8),
                  o_si = add(S->send_idx.size() * 4), o_dot = add(((size_t)D.nparts + 2) * 8), o_arr = add(16),
-                 o_st = add(16);
+                 o_st = add(16), o_sw = add(W.slice_wide.size() * 4), o_up = add(W.unit_ptr.size() * 4),
+                 o_un = add(W.units.size() * sizeof(WideUnit)), o_wp = add(W.wide_ptr.size() * 4),
+                 o_ws = add(W.wides.size() * sizeof(WideSlice)), o_ww = add((size_t)W.parts * 32 * 8);
     ehyb_status_t st = device_alloc(&S->arena, off);
     if (st != EHYB_OK) return st;
     char* base = (char*)S->arena;
@@ -313,6 +322,11 @@ ehyb_status_t ehyb_shard_create(ehyb_plan_t plan, int32_t nranks, int32_t rank, 
     up(o_esc, S->er_scol.data(), S->er_scol.size() * 4);
     up(o_esv, S->er_sval.data(), S->er_sval.size() * 8);
     up(o_si, S->send_idx.data(), S->send_idx.size() * 4);
+    up(o_sw, W.slice_wide.data(), W.slice_wide.size() * 4);
+    up(o_up, W.unit_ptr.data(), W.unit_ptr.size() * 4);
+    up(o_un, W.units.data(), W.units.size() * sizeof(WideUnit));
+    up(o_wp, W.wide_ptr.data(), W.wide_ptr.size() * 4);
+    up(o_ws, W.wides.data(), W.wides.size() * sizeof(WideSlice));
     if (e == cudaSuccess) e = cudaMemsetAsync(base + o_arr, 0, 16, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(base + o_st, 0, 16, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -333,6 +347,14 @@ ehyb_status_t ehyb_shard_create(ehyb_plan_t plan, int32_t nranks, int32_t rank, 
     D.er_scol_old = D.er_scol;
     D.er_sval = (const double*)(base + o_esv);
     D.status = (int32_t*)(base + o_st);
+    if (W.parts > 0) {
+      D.slice_wide = (const int32_t*)(base + o_sw);
+      D.unit_ptr = (const int32_t*)(base + o_up);
+      D.units = (const WideUnit*)(base + o_un);
+      D.wide_ptr = (const int32_t*)(base + o_wp);
+      D.wides = (const WideSlice*)(base + o_ws);
+      D.wide_ws = (double*)(base + o_ww);
+    }
     S->d_send_idx = (const int32_t*)(base + o_si);
     S->d_dot = (double*)(base + o_dot);
     S->d_arrive = (int32_t*)(base + o_arr);

@@ -85,22 +85,49 @@ __global__ void __launch_bounds__(512) spmm_kernel(KArgs a, const double* __rest
     const int w = (int)((a.slice_pos[s + 1] - pos) >> 5);
     const double* vp = ell_val + pos + lane;
     const uint16_t* cp = a.ell_col + pos + lane;
-    for (int kk = 0; kk < w; ++kk) {
-      const double v = __ldcs(vp + 32 * (int64_t)kk);
-      const int c = checked((int)__ldcs(reinterpret_cast<const unsigned short*>(cp + 32 * (int64_t)kk)), pe - pb, a.status);
-      const double* xr = xsl + c * KC;
-#pragma unroll
-      for (int j = 0; j < KC; ++j) acc[j] = fma(v, xr[j], acc[j]);
-    }
     const int64_t epos = a.er_slice_pos[s];
     const int we = (int)((a.er_slice_pos[s + 1] - epos) >> 5);
     const double* evp = er_val + epos + lane;
     const int32_t* ecp = a.er_scol + epos + lane;
-    for (int kk = 0; kk < we; ++kk) {
-      const double v = __ldcs(evp + 32 * (int64_t)kk);
-      const double* xr = xc + (int64_t)checked(__ldcs(ecp + 32 * (int64_t)kk), a.n, a.status) * KC;
+    // slab slots [k0, k1) into q[0..KC)
+    auto slab = [&](int k0, int k1, double (&q)[KC]) {
+      for (int kk = k0; kk < k1; ++kk) {
+        const double v = __ldcs(vp + 32 * (int64_t)kk);
+        const int c = checked((int)__ldcs(reinterpret_cast<const unsigned short*>(cp + 32 * (int64_t)kk)), pe - pb, a.status);
+        const double* xr = xsl + c * KC;
 #pragma unroll
-      for (int j = 0; j < KC; ++j) acc[j] = fma(v, __ldg(xr + j), acc[j]);
+        for (int j = 0; j < KC; ++j) q[j] = fma(v, xr[j], q[j]);
+      }
+    };
+    // extra-row slots [k0, k1)
+    auto extra = [&](int k0, int k1, double (&q)[KC]) {
+      for (int kk = k0; kk < k1; ++kk) {
+        const double v = __ldcs(evp + 32 * (int64_t)kk);
+        const double* xr = xc + (int64_t)checked(__ldcs(ecp + 32 * (int64_t)kk), a.n, a.status) * KC;
+#pragma unroll
+        for (int j = 0; j < KC; ++j) q[j] = fma(v, __ldg(xr + j), q[j]);
+      }
+    };
+    slab(0, min(w, kWideCap), acc);
+    extra(0, min(we, kWideCap), acc);
+    if (w > kWideCap || we > kWideCap) {  // a wide slice's later chunks, summed as the SpMV sums them
+      double t[KC];
+#pragma unroll
+      for (int j = 0; j < KC; ++j) t[j] = 0.0;
+#pragma unroll 1
+      for (int part = 0; part < 2; ++part)
+#pragma unroll 1
+        for (int k = kWideCap; k < (part ? we : w); k += kWideCap) {
+          double q[KC];
+#pragma unroll
+          for (int j = 0; j < KC; ++j) q[j] = 0.0;
+          if (part) extra(k, min(k + kWideCap, we), q);
+          else slab(k, min(k + kWideCap, w), q);
+#pragma unroll
+          for (int j = 0; j < KC; ++j) t[j] += q[j];
+        }
+#pragma unroll
+      for (int j = 0; j < KC; ++j) acc[j] += t[j];
     }
 #pragma unroll
     for (int j = 0; j < KC; ++j)

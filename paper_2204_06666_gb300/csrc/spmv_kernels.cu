@@ -24,7 +24,7 @@ constexpr int run_batch() {
   return (sizeof(V) == 2 && !DOT) ? 32 : 16;
 }
 template <typename V, typename X, bool SCATTER, bool ER_SLICED, bool DOT, bool GATHER = false,
-          int KB = (sizeof(V) == 8 ? kBatch : kLowBatch), bool RUNS = false>
+          int KB = (sizeof(V) == 8 ? kBatch : kLowBatch), bool RUNS = false, bool WIDE = false>
 __global__ void __launch_bounds__(1024, 1) ehyb_kernel(KArgs a, const V* __restrict__ ell_val,
                                                     const V* __restrict__ er_val, const X* __restrict__ xp,
                                                     X* __restrict__ y) {
@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(1024, 1) ehyb_kernel(KArgs a, const V* __restr
     bs.bar_ready = 0;
     bs.phase = 0;
   }
-  partition_spmv<V, X, SCATTER, ER_SLICED, DOT, GATHER, KB, RUNS, true, true>(
+  partition_spmv<V, X, SCATTER, ER_SLICED, DOT, GATHER, KB, RUNS, true, true, WIDE>(
       a, ell_val, er_val, xp, y, blockIdx.x, reinterpret_cast<X*>(smem_raw), bs);
 }
 
@@ -91,32 +91,38 @@ size_t ehyb_smem_bytes(const DevPlan& P, int elem_bytes) {
 // batch depth of the FP64 kernels for wide slices (see DevPlan::kbatch)
 constexpr int kWideBatch = 6;
 
+// the kernel of one launch form: the plan's batch depth, slot layout of the copies and wide slices choose among
+// its instantiations (`f` is called with the kernel)
+template <typename V, typename X, bool SCATTER, bool ER_SLICED, bool DOT, bool GATHER, typename F>
+static cudaError_t pick_kernel(bool deep, bool runs, bool wide, F&& f) {
+  constexpr int KB = sizeof(V) == 8 ? kBatch : kLowBatch, R = run_batch<V, DOT>();
+  if constexpr (ER_SLICED && sizeof(V) == 8) {
+    if (wide) return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, KB, false, true>);
+    if (!deep) return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, kWideBatch>);
+  } else if constexpr (ER_SLICED) {
+    if (wide && runs) return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, 16, true, true>);
+    if (wide) return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, KB, false, true>);
+    if (runs) return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, R, true>);
+  }
+  return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, KB>);
+}
+
+// every instantiation of the launch forms may use the opt-in shared memory
 template <typename V, typename X>
 static cudaError_t set_smem(int bytes) {
-  cudaError_t e;
-  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  if constexpr (std::is_same<V, double>::value) {
-    if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, true, true, false, true, kWideBatch>, attr, bytes))) return e;
-    if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, true, true, true, true, kWideBatch>, attr, bytes))) return e;
-    if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, false, true, true, false, kWideBatch>, attr, bytes))) return e;
-    if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, false, true, false, false, kWideBatch>, attr, bytes))) return e;
-    if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, true, true, false, false, kWideBatch>, attr, bytes))) return e;
+  auto set = [&](auto k) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
+  for (int v = 0; v < 8; ++v) {
+    const bool deep = v & 1, runs = v & 2, wide = v & 4;
+    cudaError_t e;
+    if ((e = pick_kernel<V, X, true, true, false, false>(deep, runs, wide, set))) return e;
+    if ((e = pick_kernel<V, X, true, false, false, false>(deep, runs, wide, set))) return e;
+    if ((e = pick_kernel<V, X, false, true, false, false>(deep, runs, wide, set))) return e;
+    if ((e = pick_kernel<V, X, false, false, false, false>(deep, runs, wide, set))) return e;
+    if ((e = pick_kernel<V, X, true, true, false, true>(deep, runs, wide, set))) return e;
+    if ((e = pick_kernel<V, X, true, true, true, true>(deep, runs, wide, set))) return e;
+    if ((e = pick_kernel<V, X, false, true, true, false>(deep, runs, wide, set))) return e;
   }
-  if constexpr (!std::is_same<V, double>::value) {  // the copies laid out in runs of four (sliced ER layout)
-    constexpr int R = run_batch<V, false>(), RD = run_batch<V, true>();
-    if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, true, true, false, false, R, true>, attr, bytes))) return e;
-    if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, false, true, false, false, R, true>, attr, bytes))) return e;
-    if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, true, true, false, true, R, true>, attr, bytes))) return e;
-    if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, true, true, true, true, RD, true>, attr, bytes))) return e;
-    if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, false, true, true, false, RD, true>, attr, bytes))) return e;
-  }
-  if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, true, true, false>, attr, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, true, false, false>, attr, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, false, true, false>, attr, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, false, false, false>, attr, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, true, true, false, true>, attr, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(ehyb_kernel<V, X, true, true, true, true>, attr, bytes))) return e;
-  return cudaFuncSetAttribute(ehyb_kernel<V, X, false, true, true>, attr, bytes);
+  return cudaSuccess;
 }
 
 // dynamic shared memory a fused-kernel launch may use (the attribute kernels_init sets)
@@ -146,12 +152,9 @@ cudaError_t launch_permute_f32(const DevPlan& P, int to_new, const float* in, fl
 template <typename V, typename X, bool SCATTER, bool ER_SLICED, bool DOT, bool GATHER = false>
 static void launch_pdl(const DevPlan& P, size_t smem, cudaStream_t s, const KArgs& a, const V* ev, const V* erv,
                        const X* xp, X* y) {
-  // FP64 kernels on plans with wide slices use the shallower batch (sliced-ER layout only); FP32 / BF16
-  // copies laid out in runs of four use the run loops
-  constexpr bool kWideOk = std::is_same<V, double>::value && ER_SLICED;
-  constexpr bool kRunsOk = !std::is_same<V, double>::value && ER_SLICED;
-  const bool wide = kWideOk && P.kbatch == kWideBatch;
-  const bool runs = kRunsOk && P.lowp_group == 4;
+  // FP64 kernels on plans with many slots a lane use the shallower batch (sliced-ER layout only); FP32 / BF16
+  // copies laid out in runs of four use the run loops; plans with wide slices the kernels that sum them in chunks
+  const bool runs = !std::is_same<V, double>::value && ER_SLICED && P.lowp_group == 4;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)P.nparts);
   cfg.blockDim = dim3((unsigned)P.threads);
@@ -162,24 +165,14 @@ static void launch_pdl(const DevPlan& P, size_t smem, cudaStream_t s, const KArg
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if constexpr (kWideOk) {
-    if (wide) {
-      cudaLaunchKernelEx(&cfg, ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, kWideBatch>, a, ev, erv, xp, y);
-      return;
-    }
+  KArgs ar = a;
+  if (runs) {  // the copies' own column arrays, in the same runs
+    ar.ell_col = P.ell_col_low;
+    ar.er_scol = P.er_scol_low;
+    ar.er_scol_old = P.er_scol_old_low;
   }
-  if constexpr (kRunsOk) {
-    if (runs) {
-      KArgs ar = a;  // the copies' own column arrays, in the same runs
-      ar.ell_col = P.ell_col_low;
-      ar.er_scol = P.er_scol_low;
-      ar.er_scol_old = P.er_scol_old_low;
-      cudaLaunchKernelEx(&cfg, ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, run_batch<V, DOT>(), true>, ar, ev, erv,
-                         xp, y);
-      return;
-    }
-  }
-  cudaLaunchKernelEx(&cfg, ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER>, a, ev, erv, xp, y);
+  pick_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER>(P.kbatch != kWideBatch, runs, ER_SLICED && P.wide_parts > 0,
+                                                     [&](auto k) { return cudaLaunchKernelEx(&cfg, k, ar, ev, erv, xp, y); });
 }
 
 template <typename V, typename X>
