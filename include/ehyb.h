@@ -450,21 +450,21 @@ typedef struct ehyb_batch_s* ehyb_batch_t;
 /*
  * Group `count` plans (FP64, sliced ER layout, all on the current device) for ehyb_batch_spmv.  The
  * batch keeps pointers to the plans: destroy the batch before any of its plans.  Its work list is the
- * (plan, partition) pairs ordered by stored slots, largest first.
+ * (plan, partition) pairs, large partitions cut into shares of their slices, ordered by stored slots, largest
+ * first.
  */
 ehyb_status_t ehyb_batch_create(int32_t count, const ehyb_plan_t* plans, ehyb_batch_t* out);
 
 /*
  * ys[i] = A_i xs[i] for every plan of the batch (device arrays, original numbering), asynchronously on
  * `stream`: ONE persistent launch whose blocks pull (plan, partition) tiles from a shared queue, each
- * tile gathering its slice of x through its plan's permutation as it stages it, replayed from a CUDA
- * graph captured on the first call.  Results equal
+ * tile gathering its slice of x through its plan's permutation as it stages it.  Results equal
  * ehyb_spmv on each plan bit for bit.  Uses the plans' workspaces: do not overlap with other calls on
  * the same plans.  xs / ys are host arrays of `count` device pointers.
  */
 ehyb_status_t ehyb_batch_spmv(ehyb_batch_t batch, const double* const* xs, double* const* ys, void* stream);
 
-/* Work list length, persistent grid size and threads per block of the batch launch. */
+/* (plan, partition) pairs, persistent grid size and threads per block of the batch launch. */
 ehyb_status_t ehyb_batch_info(ehyb_batch_t batch, int32_t* ntiles, int32_t* grid, int32_t* threads);
 
 ehyb_status_t ehyb_batch_destroy(ehyb_batch_t batch);  /* NULL is accepted */
