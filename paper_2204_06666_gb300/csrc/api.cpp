@@ -437,6 +437,10 @@ ehyb_status_t plan_finalize(std::unique_ptr<ehyb_plan_s>& P, const ehyb_options_
   D.max_part_slices = 0;
   for (int32_t p = 0; p < H.nparts; ++p)
     D.max_part_slices = std::max(D.max_part_slices, H.slice_ptr[(size_t)p + 1] - H.slice_ptr[(size_t)p]);
+  // one slice per warp and one block per SM at most: the product is latency, not throughput (ehyb_core.cuh)
+  if (H.er_layout == 0 && W.parts == 0 && D.max_part_slices <= 32 && H.nparts <= d.sms &&
+      (opt_in.block_threads == 0 || 32 * D.max_part_slices <= opt.block_threads))
+    D.small_threads = 32 * std::max(D.max_part_slices, 1);
   {  // batch depth: mean slab + sliced-ER slots per lane of a slice (measured: 6 is faster from about 32 up)
     const double w = mean_slice_width(H);
     D.kbatch = (H.er_layout == 0 && w >= 32.0) ? 6 : 8;

@@ -28,6 +28,7 @@ struct DevPlan {
   int32_t max_part_rows = 0;
   int32_t max_stage_rows = 0;  // largest rows + halo of a partition: the staged x elements (er_layout 2)
   int32_t max_part_slices = 0;  // most slices of one partition (entries of the fused kernel's slice table)
+  int32_t small_threads = 0;    // one slice per warp: threads of the small-plan kernel (0: not for this plan)
   int32_t kbatch = 8;  // FP64 batch depth (two pipelined half-batches): 6 on wide slices (>= 32 slots a lane), else 8;
                        // the FP32 / BF16 kernels hold 12 (column-major copies) or 16 / 32 (copies in runs of four)
   const int32_t* new_to_old = nullptr;

@@ -148,6 +148,26 @@ __device__ __forceinline__ float load_val<uint16_t, float>(const uint16_t* p) {
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
 
+// x from global memory, always with a plain load.  The non-coherent path (__ldg) is for memory that nobody writes
+// while the kernel is resident, and a kernel launched with programmatic stream serialization is resident while
+// the one before it still writes x; the compiler may also move such loads across the wait (it did where the
+// gathers stood right behind it).  The same speed on every workload measured.
+__device__ __forceinline__ double load_x(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float load_x(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double2 load_x2(const double* p) {  // p on 16 bytes
+  double2 v;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
+
 constexpr int kBatch = 8;   // slots whose loads are issued before their FMAs (default batch depth)
 constexpr int kStage = 16;  // elements of x per thread in flight while a slice of x is gathered
 
@@ -211,13 +231,13 @@ __device__ __forceinline__ X er_dot(const V* __restrict__ vp, const int32_t* __r
     }
     X xv[KB];
 #pragma unroll
-    for (int u = 0; u < KB; ++u) xv[u] = __ldg(xg + c[u]);
+    for (int u = 0; u < KB; ++u) xv[u] = load_x(xg + c[u]);
 #pragma unroll
     for (int u = 0; u < KB; ++u) acc = fma_t(v[u], xv[u], acc);
   }
   for (; k < w; ++k)
-    acc = fma_t(load_val<V, X>(vp + 32 * (int64_t)k), __ldg(xg + checked(__ldcs(cp + 32 * (int64_t)k), lim, status)),
-                acc);
+    acc = fma_t(load_val<V, X>(vp + 32 * (int64_t)k),
+                load_x(xg + checked(__ldcs(cp + 32 * (int64_t)k), lim, status)), acc);
   return acc;
 }
 
@@ -355,10 +375,9 @@ __device__ __forceinline__ X slab_dot_runs(const V* __restrict__ vb, const uint1
 
 // er_dot on runs of four: batches of kErGroups runs (values and columns loaded, then their x gathers, then
 // the FMAs in slot order), then the remaining run and the column-major tail
-template <typename V, typename X>
+template <typename V, typename X, int NB = kErGroups>
 __device__ __forceinline__ X er_dot_runs(const V* __restrict__ vb, const int32_t* __restrict__ cb, int lane, int w,
                                          const X* __restrict__ xg, X acc, int64_t lim, int32_t* status) {
-  constexpr int NB = kErGroups;
   const int ng = w >> 2;
   const V* vp = vb + kGroup * lane;
   const int32_t* cp = cb + kGroup * lane;
@@ -375,7 +394,7 @@ __device__ __forceinline__ X er_dot_runs(const V* __restrict__ vb, const int32_t
 #pragma unroll
     for (int u = 0; u < NB; ++u)
 #pragma unroll
-      for (int t = 0; t < kGroup; ++t) xv[u][t] = __ldg(xg + checked(c[u][t], lim, status));
+      for (int t = 0; t < kGroup; ++t) xv[u][t] = load_x(xg + checked(c[u][t], lim, status));
 #pragma unroll
     for (int u = 0; u < NB; ++u)
 #pragma unroll
@@ -388,7 +407,7 @@ __device__ __forceinline__ X er_dot_runs(const V* __restrict__ vb, const int32_t
     ld_cols(cp + 128 * (int64_t)g, c);
     X xv[kGroup];
 #pragma unroll
-    for (int t = 0; t < kGroup; ++t) xv[t] = __ldg(xg + checked(c[t], lim, status));
+    for (int t = 0; t < kGroup; ++t) xv[t] = load_x(xg + checked(c[t], lim, status));
 #pragma unroll
     for (int t = 0; t < kGroup; ++t) acc = fma_t(v[t], xv[t], acc);
   }
@@ -411,7 +430,7 @@ __device__ __forceinline__ X er_dot_runs(const V* __restrict__ vb, const int32_t
 #pragma unroll
   for (int t = 0; t < kGroup - 1; ++t) {
     tx[t] = X(0);
-    if (t < nt) tx[t] = __ldg(xg + tc[t]);
+    if (t < nt) tx[t] = load_x(xg + tc[t]);
   }
 #pragma unroll
   for (int t = 0; t < kGroup - 1; ++t)
@@ -632,7 +651,7 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
         c[u] = (i0 + u * bd < pe) ? checked(__ldg(a.new_to_old + i0 + u * bd), a.n, a.status) : -1;
       X v[kStage];
 #pragma unroll
-      for (int u = 0; u < kStage; ++u) v[u] = c[u] >= 0 ? __ldg(xp + c[u]) : X(0);
+      for (int u = 0; u < kStage; ++u) v[u] = c[u] >= 0 ? load_x(xp + c[u]) : X(0);
 #pragma unroll
       for (int u = 0; u < kStage; ++u)
         if (i0 + u * bd < pe) xs[checked(i0 + u * bd - a0, a.smem_elems, a.status)] = v[u];
@@ -640,7 +659,7 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
   } else {
     // plain loads: everything when the source is unaligned, else the ragged tail [a1, pe)
     const int lo = bulk_bytes ? (a1 > pb ? a1 : pb) : pb;
-    for (int i = lo + tid; i < pe; i += blockDim.x) xs[checked(i - a0, a.smem_elems, a.status)] = xp[i];
+    for (int i = lo + tid; i < pe; i += blockDim.x) xs[checked(i - a0, a.smem_elems, a.status)] = load_x(xp + i);
   }
   // er_layout 2: the halo's x values right after the slice (xs[pe - a0 + j], j < nh), gathered like the
   // slice itself (plain loads; disjoint from the bulk copy's destination, which ends at a1 - a0).  A loop of
@@ -656,7 +675,7 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
       for (int u = 0; u < kStage; ++u) c[u] = (j0 + u * bd < nh) ? checked(__ldg(hc + j0 + u * bd), a.n, a.status) : -1;
       X v[kStage];
 #pragma unroll
-      for (int u = 0; u < kStage; ++u) v[u] = c[u] >= 0 ? __ldg(xp + c[u]) : X(0);
+      for (int u = 0; u < kStage; ++u) v[u] = c[u] >= 0 ? load_x(xp + c[u]) : X(0);
 #pragma unroll
       for (int u = 0; u < kStage; ++u)
         if (j0 + u * bd < nh) xs[checked(pe - a0 + j0 + u * bd, a.smem_elems, a.status)] = v[u];
@@ -848,12 +867,12 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
           c[u] = checked(__ldcs(a.er_col + k + u * etpr), a.n, a.status);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) xv[u] = __ldg(xp + c[u]);
+        for (int u = 0; u < 4; ++u) xv[u] = load_x(xp + c[u]);
 #pragma unroll
         for (int u = 0; u < 4; ++u) acc = fma_t(v[u], xv[u], acc);
       }
       for (; k < k1; k += etpr)
-        acc = fma_t(load_val<V, X>(er_val + k), __ldg(xp + checked(__ldcs(a.er_col + k), a.n, a.status)), acc);
+        acc = fma_t(load_val<V, X>(er_val + k), load_x(xp + checked(__ldcs(a.er_col + k), a.n, a.status)), acc);
     }
     for (int off = etpr >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(FULL, acc, off);
     if (esub == 0 && e < e1) {
@@ -863,6 +882,149 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
     }
   }
   return true;
+}
+
+// ---- one slice per warp.  With at most 32 slices per partition (155k rows over 152 blocks) a product is a chain of
+// latencies, not a stream: partition_spmv reads the slice's metadata, then stages x (an index load, a gather, a
+// barrier), then loads the first slots, multiplies, loads the extra-row columns, gathers, loads the index that y
+// is stored at.  Here warp w owns slice w, and everything that depends on the plan alone -- the slice's first
+// slots, its first extra-row slots, the staging index, which is also the store index -- is loaded at once, before
+// the wait on the previous grid; after the wait only the gathers of x, one barrier, the FMAs and the store remain.
+// The slots run in the same order as in partition_spmv: same bits.  Back to back, before -> now: 2D 40k rows 4.62 ->
+// 3.89 us, 2D 90k 5.61 -> 4.56, tet 64k 6.26 -> 5.90, elasticity 12k 10.24 -> 7.72 (BF16 24k 5.86 -> 4.81).  Plans with
+// more than 32 slices in a partition, or more partitions than SMs, have enough work to hide the loads behind.
+
+// the first R slab slots of a lane (R a multiple of 4), held until x is staged
+template <typename V, typename X, int R, bool RUNS>
+struct SlabHead {
+  X v[R];
+  int c[R];
+  __device__ __forceinline__ void load(const V* __restrict__ vp, const uint16_t* __restrict__ cp, int w, int lane,
+                                       int lim, int32_t* status) {
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      v[u] = X(0);
+      c[u] = 0;
+      if (u < w) {
+        v[u] = load_val<V, X>(vp + 32 * u + lane);
+        c[u] = checked((int)__ldcs(reinterpret_cast<const unsigned short*>(cp + 32 * u + lane)), lim, status);
+      }
+    }
+  }
+  __device__ __forceinline__ X dot(const V* __restrict__ vp, const uint16_t* __restrict__ cp, int w, int lane,
+                                   const X* xs, int lim, int32_t* status) const {
+    X acc = X(0);
+#pragma unroll
+    for (int u = 0; u < R; ++u)
+      if (u < w) acc = fma_t(v[u], xs[c[u]], acc);
+    if (w > R) acc = slab_dot<V, X, R>(vp + 32 * R + lane, cp + 32 * R + lane, w - R, xs, acc, lim, status);
+    return acc;
+  }
+};
+template <typename V, typename X, int R>
+struct SlabHead<V, X, R, true> {
+  Run<V> run[R / 4];
+  X tv[kGroup - 1];
+  int tc[kGroup - 1];
+  __device__ __forceinline__ void load(const V* __restrict__ vp, const uint16_t* __restrict__ cp, int w, int lane,
+                                       int lim, int32_t* status) {
+    const int ng = w >> 2, nt = w & (kGroup - 1);
+#pragma unroll
+    for (int u = 0; u < R / 4; ++u) {
+      zero_run(run[u]);
+      if (u < ng) ld_run(vp + 128 * u + kGroup * lane, cp + 128 * u + kGroup * lane, run[u]);
+    }
+#pragma unroll
+    for (int t = 0; t < kGroup - 1; ++t) {
+      tv[t] = X(0);
+      tc[t] = 0;
+      if (w < R && t < nt) {
+        const int o = 128 * ng + 32 * t + lane;
+        tv[t] = load_val<V, X>(vp + o);
+        tc[t] = checked((int)__ldcs(reinterpret_cast<const unsigned short*>(cp + o)), lim, status);
+      }
+    }
+  }
+  __device__ __forceinline__ X dot(const V* __restrict__ vp, const uint16_t* __restrict__ cp, int w, int lane,
+                                   const X* xs, int lim, int32_t* status) const {
+    const int ng = w >> 2, nt = w & (kGroup - 1);
+    X acc = X(0);
+#pragma unroll
+    for (int u = 0; u < R / 4; ++u)
+      if (u < ng) acc = fma_run(run[u], xs, acc, lim, status);
+    if (w < R) {
+#pragma unroll
+      for (int t = 0; t < kGroup - 1; ++t)
+        if (t < nt) acc = fma_t(tv[t], xs[tc[t]], acc);
+    } else if (w > R) {
+      acc = slab_dot_runs<V, X, (R < 16 ? 16 : R)>(vp + 32 * R, cp + 32 * R, lane, w - R, xs, acc, lim, status);
+    }
+    return acc;
+  }
+};
+
+// Partition p with one slice per warp (er_layout 0, no wide slices, blockDim.x >= the partition's rows); x and y as in
+// partition_spmv, gathered and scattered through new_to_old with GATHER, in the plan's numbering without.
+// R slab and 4 extra-row slots are held from before the wait; R is also the depth of the loops over the rest.
+template <typename V, typename X, bool GATHER, bool RUNS, int R>
+__device__ __forceinline__ void small_partition_spmv(const KArgs& a, const V* __restrict__ ell_val,
+                                                     const V* __restrict__ er_val, const X* __restrict__ xp,
+                                                     X* __restrict__ y, const int p, X* xs) {
+  constexpr int E = 4;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int pb = a.part_ptr[p], rows = a.part_ptr[p + 1] - pb;
+  const int s = a.slice_ptr[p] + warp;
+  const bool on = s < a.slice_ptr[p + 1];
+  int64_t pos = 0, epos = 0;
+  int w = 0, we = 0;
+  if (on) {
+    pos = a.slice_pos[s];
+    w = (int)((a.slice_pos[s + 1] - pos) >> 5);
+    epos = a.er_slice_pos[s];
+    we = (int)((a.er_slice_pos[s + 1] - epos) >> 5);
+  }
+  const int tpr = 1 << a.tpr_log2;
+  const int orow = warp * (32 >> a.tpr_log2) + (lane >> a.tpr_log2);  // the row this lane stores
+  const bool stores = on && (lane & (tpr - 1)) == 0 && orow < rows;
+  int src = -1, dst = -1;
+  if (tid < rows) src = GATHER ? checked(a.new_to_old[pb + tid], a.n, a.status) : pb + tid;
+  if (stores) dst = GATHER ? checked(a.new_to_old[pb + orow], a.n, a.status) : pb + orow;
+  const V* vp = ell_val + pos;
+  const uint16_t* cp = a.ell_col + pos;
+  const V* evp = er_val + epos;
+  const int32_t* ecp = (GATHER ? a.er_scol_old : a.er_scol) + epos;
+  SlabHead<V, X, R, RUNS> head;
+  head.load(vp, cp, w, lane, rows, a.status);
+  X ev[E];
+  int ec[E];
+  const int ewg = RUNS ? (we & ~3) : 0;
+#pragma unroll
+  for (int u = 0; u < E; ++u) {
+    ev[u] = X(0);
+    ec[u] = 0;
+    if (u < we) {
+      const int o = u < ewg ? 4 * lane + u : 32 * u + lane;
+      ev[u] = load_val<V, X>(evp + o);
+      ec[u] = checked(__ldcs(ecp + o), a.n_x, a.status);
+    }
+  }
+  pdl_wait();
+  X xe[E];
+#pragma unroll
+  for (int u = 0; u < E; ++u) xe[u] = u < we ? load_x(xp + ec[u]) : X(0);
+  if (src >= 0) xs[checked(tid, a.smem_elems, a.status)] = load_x(xp + src);
+  __syncthreads();
+  if (!on) return;
+  X acc = head.dot(vp, cp, w, lane, xs, rows, a.status);
+#pragma unroll
+  for (int u = 0; u < E; ++u)
+    if (u < we) acc = fma_t(ev[u], xe[u], acc);
+  if (we > E) {
+    if constexpr (RUNS) acc = er_dot_runs<V, X, R / 4>(evp + 32 * E, ecp + 32 * E, lane, we - E, xp, acc, a.n_x, a.status);
+    else acc = er_dot<V, X, R>(evp + 32 * E + lane, ecp + 32 * E + lane, we - E, xp, acc, a.n_x, a.status);
+  }
+  for (int off = tpr >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(FULL, acc, off);
+  if (stores) y[dst] = acc;
 }
 
 // host helpers

@@ -45,6 +45,18 @@ __global__ void __launch_bounds__(1024, 1) ehyb_kernel(KArgs a, const V* __restr
       a, ell_val, er_val, xp, y, blockIdx.x, reinterpret_cast<X*>(smem_raw), bs);
 }
 
+// Plans with one slice per warp (small_partition_spmv): 1024 threads leave 64 registers each for 8 slots in flight,
+// 512 and 256 threads room for 16 and 32.
+template <typename V, typename X, bool GATHER, bool RUNS, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) ehyb_small_kernel(KArgs a, const V* __restrict__ ell_val,
+                                                          const V* __restrict__ er_val, const X* __restrict__ xp,
+                                                          X* __restrict__ y) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_launch_dependents();
+  small_partition_spmv<V, X, GATHER, RUNS, 8192 / MAXT>(a, ell_val, er_val, xp, y, blockIdx.x,
+                                                                reinterpret_cast<X*>(smem_raw));
+}
+
 template <typename X>
 __global__ void permute_kernel(int64_t n, const int32_t* __restrict__ n2o, int to_new, const X* __restrict__ in,
                                X* __restrict__ out) {
@@ -175,11 +187,50 @@ static void launch_pdl(const DevPlan& P, size_t smem, cudaStream_t s, const KArg
                                                      [&](auto k) { return cudaLaunchKernelEx(&cfg, k, ar, ev, erv, xp, y); });
 }
 
+// the small-plan kernel of a plan with small_threads > 0 (its shared memory is at most 8 KB: no opt-in)
+template <typename V, typename X, bool GATHER>
+static void launch_small(const DevPlan& P, size_t smem, cudaStream_t s, const KArgs& a, const V* ev, const V* erv,
+                         const X* xp, X* y) {
+  const bool runs = !std::is_same<V, double>::value && P.lowp_group == 4;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)P.nparts);
+  cfg.blockDim = dim3((unsigned)P.small_threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  KArgs ar = a;
+  if (runs) {  // the copies' own column arrays, in the same runs
+    ar.ell_col = P.ell_col_low;
+    ar.er_scol = P.er_scol_low;
+    ar.er_scol_old = P.er_scol_old_low;
+  }
+  auto go = [&](auto k) { cudaLaunchKernelEx(&cfg, k, ar, ev, erv, xp, y); };
+  auto sized = [&](auto r) {
+    constexpr bool R = decltype(r)::value;
+    if (P.small_threads <= 256) go(ehyb_small_kernel<V, X, GATHER, R, 256>);
+    else if (P.small_threads <= 512) go(ehyb_small_kernel<V, X, GATHER, R, 512>);
+    else go(ehyb_small_kernel<V, X, GATHER, R, 1024>);
+  };
+  if constexpr (!std::is_same<V, double>::value) {
+    if (runs) return sized(std::true_type());
+  }
+  sized(std::false_type());
+}
+
 template <typename V, typename X>
 static void launch_typed(const DevPlan& P, const V* ev, const V* erv_csr, const V* erv_sl, const X* xp, X* y,
                          int scatter, size_t smem, cudaStream_t s, const DotOut* dot, const int32_t* skip) {
   KArgs a = make_kargs(P);
   a.smem_elems = (int64_t)(smem / sizeof(X));
+  if (P.small_threads > 0 && !dot && !skip && scatter != 1 && !P.inject_wait_fault) {
+    if (scatter == 2) launch_small<V, X, true>(P, smem, s, a, ev, erv_sl, xp, y);
+    else launch_small<V, X, false>(P, smem, s, a, ev, erv_sl, xp, y);
+    return;
+  }
   // the partition's slice table after the staged x, when both fit the block's shared memory
   const size_t tbytes = (size_t)P.max_part_slices * sizeof(SliceMeta);
   if (P.max_part_slices > 0 && smem + tbytes <= g_smem_max) {
