@@ -263,8 +263,8 @@ ehyb_status_t ehyb_spmv_lowp(ehyb_plan_t plan, const float* x, float* y, void* s
 /*
  * Y = A X for k right-hand sides in FP64: X and Y are row-major n x k device arrays (original
  * numbering).  The columns run in chunks of KC in {8, 4, 2, 1} (the largest that divides k and whose
- * KC-wide slice of X fits a block's shared memory), one launch per chunk, after one gather of X into a
- * chunk-major workspace (n x k doubles, allocated by the first call).  Column j of Y equals ehyb_spmv of
+ * KC-wide slice of X fits a block's shared memory), one launch per chunk, which gathers its columns of X
+ * through the permutation as it stages them.  Column j of Y equals ehyb_spmv of
  * column j of X bit for bit.  Requires the sliced ER layout.  Asynchronous on `stream`.  A plan built with
  * opt.spmm_rhs = k has partitions small enough for whole 8-column chunks (one pass over A per 8 columns).
  */

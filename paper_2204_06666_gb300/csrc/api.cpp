@@ -600,7 +600,7 @@ extern "C" {
 ehyb_status_t ehyb_destroy(ehyb_plan_t p) {
   if (!p) return EHYB_OK;
   ehyb_status_t st = EHYB_OK;
-  if (p->arena || p->hx || p->cg || p->spmm_ws || !p->ev_pool.empty() || p->px[0] || p->s_in) {
+  if (p->arena || p->hx || p->cg || !p->ev_pool.empty() || p->px[0] || p->s_in) {
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) st = cuda_fail(e, "cudaDeviceSynchronize");
     if (p->arena) cudaFree(p->arena);
@@ -616,7 +616,6 @@ ehyb_status_t ehyb_destroy(ehyb_plan_t p) {
     if (p->s_in) cudaStreamDestroy(p->s_in);
     if (p->s_out) cudaStreamDestroy(p->s_out);
     if (p->cg) cg_work_free(p->cg);
-    if (p->spmm_ws) cudaFree(p->spmm_ws);
     for (auto& ev : p->ev_pool) {
       cudaEventDestroy(ev.first);
       cudaEventDestroy(ev.second);
