@@ -12,7 +12,9 @@
 // alpha and beta never leave the device.  Every reduction runs in a fixed order, so a solve is bit-
 // reproducible.  Once `done` is up the remaining kernels of a chunk return at once, so the iteration
 // count is exact although the host looks at the flag only once per chunk.  A chunk of kChunk
-// iterations is captured once into a CUDA graph and replayed.
+// iterations is captured once into a CUDA graph and replayed.  A plan whose partitions are all resident at
+// once (Eq. 1's are, up to 4.4 M rows) runs its iterations inside one cooperative kernel instead
+// (cg_persist_kernel).
 //
 // Refinement (refine = 1: FP32 values, 2: BF16 values): outer FP64 residual r = b - A x on the FP64
 // plan, inner CG on the low-precision copy of the values with FP32 vectors, FP32 SpMV accumulation and
@@ -24,13 +26,14 @@
 #include <cstring>
 #include <vector>
 
+#include "persist.cuh"
 #include "plan_internal.h"
 
 namespace ehyb {
 
 namespace {
 
-constexpr unsigned FULL = 0xffffffffu;
+using core::FULL;
 constexpr int kVB = 608;  // vector-kernel blocks (4 per SM; 8 per SM measured slower)
 constexpr int kVT = 256;
 constexpr int kChunk = 16;
@@ -52,6 +55,7 @@ struct CgWork {
   float *r32 = nullptr, *p32 = nullptr, *q32 = nullptr, *d32 = nullptr;
   double *part_a = nullptr, *part_b = nullptr, *pq_part = nullptr, *hist = nullptr;
   CgState* st = nullptr;
+  persist::Meeting* meeting = nullptr;  // of the persistent kernel's blocks
   cudaStream_t cap = nullptr;
   cudaGraphExec_t g64 = nullptr, g32 = nullptr;
   int g32_lowp = 0;
@@ -349,6 +353,283 @@ __global__ void fcg_update_kernel(int64_t n, double alpha, const double* __restr
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
+// ---- persistent iterations: up to max_steps CG iterations (K1, K2, K3 of the launches above, the same arithmetic
+// per element) in one cooperative launch, block p owning partition p's rows.  p stays in shared memory (it is the
+// product's slice of x) and is mirrored to memory for the other blocks' extra rows; q, r and x stay there too as
+// far as they fit (in that order: q is written and read twice an iteration, r read and written, x likewise but by
+// one pass).  The blocks meet three times an iteration: for p.q, for r.r (x is updated while the sum travels)
+// and for the new p, which a warp waits for only when it comes to its first extra row.
+template <typename X>
+struct CgPersist {
+  X *x, *r, *p, *q;                 // global vectors, plan numbering
+  int32_t q_off, r_off, x_off;      // byte offsets in dynamic shared memory; -1: the vector stays in global memory
+  int32_t red_off, tbl_off;         // the block sum's terms; the slice table (-1: none)
+  int32_t max_steps;
+  CgState* st;
+  double* hist;
+  persist::SyncArgs sync;
+};
+
+// A block's state, in shared memory: thread 0's scalars (it alone divides and decides) and where the vectors are.
+template <typename V, typename X>
+struct CgBlock {
+  double alpha, beta, rr, tol2, grow_limit;
+  int it, max_iter, converged, breakdown, done, stop, seen, nh;
+  const int32_t* halo;
+  X *q, *r, *x, *p;  // p: the block's rows of p in memory
+  persist::Product<V, X> prod;
+  double* hist;
+  int32_t red_off;
+  persist::SyncArgs sync;
+};
+
+// p.q and alpha
+template <typename V, typename X>
+__device__ __noinline__ void cg_step_pq(CgBlock<V, X>& sh, int round) {
+  constexpr int U = 4;  // elements a thread has in flight
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  X* const ps = reinterpret_cast<X*>(smem_raw);
+  const int bd = blockDim.x;
+      double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
+      {
+        const X* const q = sh.q;
+        const int rows = sh.prod.rows;
+        double acc = 0.0;
+        const int tid = threadIdx.x;
+        for (int i0 = tid; i0 < rows; i0 += U * bd) {
+          X qv[U], pv[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * bd;
+            qv[u] = i < rows ? q[i] : X(0);
+            pv[u] = i < rows ? ps[i] : X(0);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (i0 + u * bd < rows) acc = fma((double)qv[u], (double)pv[u], acc);
+        }
+        red[tid] = acc;
+      }
+      __syncthreads();
+      if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round, red);
+      if (threadIdx.x < 32) {
+        double pq;
+        const bool ok = persist::gather_sum<false>(sh.sync, round, &pq);
+        if (threadIdx.x == 0) {
+          sh.prod.counter = bd >> 5;  // for the next product
+        const double rr = sh.rr, alpha = ok && pq > 0.0 ? rr / pq : 0.0;
+          if (!ok) {
+            sh.stop = 1;
+          } else if (!(alpha > 0.0) && rr > 0.0) {  // A is not positive definite along p: nothing is updated
+            sh.breakdown = sh.done = sh.stop = 1;
+          }
+          sh.alpha = alpha;
+        }
+      }
+      __syncthreads();
+}
+
+template <typename V, typename X>
+__device__ __noinline__ void cg_step_update(CgBlock<V, X>& sh, int round) {
+  constexpr int U = 4;  // elements a thread has in flight
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  X* const ps = reinterpret_cast<X*>(smem_raw);
+  const int bd = blockDim.x;
+  double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
+      // r -= alpha q, r.r; then x += alpha p while the sum is on its way
+      {
+        const X al = (X)sh.alpha;
+        const X* const q = sh.q;
+        X* const r = sh.r;
+        const int rows = sh.prod.rows;
+        double acc = 0.0;
+        const int tid = threadIdx.x;
+        for (int i0 = tid; i0 < rows; i0 += U * bd) {
+          X qv[U], rv[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * bd;
+            qv[u] = i < rows ? q[i] : X(0);
+            rv[u] = i < rows ? r[i] : X(0);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (i0 + u * bd < rows) {
+              rv[u] = fma(-al, qv[u], rv[u]);
+              r[i0 + u * bd] = rv[u];
+              acc = fma((double)rv[u], (double)rv[u], acc);
+            }
+        }
+        red[tid] = acc;
+      }
+      __syncthreads();
+      if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round + 1, red);
+  __syncthreads();  // the update of x would delay the sum: both need the FP64 unit
+      if (threadIdx.x >= 32 || bd == 32) {
+        const int tid = threadIdx.x;
+        const X al = (X)sh.alpha;
+        X* const x = sh.x;
+        const int rows = sh.prod.rows, ts = bd == 32 ? 32 : bd - 32;
+        for (int i0 = bd == 32 ? tid : tid - 32; i0 < rows; i0 += U * ts) {
+          X xv[U], pv[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * ts;
+            xv[u] = i < rows ? x[i] : X(0);
+            pv[u] = i < rows ? ps[i] : X(0);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (i0 + u * ts < rows) x[i0 + u * ts] = fma(al, pv[u], xv[u]);
+        }
+      }
+      if (threadIdx.x < 32) {
+        double rrn;
+        const bool ok = persist::gather_sum<false>(sh.sync, round + 1, &rrn);
+        if (threadIdx.x == 0) {
+          if (!ok) {
+            sh.stop = 1;
+          } else {
+            const int it = sh.it + 1;
+            if (blockIdx.x == 0) sh.hist[it] = rrn;
+            sh.beta = rrn / sh.rr;
+            sh.rr = rrn;
+            sh.it = it;
+            if (rrn <= sh.tol2) sh.converged = sh.stop = 1;
+            else if (!(rrn <= sh.grow_limit)) sh.breakdown = sh.stop = 1;  // non-finite or diverging
+            else if (it >= sh.max_iter) sh.stop = 1;
+            sh.done = sh.stop;
+          }
+        }
+      }
+      __syncthreads();
+}
+
+template <typename V, typename X>
+__device__ __noinline__ void cg_step_direction(CgBlock<V, X>& sh) {
+  constexpr int U = 4;  // elements a thread has in flight
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  X* const ps = reinterpret_cast<X*>(smem_raw);
+  const int bd = blockDim.x;
+      // p = r + beta p
+      {
+        const X be = (X)sh.beta;
+        const X* const r = sh.r;
+        X* const p = sh.p;
+        const int rows = sh.prod.rows;
+        const int tid = threadIdx.x;
+        for (int i0 = tid; i0 < rows; i0 += U * bd) {
+          X pv[U], rv[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * bd;
+            pv[u] = i < rows ? ps[i] : X(0);
+            rv[u] = i < rows ? r[i] : X(0);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * bd;
+            if (i < rows) {
+              const X pi = fma(be, pv[u], rv[u]);
+              ps[i] = pi;
+              p[i] = pi;
+            }
+          }
+        }
+      }
+}
+
+// MAXT 512 for blocks that are no larger: 128 registers a thread, and with them deeper batches (KB)
+template <typename V, typename X, int KB, bool RUNS, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) cg_persist_kernel(core::KArgs a, const V* __restrict__ ell_val,
+                                                             const V* __restrict__ er_val, CgPersist<X> c) {
+  using namespace core;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ CgBlock<V, X> sh;
+  X* const ps = reinterpret_cast<X*>(smem_raw);
+  const int bd = blockDim.x;
+  if (c.st->done) return;  // uniform over the grid: nobody writes it before every block has met the others
+  {
+    const int tid = threadIdx.x, blk = blockIdx.x;
+    const int pb = a.part_ptr[blk], rows = a.part_ptr[blk + 1] - pb;
+    X* r = c.r_off >= 0 ? reinterpret_cast<X*>(smem_raw + c.r_off) : c.r + pb;
+    X* x = c.x_off >= 0 ? reinterpret_cast<X*>(smem_raw + c.x_off) : c.x + pb;
+    if (tid == 0) {
+      const int it = c.st->it;
+      sh.it = it;
+      sh.max_iter = c.st->max_iter;
+      sh.tol2 = c.st->tol2;
+      sh.grow_limit = c.st->grow_limit;
+      sh.rr = c.hist[it];
+      sh.beta = 0.0;
+      sh.converged = sh.breakdown = sh.done = sh.stop = sh.seen = 0;
+      sh.q = c.q_off >= 0 ? reinterpret_cast<X*>(smem_raw + c.q_off) : c.q + pb;
+      sh.r = r;
+      sh.x = x;
+      sh.p = c.p + pb;
+      sh.hist = c.hist;
+      sh.red_off = c.red_off;
+      sh.sync = c.sync;
+      sh.nh = a.halo_ptr ? (int)(a.halo_ptr[blk + 1] - a.halo_ptr[blk]) : 0;
+      sh.halo = a.halo_ptr ? a.halo_new + a.halo_ptr[blk] : nullptr;
+    }
+    persist::init_product(&sh.prod, a, ell_val, er_val, a.er_scol, blk,
+                          c.tbl_off >= 0 ? reinterpret_cast<SliceMeta*>(smem_raw + c.tbl_off) : nullptr);
+    if (tid == 0) {
+      sh.prod.xs_off = 0;
+      sh.prod.counter = bd >> 5;
+      sh.prod.xg = c.p;
+      sh.prod.out = sh.q;
+      sh.prod.lim = rows + sh.nh;
+      sh.prod.stop = &sh.stop;
+      sh.prod.seen = &sh.seen;
+    }
+    for (int i = tid; i < rows; i += bd) {
+      ps[checked(i, a.smem_elems, a.status)] = c.p[pb + i];
+      if (c.r_off >= 0) r[i] = c.r[pb + i];
+      if (c.x_off >= 0) x[i] = c.x[pb + i];
+    }
+  }
+  __syncthreads();
+  for (int step = 0; step < c.max_steps; ++step) {
+    const int round = 2 * step + 1;  // of the sums
+    // q = A p; p of the other blocks from round `step` on (their p at launch: nothing to wait for)
+    if (sh.nh > 0) {
+      if (!persist::wait_round(sh.sync, step, &sh.seen)) sh.stop = 1;
+      for (int j = threadIdx.x; j < sh.nh; j += bd)
+        ps[checked(sh.prod.rows + j, a.smem_elems, a.status)] = load_x(c.p + checked(sh.halo[j], a.n, a.status));
+      __syncthreads();
+    }
+    persist::run_slices<V, X, KB, RUNS>(&sh.prod, &sh.sync, step);
+    __syncthreads();
+    if (sh.stop) break;
+    cg_step_pq(sh, round);
+    if (sh.stop) break;
+    cg_step_update(sh, round);
+    if (sh.stop) break;
+    cg_step_direction(sh);
+    __syncthreads();
+    if (threadIdx.x == 0) persist::arrive(sh.sync);
+  }
+  __syncthreads();
+  {
+    const X *const r = sh.r, *const x = sh.x;
+    const int rows = sh.prod.rows, pb = sh.prod.pb;
+    for (int i = threadIdx.x; i < rows; i += bd) {
+      if (c.r_off >= 0) c.r[pb + i] = r[i];
+      if (c.x_off >= 0) c.x[pb + i] = x[i];
+    }
+  }
+  // a launch that ran out of steps leaves with p updated; one that gave up has told the host already
+  if (blockIdx.x == 0 && threadIdx.x == 0 && (sh.done || !sh.stop)) {
+    c.st->it = sh.it;
+    c.st->beta = sh.beta;
+    c.st->converged = sh.converged;
+    c.st->breakdown = sh.breakdown;
+    c.st->done = sh.done;
+  }
+}
+
 double now_s() {
   return std::chrono::duration<double>(std::chrono::steady_clock::now().time_since_epoch()).count();
 }
@@ -379,7 +660,8 @@ ehyb_status_t work_get(ehyb_plan_t P, int hist_need, CgWork** out) {
   const size_t v64 = al((size_t)(n + 2) * 8), v32 = al((size_t)(n + 4) * 4);
   const size_t parts = al((size_t)kVB * 8), pq = al((size_t)(w->nparts + 1) * 8);
   const size_t hist = al((size_t)(w->hist_cap + 2) * 8), st = al(sizeof(CgState));
-  const size_t total = 6 * v64 + 4 * v32 + 2 * parts + pq + hist + st;
+  const size_t meeting = al(sizeof(persist::Meeting));
+  const size_t total = 6 * v64 + 4 * v32 + 2 * parts + pq + hist + st + meeting;
   ehyb_status_t s = device_alloc(&w->arena, total);
   if (s != EHYB_OK) {
     delete w;
@@ -400,11 +682,12 @@ ehyb_status_t work_get(ehyb_plan_t P, int hist_need, CgWork** out) {
   w->part_b = (double*)b; b += parts;
   w->pq_part = (double*)b; b += pq;
   w->hist = (double*)b; b += hist;
-  w->st = (CgState*)b;
+  w->st = (CgState*)b; b += st;
+  w->meeting = (persist::Meeting*)b;
   cudaError_t e = cudaStreamCreateWithFlags(&w->cap, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
     cg_work_free(w);
-    return cuda_error_status(e, "cudaStreamCreateWithFlags");
+    return cuda_error_status(e, "cg workspace");
   }
   P->cg = w;
   *out = w;
@@ -452,6 +735,76 @@ ehyb_status_t run_chunk(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s) {
   }
   CKC(cudaGraphLaunch(*g, s));
   return EHYB_OK;
+}
+
+// One persistent launch of at most kPersistSteps iterations; *ran = false (and nothing launched) for a plan that
+// needs the separate launches: more partitions than SMs (a block owns one partition, all blocks resident), a
+// wide slice (its sums go through the plan's workspace), the staging-fault test hook.
+constexpr int kPersistSteps = 2000;  // bounds one launch to a fraction of a second
+
+template <typename V, typename X, int KB, bool RUNS, int MAXT>
+ehyb_status_t launch_persist(ehyb_plan_t P, const V* ev, const V* erv, CgPersist<X> c, cudaStream_t s, bool* ran) {
+  const DevPlan& D = P->dev;
+  auto kernel = cg_persist_kernel<V, X, KB, RUNS, MAXT>;
+  core::KArgs a = core::make_kargs(D);
+  if (RUNS) {
+    a.ell_col = D.ell_col_low;
+    a.er_scol = D.er_scol_low;
+  }
+  int optin = 0, resident = 0, sms = 0;
+  CKC(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, P->device));
+  CKC(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device));
+  const size_t budget = (size_t)optin - 1024;
+  auto al = [](size_t b) { return (b + 15) & ~(size_t)15; };
+  size_t smem = ehyb_smem_bytes(D, (int)sizeof(X));
+  a.smem_elems = (int64_t)(smem / sizeof(X));
+  const size_t tbl = al((size_t)D.max_part_slices * sizeof(core::SliceMeta));
+  const size_t vec = al((size_t)D.max_part_rows * sizeof(X));
+  auto place = [&](size_t bytes) -> int32_t {
+    if (smem + bytes > budget) return -1;
+    const size_t o = smem;
+    smem += bytes;
+    return (int32_t)o;
+  };
+  c.red_off = place((size_t)D.threads * sizeof(double));
+  c.tbl_off = place(tbl);
+  a.meta_cap = D.max_part_slices;
+  *ran = false;
+  if (c.red_off < 0) return EHYB_OK;
+  c.q_off = place(vec);
+  c.r_off = place(vec);
+  c.x_off = place(vec);
+  CKC(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
+  CKC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, D.threads, smem));
+  *ran = D.nparts <= sms * resident && D.nparts <= persist::kMaxGrid;
+  if (!*ran) return EHYB_OK;
+  CKC(cudaMemsetAsync(c.sync.m, 0, sizeof(persist::Meeting), s));
+  void* args[] = {&a, (void*)&ev, (void*)&erv, &c};
+  CKC(cudaLaunchCooperativeKernel((const void*)kernel, dim3((unsigned)D.nparts), dim3((unsigned)D.threads), args, smem,
+                                  s));
+  return EHYB_OK;
+}
+
+ehyb_status_t run_persist(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s, bool* ran) {
+  const DevPlan& D = P->dev;
+  *ran = false;
+  if (D.wide_parts > 0 || D.inject_wait_fault || D.nparts > persist::kMaxGrid) return EHYB_OK;
+  const persist::SyncArgs sync{w->meeting, D.status, &w->st->done, std::max(D.wait_timeout_ns, persist::kMinLimitNs)};
+  if (lowp == 0) {
+    const CgPersist<double> c{w->xp, w->r, w->p, w->q, -1, -1, -1, -1, -1, kPersistSteps, w->st, w->hist, sync};
+    if (D.threads <= 512) return launch_persist<double, double, 16, false, 512>(P, D.ell_val, D.er_sval, c, s, ran);
+    return D.kbatch == 6 ? launch_persist<double, double, 6, false, 1024>(P, D.ell_val, D.er_sval, c, s, ran)
+                         : launch_persist<double, double, 8, false, 1024>(P, D.ell_val, D.er_sval, c, s, ran);
+  }
+  const CgPersist<float> c{w->d32, w->r32, w->p32, w->q32, -1, -1, -1, -1, -1, kPersistSteps, w->st, w->hist, sync};
+  const bool runs = D.lowp_group == 4, half = D.threads <= 512;
+  if (lowp == 1)
+    return !runs  ? launch_persist<float, float, 12, false, 1024>(P, D.ell_val_f32, D.er_sval_f32, c, s, ran)
+           : half ? launch_persist<float, float, 32, true, 512>(P, D.ell_val_f32, D.er_sval_f32, c, s, ran)
+                  : launch_persist<float, float, 16, true, 1024>(P, D.ell_val_f32, D.er_sval_f32, c, s, ran);
+  return !runs  ? launch_persist<uint16_t, float, 12, false, 1024>(P, D.ell_val_bf16, D.er_sval_bf16, c, s, ran)
+         : half ? launch_persist<uint16_t, float, 32, true, 512>(P, D.ell_val_bf16, D.er_sval_bf16, c, s, ran)
+                : launch_persist<uint16_t, float, 16, true, 1024>(P, D.ell_val_bf16, D.er_sval_bf16, c, s, ran);
 }
 
 ehyb_status_t read_state(CgWork* w, cudaStream_t s, CgState* out) {
@@ -548,10 +901,14 @@ ehyb_status_t fcg_solve(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s, doub
 ehyb_status_t cg_loop(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s, int* iters, int* converged,
                       int* breakdown) {
   CgState h;
+  bool persistent = true;
   for (;;) {
-    ehyb_status_t st = run_chunk(P, w, lowp, s);
+    ehyb_status_t st = EHYB_OK;
+    if (persistent) st = run_persist(P, w, lowp, s, &persistent);
+    if (st == EHYB_OK && !persistent) st = run_chunk(P, w, lowp, s);
     if (st != EHYB_OK) return st;
     if ((st = read_state(w, s, &h)) != EHYB_OK) return st;
+    if (h.done == persist::kAborted) return EHYB_ERR_TIMEOUT;
     if (h.done) break;
   }
   *iters = h.it;
