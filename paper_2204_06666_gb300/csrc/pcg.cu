@@ -14,7 +14,9 @@
 //       stores measured slower).
 // alpha, beta and the inner products never leave the device; every reduction has a fixed order, so a
 // solve is bit-reproducible.  Chunks of kChunk iterations are captured once into a CUDA graph and
-// replayed; once `done` is up the remaining launches of a chunk return at once.
+// replayed; once `done` is up the remaining launches of a chunk return at once.  Plans whose partitions are all
+// resident at once (Eq. 1's are, up to 4.4 M rows) run their iterations inside one cooperative kernel instead
+// (pcg_persist_kernel), which also leaves at the iteration that met its threshold.
 //
 // Mixed precision (ehyb_pcg_refined): one PCG that runs on FP32 vectors -- A's FP32 / BF16 values, G's
 // FP32 / BF16 values, FP32 accumulation, FP64 inner products and alpha / beta -- with FP64 residual
@@ -24,17 +26,20 @@
 // (and (r.z)_old by (s / s')^2), so the Krylov iteration is not restarted.  Stops when ||b - A x|| <= rtol ||b||.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
+#include "persist.cuh"
 #include "plan_internal.h"
 
 namespace ehyb {
 
 namespace {
 
-constexpr unsigned FULL = 0xffffffffu;
+using core::FULL;
 constexpr int kVB = 608;  // vector-kernel blocks (4 per SM; 8 per SM measured slower)
 constexpr int kVT = 256;
 constexpr int kChunk = 16;
@@ -51,11 +56,13 @@ struct PcgState {
 struct PcgWork {
   int64_t n = 0;
   int32_t hist_cap = 0, lowp = 0;
+  bool persistent[2] = {true, true};  // FP64 / FP32 iterations: until a launch form says they cannot be
   void* arena = nullptr;
   double *bp = nullptr, *xp = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr, *t = nullptr;
   float *r32 = nullptr, *t32 = nullptr, *z32 = nullptr, *p32 = nullptr, *q32 = nullptr, *d32 = nullptr;
   double *part = nullptr, *pq_part = nullptr, *rz_part = nullptr, *hist = nullptr;
   PcgState* st = nullptr;
+  persist::Meeting* meeting = nullptr;  // of the persistent kernel's blocks
   cudaStream_t cap = nullptr;
   cudaGraphExec_t graph = nullptr, graph32 = nullptr;
 };
@@ -379,6 +386,365 @@ __global__ void pcg_pupdate32_force(int64_t n, const float* __restrict__ z, floa
   for (int64_t i = gtid(); i < n; i += gstride()) p[i] = fmaf(beta, p[i], z[i]);
 }
 
+// ---- persistent iterations (persist.cuh): up to max_steps iterations of K1 .. K5 in one cooperative launch, block p
+// owning partition p's rows, which are the same rows in A's, G's and G^T's plans.  XA is the type of x, p, q
+// and r, XG that of the preconditioner's vectors.  p, r, t, q (z after the update) and x stay in shared memory as
+// far as they fit; p, r and t are mirrored to memory for the other blocks' extra rows.  The blocks meet five times
+// an iteration: for the sums p.q, r.r (which orders r for K3) and t.t, and for t and the new p, which a warp waits
+// for only when it comes to its first extra row (t.t is not needed before K5: it travels during K4).
+template <typename XA, typename XG>
+struct PcgPersist {
+  XA *x, *r, *p, *q;
+  XG *rg, *t, *z;                             // rg: r in XG's type (r itself when the types agree)
+  int32_t gs_off, q_off, r_off, t_off, x_off;  // byte offsets in dynamic shared memory; -1: in global memory
+  int32_t red_off;
+  int32_t tbl_off[3];
+  int32_t max_steps;
+  double rr_limit;
+  PcgState* st;
+  double* hist;
+  persist::SyncArgs sync;
+};
+
+// A block's state, in shared memory: thread 0's scalars (it alone divides and decides) and where the vectors are.
+template <typename VA, typename XA, typename VG, typename XG>
+struct PcgBlock {
+  double alpha, beta, rz, rz_old, tol2;
+  int it, max_iter, converged, breakdown, done, stop, seen;
+  XA *q, *r, *x, *p;  // p: the block's rows of p in memory
+  XG *z, *t, *rg;     // rg: its rows of r in memory, in XG's type
+  persist::Product<VA, XA> a;
+  persist::Product<VG, XG> g, h;
+  double* hist;
+  double rr_limit;
+  int32_t red_off, gs_off;
+  persist::SyncArgs sync;
+};
+
+// p.q and alpha
+template <typename VA, typename XA, typename VG, typename XG>
+__device__ __noinline__ void pcg_step_pq(PcgBlock<VA, XA, VG, XG>& sh, int round) {
+  constexpr int U = 4;  // elements a thread has in flight
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  XA* const ps = reinterpret_cast<XA*>(smem_raw);
+  double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
+  const int bd = blockDim.x;
+      {
+        const XA* const q = sh.q;
+        const int rows = sh.a.rows;
+        double acc = 0.0;
+        const int tid = threadIdx.x;
+        for (int i0 = tid; i0 < rows; i0 += U * bd) {
+          XA qv[U], pv[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * bd;
+            qv[u] = i < rows ? q[i] : XA(0);
+            pv[u] = i < rows ? ps[i] : XA(0);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (i0 + u * bd < rows) acc = fma((double)qv[u], (double)pv[u], acc);
+        }
+        red[tid] = acc;
+      }
+      __syncthreads();
+      if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round, red);
+      if (threadIdx.x < 32) {
+        double pq;
+        const bool ok = persist::gather_sum<false>(sh.sync, round, &pq);
+        if (threadIdx.x == 0) {
+      sh.a.counter = sh.h.counter = bd >> 5;  // for the next products of A and G^T
+          if (!ok) sh.stop = 1;
+          else if (!(pq > 0.0)) sh.breakdown = sh.done = sh.stop = 1;  // not positive definite along p (or p vanished)
+          else sh.alpha = sh.rz / pq;
+        }
+      }
+      __syncthreads();
+}
+
+template <typename VA, typename XA, typename VG, typename XG>
+__device__ __noinline__ void pcg_step_update(PcgBlock<VA, XA, VG, XG>& sh, int round) {
+  using namespace core;
+  constexpr int U = 4;  // elements a thread has in flight
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  XA* const ps = reinterpret_cast<XA*>(smem_raw);
+  XG* const gs = reinterpret_cast<XG*>(smem_raw + sh.gs_off);
+  double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
+  const int bd = blockDim.x;
+      // K2: r -= alpha q (and r for the other blocks' extra rows), r.r; then x += alpha p while the sum is on its way
+      {
+        const XA al = (XA)sh.alpha;
+        const XA* const q = sh.q;
+        XA* const r = sh.r;
+        XG* const rg = sh.rg;
+        const int rows = sh.a.rows;
+        double acc = 0.0;
+        const int tid = threadIdx.x;
+        for (int i0 = tid; i0 < rows; i0 += U * bd) {
+          XA qv[U], rv[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * bd;
+            qv[u] = i < rows ? q[i] : XA(0);
+            rv[u] = i < rows ? r[i] : XA(0);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * bd;
+            if (i < rows) {
+              rv[u] = fma(-al, qv[u], rv[u]);
+              r[i] = rv[u];
+              rg[i] = (XG)rv[u];
+              acc = fma((double)rv[u], (double)rv[u], acc);
+            }
+          }
+        }
+        red[tid] = acc;
+      }
+      __syncthreads();
+      if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<true>(sh.sync, round + 1, red);
+  __syncthreads();  // the update of x would delay the sum: both need the FP64 unit
+      if (threadIdx.x >= 32 || bd == 32) {
+        const int tid = threadIdx.x;
+        const XA al = (XA)sh.alpha;
+        XA* const x = sh.x;
+        const XA* const r = sh.r;
+        const int32_t* const n2o = sh.g.n2o;
+        const int rows = sh.a.rows, pb = sh.a.pb, ts = bd == 32 ? 32 : bd - 32, t0 = bd == 32 ? tid : tid - 32;
+        for (int i0 = t0; i0 < rows; i0 += U * ts) {
+          XA xv[U], pv[U];
+          int m[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * ts;
+            m[u] = i < rows ? checked(n2o[i] - pb, rows, sh.a.status) : 0;
+            xv[u] = i < rows ? x[i] : XA(0);
+            pv[u] = i < rows ? ps[i] : XA(0);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * ts;
+            if (i < rows) {
+              x[i] = fma(al, pv[u], xv[u]);
+              gs[checked(i, rows, sh.a.status)] = (XG)r[m[u]];  // K3's slice of r in G's row order
+            }
+          }
+        }
+      }
+      if (threadIdx.x < 32) {
+        double rr;
+        const bool ok = persist::gather_sum<true>(sh.sync, round + 1, &rr);
+        if (threadIdx.x == 0) {
+          if (!ok) {
+            sh.stop = 1;
+          } else {
+            const int it = sh.it + 1;
+            sh.it = it;
+            if (blockIdx.x == 0) sh.hist[it] = rr;
+            sh.rz_old = sh.rz;
+            if (rr <= sh.tol2) sh.converged = sh.stop = 1;
+            else if (!(rr < sh.rr_limit) || it >= sh.max_iter) sh.stop = 1;
+            sh.done = sh.stop;
+          }
+        }
+      }
+      __syncthreads();
+}
+
+// t.t, published, and K4's slice of t
+template <typename VA, typename XA, typename VG, typename XG>
+__device__ __noinline__ void pcg_step_tt(PcgBlock<VA, XA, VG, XG>& sh, int round) {
+  using namespace core;
+  constexpr int U = 4;  // elements a thread has in flight
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  XG* const gs = reinterpret_cast<XG*>(smem_raw + sh.gs_off);
+  double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
+  const int bd = blockDim.x;
+      {
+        const XG* const t = sh.t;
+        const int32_t* const n2o = sh.h.n2o;
+        const int rows = sh.a.rows, pb = sh.a.pb;
+        double acc = 0.0;
+        const int tid = threadIdx.x;
+        for (int i0 = tid; i0 < rows; i0 += U * bd) {
+          int m[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) m[u] = i0 + u * bd < rows ? checked(n2o[i0 + u * bd] - pb, rows, sh.a.status) : 0;
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * bd;
+            if (i < rows) {
+              const XG v = t[m[u]];
+              gs[checked(i, rows, sh.a.status)] = v;  // K4's slice of t in G^T's row order
+              acc = fma((double)v, (double)v, acc);
+            }
+          }
+        }
+        red[tid] = acc;
+      }
+      __syncthreads();
+      if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round + 2, red);
+}
+
+// beta from t.t, then the direction
+template <typename VA, typename XA, typename VG, typename XG>
+__device__ __noinline__ void pcg_step_direction(PcgBlock<VA, XA, VG, XG>& sh, int round) {
+  constexpr int U = 4;  // elements a thread has in flight
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  XA* const ps = reinterpret_cast<XA*>(smem_raw);
+  const int bd = blockDim.x;
+      if (threadIdx.x < 32) {
+        double tt;
+        const bool ok = persist::gather_sum<false>(sh.sync, round + 2, &tt);
+        if (threadIdx.x == 0) {
+      sh.g.counter = bd >> 5;
+          if (!ok) {
+            sh.stop = 1;
+          } else {
+            sh.rz = tt;
+            sh.beta = tt / sh.rz_old;
+          }
+        }
+      }
+      __syncthreads();
+      // K5: p = z + beta p
+      {
+        const XA be = (XA)sh.beta;
+        const XG* const z = sh.z;
+        XA* const p = sh.p;
+        const int rows = sh.a.rows;
+        const int tid = threadIdx.x;
+        for (int i0 = tid; i0 < rows; i0 += U * bd) {
+          XA pv[U], zv[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * bd;
+            pv[u] = i < rows ? ps[i] : XA(0);
+            zv[u] = i < rows ? (XA)z[i] : XA(0);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * bd;
+            if (i < rows) {
+              const XA pi = fma(be, pv[u], zv[u]);
+              ps[i] = pi;
+              p[i] = pi;
+            }
+          }
+        }
+      }
+}
+
+// MAXT 512 for blocks that are no larger: 128 registers a thread, and with them deeper batches
+template <typename VA, typename XA, int KA, typename VG, typename XG, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) pcg_persist_kernel(core::KArgs a, const VA* __restrict__ av,
+                                                              const VA* __restrict__ aev, core::KArgs g,
+                                                              const VG* __restrict__ gv, const VG* __restrict__ gev,
+                                                              core::KArgs h, const VG* __restrict__ hv,
+                                                              const VG* __restrict__ hev, PcgPersist<XA, XG> c) {
+  using namespace core;
+  constexpr bool kRunsA = sizeof(VA) < 8, kRunsG = sizeof(VG) < 8;
+  constexpr int KG = (kRunsG ? 16 : 8) * (1024 / MAXT);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ PcgBlock<VA, XA, VG, XG> sh;
+  XA* const ps = reinterpret_cast<XA*>(smem_raw);
+  const int bd = blockDim.x;
+  if (c.st->done) return;  // uniform over the grid: nobody writes it before every block has met the others
+  {
+    const int tid = threadIdx.x, blk = blockIdx.x;
+    const int pb = a.part_ptr[blk], rows = a.part_ptr[blk + 1] - pb;
+    XA* r = c.r_off >= 0 ? reinterpret_cast<XA*>(smem_raw + c.r_off) : c.r + pb;
+    XA* x = c.x_off >= 0 ? reinterpret_cast<XA*>(smem_raw + c.x_off) : c.x + pb;
+    if (tid == 0) {
+      sh.it = c.st->it;
+      sh.max_iter = c.st->max_iter;
+      sh.tol2 = c.st->tol2;
+      sh.rz = c.st->rz_new;
+      sh.rz_old = c.st->rz_old;
+      sh.converged = sh.breakdown = sh.done = sh.stop = sh.seen = 0;
+      sh.q = c.q_off >= 0 ? reinterpret_cast<XA*>(smem_raw + c.q_off) : c.q + pb;
+      sh.z = c.q_off >= 0 ? reinterpret_cast<XG*>(smem_raw + c.q_off) : c.z + pb;  // q is not read after the update
+      sh.t = c.t_off >= 0 ? reinterpret_cast<XG*>(smem_raw + c.t_off) : c.t + pb;
+      sh.r = r;
+      sh.x = x;
+      sh.p = c.p + pb;
+      sh.rg = c.rg + pb;
+      sh.hist = c.hist;
+      sh.rr_limit = c.rr_limit;
+      sh.red_off = c.red_off;
+      sh.gs_off = c.gs_off;
+      sh.sync = c.sync;
+    }
+    auto tbl = [&](int k) { return c.tbl_off[k] >= 0 ? reinterpret_cast<SliceMeta*>(smem_raw + c.tbl_off[k]) : nullptr; };
+    persist::init_product(&sh.a, a, av, aev, a.er_scol, blk, tbl(0));
+    persist::init_product(&sh.g, g, gv, gev, g.er_scol_old, blk, tbl(1));
+    persist::init_product(&sh.h, h, hv, hev, h.er_scol_old, blk, tbl(2));
+    if (tid == 0) {
+      sh.a.xs_off = 0;
+      sh.a.counter = sh.g.counter = sh.h.counter = bd >> 5;
+      sh.a.xg = c.p;
+      sh.a.out = sh.q;
+      sh.g.xs_off = sh.h.xs_off = c.gs_off;
+      sh.g.xg = c.rg;
+      sh.g.out = sh.t;
+      sh.g.mirror = c.t_off >= 0 ? c.t + pb : nullptr;
+      sh.g.n2o = g.new_to_old + pb;
+      sh.h.xg = c.t;
+      sh.h.out = sh.z;
+      sh.h.n2o = h.new_to_old + pb;
+      sh.a.stop = sh.g.stop = sh.h.stop = &sh.stop;
+      sh.a.seen = sh.g.seen = sh.h.seen = &sh.seen;
+    }
+    for (int i = tid; i < rows; i += bd) {
+      ps[checked(i, a.smem_elems, a.status)] = c.p[pb + i];
+      if (c.r_off >= 0) r[i] = c.r[pb + i];
+      if (c.x_off >= 0) x[i] = c.x[pb + i];
+    }
+  }
+  __syncthreads();
+  for (int step = 0; step < c.max_steps; ++step) {
+    const int round = 3 * step + 1;  // of the sums
+    // K1: q = A p (p of the other blocks from round 2 step on), p.q
+    persist::run_slices<VA, XA, KA, kRunsA>(&sh.a, &sh.sync, 2 * step);
+    __syncthreads();
+    if (sh.stop) break;
+    pcg_step_pq(sh, round);
+    if (sh.stop) break;
+    pcg_step_update(sh, round);
+    if (sh.stop) break;
+    // K3: t = G r, t.t = r.z
+    persist::run_slices<VG, XG, KG, kRunsG>(&sh.g, &sh.sync, 0);  // r of all blocks: ordered by the sum above
+    __syncthreads();
+    if (threadIdx.x == 0) persist::arrive(sh.sync);  // t: round 2 step + 1
+    pcg_step_tt(sh, round);
+    // K4: z = G^T t
+    persist::run_slices<VG, XG, KG, kRunsG>(&sh.h, &sh.sync, 2 * step + 1);
+    pcg_step_direction(sh, round);
+    if (sh.stop) break;
+    __syncthreads();
+    if (threadIdx.x == 0) persist::arrive(sh.sync);  // p: round 2 (step + 1)
+  }
+  __syncthreads();
+  {
+    const XA *const r = sh.r, *const x = sh.x;
+    const int rows = sh.a.rows, pb = sh.a.pb;
+    for (int i = threadIdx.x; i < rows; i += bd) {
+      if (c.r_off >= 0) c.r[pb + i] = r[i];
+      if (c.x_off >= 0) c.x[pb + i] = x[i];
+    }
+  }
+  // a launch that ran out of steps leaves with p updated; one that gave up has told the host already
+  if (blockIdx.x == 0 && threadIdx.x == 0 && (sh.done || !sh.stop)) {
+    c.st->it = sh.it;
+    c.st->rz_old = sh.rz_old;
+    c.st->rz_new = sh.rz;
+    c.st->converged = sh.converged;
+    c.st->breakdown = sh.breakdown;
+    c.st->done = sh.done;
+  }
+}
+
 #define CKP(call)                                                     \
   do {                                                                \
     cudaError_t e_ = (call);                                          \
@@ -410,7 +776,8 @@ ehyb_status_t work_get(ehyb_precond_t M, int hist_need, PcgWork** out) {
   const size_t v64 = al((size_t)(n + 2) * 8), v32 = al((size_t)(n + 4) * 4);
   const size_t parts = al((size_t)kVB * 8), pp = al((size_t)(nparts + 1) * 8);
   const size_t hist = al((size_t)(w->hist_cap + 2) * 8), st = al(sizeof(PcgState));
-  const size_t total = 7 * v64 + 6 * v32 + parts + 2 * pp + hist + st;
+  const size_t meeting = al(sizeof(persist::Meeting));
+  const size_t total = 7 * v64 + 6 * v32 + parts + 2 * pp + hist + st + meeting;
   ehyb_status_t s = device_alloc(&w->arena, total);
   if (s != EHYB_OK) {
     delete w;
@@ -425,7 +792,8 @@ ehyb_status_t work_get(ehyb_precond_t M, int hist_need, PcgWork** out) {
   w->pq_part = (double*)b; b += pp;
   w->rz_part = (double*)b; b += pp;
   w->hist = (double*)b; b += hist;
-  w->st = (PcgState*)b;
+  w->st = (PcgState*)b; b += st;
+  w->meeting = (persist::Meeting*)b;
   cudaError_t e = cudaMemsetAsync(w->arena, 0, total, 0);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&w->cap, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
@@ -483,7 +851,125 @@ ehyb_status_t enqueue_chunk32(ehyb_precond_t M, PcgWork* w, cudaStream_t s) {
   return EHYB_OK;
 }
 
+// One persistent launch of at most kPersistSteps iterations; *ran = false (and nothing launched) where the separate
+// launches are needed: more partitions than SMs, a wide slice, copies not in runs of four, vectors that do not
+// fit a block's shared memory, the staging-fault test hook.
+constexpr int kPersistSteps = 2000;  // bounds one launch to a fraction of a second
+
+template <typename VA, typename XA, int KA, typename VG, typename XG, int MAXT>
+ehyb_status_t launch_persist(ehyb_precond_t M, const VA* av, const VA* aev, const VG* gv, const VG* gev,
+                             const VG* hv, const VG* hev, PcgPersist<XA, XG> c, cudaStream_t s, bool* ran) {
+  const DevPlan &D = M->plan->dev, &G = M->g->dev, &H = M->gt->dev;
+  auto kernel = pcg_persist_kernel<VA, XA, KA, VG, XG, MAXT>;
+  auto args_of = [](const DevPlan& P, bool runs) {
+    core::KArgs a = core::make_kargs(P);
+    if (runs) {
+      a.ell_col = P.ell_col_low;
+      a.er_scol = P.er_scol_low;
+      a.er_scol_old = P.er_scol_old_low;
+    }
+    a.meta_cap = P.max_part_slices;
+    return a;
+  };
+  core::KArgs a = args_of(D, sizeof(VA) < 8), g = args_of(G, sizeof(VG) < 8), h = args_of(H, sizeof(VG) < 8);
+  int optin = 0, resident = 0, sms = 0;
+  CKP(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, M->plan->device));
+  CKP(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, M->plan->device));
+  const size_t budget = (size_t)optin - 1024;
+  auto al = [](size_t b) { return (b + 15) & ~(size_t)15; };
+  size_t smem = ehyb_smem_bytes(D, (int)sizeof(XA));
+  a.smem_elems = (int64_t)(smem / sizeof(XA));
+  auto place = [&](size_t bytes) -> int32_t {
+    if (smem + al(bytes) > budget) return -1;
+    const size_t o = smem;
+    smem += al(bytes);
+    return (int32_t)o;
+  };
+  const size_t va = (size_t)D.max_part_rows * sizeof(XA), vg = (size_t)D.max_part_rows * sizeof(XG);
+  *ran = false;
+  c.gs_off = place(vg);
+  c.red_off = place((size_t)D.threads * sizeof(double));
+  if (c.gs_off < 0 || c.red_off < 0) return EHYB_OK;
+  g.smem_elems = h.smem_elems = D.max_part_rows;
+  c.q_off = place(va);
+  c.r_off = place(va);
+  c.t_off = place(vg);
+  c.tbl_off[0] = place((size_t)D.max_part_slices * sizeof(core::SliceMeta));
+  c.tbl_off[1] = place((size_t)G.max_part_slices * sizeof(core::SliceMeta));
+  c.tbl_off[2] = place((size_t)H.max_part_slices * sizeof(core::SliceMeta));
+  c.x_off = place(va);
+  CKP(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
+  CKP(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, D.threads, smem));
+  *ran = D.nparts <= sms * resident;
+  if (!*ran) return EHYB_OK;
+  CKP(cudaMemsetAsync(c.sync.m, 0, sizeof(persist::Meeting), s));
+  void* args[] = {&a, (void*)&av, (void*)&aev, &g, (void*)&gv, (void*)&gev, &h, (void*)&hv, (void*)&hev, &c};
+  CKP(cudaLaunchCooperativeKernel((const void*)kernel, dim3((unsigned)D.nparts), dim3((unsigned)D.threads), args, smem,
+                                  s));
+  return EHYB_OK;
+}
+
+ehyb_status_t run_persist(ehyb_precond_t M, PcgWork* w, cudaStream_t s, bool inner32, bool* ran) {
+  const ehyb_plan_t P = M->plan;
+  const DevPlan &D = P->dev, &G = M->g->dev, &H = M->gt->dev;
+  *ran = false;
+  if (D.nparts > persist::kMaxGrid || D.wide_parts > 0 || G.wide_parts > 0 || H.wide_parts > 0 || D.inject_wait_fault ||
+      D.er_layout != 0 || G.er_layout != 0 || H.er_layout != 0)
+    return EHYB_OK;
+  // the three plans own the same rows block by block
+  if (M->g->host.part_ptr != P->host.part_ptr || M->gt->host.part_ptr != P->host.part_ptr) return EHYB_OK;
+  if (M->lowp && (G.lowp_group != 4 || H.lowp_group != 4)) return EHYB_OK;
+  if (inner32 && D.lowp_group != 4) return EHYB_OK;
+  const persist::SyncArgs sync{w->meeting, D.status, &w->st->done, std::max(D.wait_timeout_ns, persist::kMinLimitNs)};
+  const bool half = D.threads <= 512;
+  auto with_g = [&](auto va, const auto* av, const auto* aev, auto c, auto ka, auto mt) -> ehyb_status_t {
+    using VA = decltype(va);
+    using XA = std::remove_pointer_t<decltype(c.x)>;
+    using XG = std::remove_pointer_t<decltype(c.t)>;
+    constexpr int KA = decltype(ka)::value, MT = decltype(mt)::value;
+    if constexpr (std::is_same<XG, double>::value)
+      return launch_persist<VA, XA, KA, double, double, MT>(M, av, aev, G.ell_val, G.er_sval, H.ell_val, H.er_sval, c, s,
+                                                            ran);
+    else if (M->lowp == 1)
+      return launch_persist<VA, XA, KA, float, float, MT>(M, av, aev, G.ell_val_f32, G.er_sval_f32, H.ell_val_f32,
+                                                          H.er_sval_f32, c, s, ran);
+    else
+      return launch_persist<VA, XA, KA, uint16_t, float, MT>(M, av, aev, G.ell_val_bf16, G.er_sval_bf16, H.ell_val_bf16,
+                                                             H.er_sval_bf16, c, s, ran);
+  };
+  using std::integral_constant;
+  const integral_constant<int, 512> t512{};
+  const integral_constant<int, 1024> t1024{};
+  auto fp64 = [&](auto c) {
+    if (half) return with_g(double(), D.ell_val, D.er_sval, c, integral_constant<int, 16>(), t512);
+    return D.kbatch == 6 ? with_g(double(), D.ell_val, D.er_sval, c, integral_constant<int, 6>(), t1024)
+                         : with_g(double(), D.ell_val, D.er_sval, c, integral_constant<int, 8>(), t1024);
+  };
+  auto fp32 = [&](auto va, const auto* av, const auto* aev, auto c) {
+    return half ? with_g(va, av, aev, c, integral_constant<int, 32>(), t512)
+                : with_g(va, av, aev, c, integral_constant<int, 16>(), t1024);
+  };
+  if (inner32) {
+    const PcgPersist<float, float> c{w->d32, w->r32, w->p32, w->q32, w->r32, w->t32, w->z32, -1, -1, -1, -1, -1, -1,
+                                     {-1, -1, -1}, kPersistSteps, 1e30, w->st, w->hist, sync};
+    return P->lowp == 1 ? fp32(float(), D.ell_val_f32, D.er_sval_f32, c)
+                        : fp32(uint16_t(), D.ell_val_bf16, D.er_sval_bf16, c);
+  }
+  if (M->lowp) {
+    const PcgPersist<double, float> c{w->xp, w->r, w->p, w->q, w->r32, w->t32, w->z32, -1, -1, -1, -1, -1, -1,
+                                      {-1, -1, -1}, kPersistSteps, 1e300, w->st, w->hist, sync};
+    return fp64(c);
+  }
+  const PcgPersist<double, double> c{w->xp, w->r, w->p, w->q, w->r, w->t, w->z, -1, -1, -1, -1, -1, -1,
+                                     {-1, -1, -1}, kPersistSteps, 1e300, w->st, w->hist, sync};
+  return fp64(c);
+}
+
 ehyb_status_t run_chunk(ehyb_precond_t M, PcgWork* w, cudaStream_t s, bool inner32 = false) {
+  if (w->persistent[inner32]) {
+    const ehyb_status_t st = run_persist(M, w, s, inner32, &w->persistent[inner32]);
+    if (st != EHYB_OK || w->persistent[inner32]) return st;
+  }
   cudaGraphExec_t* g = inner32 ? &w->graph32 : &w->graph;
   if (!*g) {
     cudaGraph_t graph;
@@ -556,6 +1042,7 @@ extern "C" ehyb_status_t ehyb_pcg(ehyb_plan_t P, ehyb_precond_t M, const double*
   for (;;) {
     CKP(cudaMemcpyAsync(&h, w->st, sizeof(h), cudaMemcpyDeviceToHost, s));
     CKP(cudaStreamSynchronize(s));
+    if (h.done == persist::kAborted) return EHYB_ERR_TIMEOUT;
     if (h.done) break;
     if ((st = run_chunk(M, w, s)) != EHYB_OK) return st;
   }
@@ -640,6 +1127,7 @@ extern "C" ehyb_status_t ehyb_pcg_refined(ehyb_plan_t P, ehyb_precond_t M, const
       for (;;) {
         CKP(cudaMemcpyAsync(&h, w->st, sizeof(h), cudaMemcpyDeviceToHost, s));
         CKP(cudaStreamSynchronize(s));
+        if (h.done == persist::kAborted) return EHYB_ERR_TIMEOUT;
         if (h.done) break;
         if ((st = run_chunk(M, w, s, true)) != EHYB_OK) return st;
       }
