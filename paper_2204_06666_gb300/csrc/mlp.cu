@@ -73,10 +73,10 @@ __device__ __forceinline__ void dense_relu(const float* W, const float* bias, co
 // One block's samples [blockIdx.x * per, ...): forward (BWD false: outputs to `out`), or forward, squared error
 // against T and the gradient summed over the block's samples, to part + kPart * blockIdx.x; with `direct` (one
 // block) the mean-squared-error loss and the gradient themselves.  Global reads are scalar: the caller's
-// arrays are aligned to their element only.
+// arrays are aligned to their element only.  No __restrict__ on what an earlier kernel of the stream may still
+// be writing when this one becomes resident: such loads must not be moved across the wait.
 template <bool BWD>
-__global__ void __launch_bounds__(kMlpT) mlp_kernel(const float* __restrict__ P, const float* __restrict__ X,
-                                                    const float* __restrict__ T, int B, int per, float* part,
+__global__ void __launch_bounds__(kMlpT) mlp_kernel(const float* P, const float* X, const float* T, int B, int per, float* part,
                                                     float* grad, float* loss, int direct) {
   __shared__ __align__(16) MlpSmem m;
   const int t = threadIdx.x;
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kMlpT) mlp_kernel(const float* __restrict__ P,
 // gradient = sum of the blocks' partial gradients, loss = the mean of their squared errors.  32 parameters a
 // block, eight warps each summing every eighth partial, then the eight sums in order; the last block takes
 // the loss.
-__global__ void __launch_bounds__(256) mlp_reduce(const float* __restrict__ part, int nb, int B, float* grad,
+__global__ void __launch_bounds__(256) mlp_reduce(const float* part, int nb, int B, float* grad,
                                                   float* loss) {
   __shared__ float ws[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(256) mlp_reduce(const float* __restrict__ part
   }
 }
 
-__global__ void adam_kernel(float* p, float* m, float* v, const float* __restrict__ g, int count, float lr,
+__global__ void adam_kernel(float* p, float* m, float* v, const float* g, int count, float lr,
                             float b1, float b2, float eps, float c1, float c2) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   pdl_launch_dependents();
