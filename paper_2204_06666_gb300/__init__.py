@@ -189,18 +189,41 @@ def _check(st: int, where: str):
         raise EhybError(st, where)
 
 
+_raw_stream = _device = None   # torch's own lookups of the current stream's handle and the current device
+
+
 def _stream(stream) -> int | None:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        # every product asks for the current stream: past the first call (which initialises CUDA) its handle is
+        # read without building a Stream object (2.1 us of a 6.9 us call on the smallest matrices, with _dev)
+        if _raw_stream is not None:
+            return _raw_stream(_device())
+        return _first_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
 
 
+def _first_stream() -> int:
+    global _raw_stream, _device
+    import torch
+    s = torch.cuda.current_stream().cuda_stream
+    raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if raw is not None and dev is not None:
+        _raw_stream, _device = raw, dev
+    return s
+
+
+_DTYPES: dict = {}   # dtype name -> torch dtype
+
+
 def _dev(t, dtype_name: str) -> int:
     """Device pointer of a contiguous CUDA tensor of the given dtype."""
-    if not (t.is_cuda and t.is_contiguous() and str(t.dtype) == "torch." + dtype_name):
+    dt = _DTYPES.get(dtype_name)
+    if dt is None:
+        import torch
+        dt = _DTYPES[dtype_name] = getattr(torch, dtype_name)
+    if not (t.is_cuda and t.is_contiguous() and t.dtype is dt):
         raise TypeError(f"expected a contiguous CUDA torch.{dtype_name} tensor, got {t.dtype} on {t.device}")
     return t.data_ptr()
 
@@ -292,6 +315,10 @@ def ehyb_test_bounds_probe(i: int, lim: int) -> int:
     return int(_lib.ehyb_test_bounds_probe(int(i), int(lim)))
 
 
+# the products' entry points, looked up once: a product of a small matrix takes as long as the call that asks for it
+_spmv, _spmv_permuted, _spmv_lowp = _lib.ehyb_spmv, _lib.ehyb_spmv_permuted, _lib.ehyb_spmv_lowp
+
+
 # ---------------------------------------------------------------- owning wrappers
 
 class Plan:
@@ -348,11 +375,14 @@ class Plan:
             pass
 
     def spmv(self, x, y, stream=None):
-        _check(ehyb_spmv(self._h, _dev(x, "float64"), _dev(y, "float64"), _stream(stream)), "ehyb_spmv")
+        st = _spmv(self._h, _dev(x, "float64"), _dev(y, "float64"), _stream(stream))
+        if st:
+            raise EhybError(st, "ehyb_spmv")
 
     def spmv_permuted(self, xp, yp, stream=None):
-        _check(ehyb_spmv_permuted(self._h, _dev(xp, "float64"), _dev(yp, "float64"), _stream(stream)),
-               "ehyb_spmv_permuted")
+        st = _spmv_permuted(self._h, _dev(xp, "float64"), _dev(yp, "float64"), _stream(stream))
+        if st:
+            raise EhybError(st, "ehyb_spmv_permuted")
 
     def permute(self, to_new: bool, x, y, stream=None):
         _check(ehyb_permute(self._h, int(bool(to_new)), _dev(x, "float64"), _dev(y, "float64"), _stream(stream)),
@@ -371,7 +401,9 @@ class Plan:
         _check(_lib.ehyb_spmv_host_many(self._h, len(xs), X, Y, _stream(stream)), "ehyb_spmv_host_many")
 
     def spmv_lowp(self, x, y, stream=None):
-        _check(ehyb_spmv_lowp(self._h, _dev(x, "float32"), _dev(y, "float32"), _stream(stream)), "ehyb_spmv_lowp")
+        st = _spmv_lowp(self._h, _dev(x, "float32"), _dev(y, "float32"), _stream(stream))
+        if st:
+            raise EhybError(st, "ehyb_spmv_lowp")
 
     def spmv_noalloc(self, x, y, stream=None):
         _check(ehyb_spmv_noalloc(self._h, _dev(x, "float64"), _dev(y, "float64"), _stream(stream)),

@@ -98,3 +98,32 @@ def test_chain_of_products_in_stream_order():
             plan.spmv(b, a)
         outs.append(a.cpu().numpy())
     assert np.array_equal(outs[0], outs[1])
+
+
+def test_products_run_on_the_current_stream():
+    # the binding asks torch for the current stream at every call, also after the first one
+    import threading
+
+    import paper_2204_06666_gb300 as eh
+    side, other = torch.cuda.Stream(), torch.cuda.Stream()
+    assert eh._stream(None) == torch.cuda.current_stream().cuda_stream
+    with torch.cuda.stream(side):
+        assert eh._stream(None) == side.cuda_stream
+        seen = []
+
+        def look():
+            with torch.cuda.stream(other):
+                seen.append(eh._stream(None))
+            seen.append(eh._stream(None))
+        t = threading.Thread(target=look)
+        t.start()
+        t.join()
+        assert seen == [other.cuda_stream, torch.cuda.default_stream().cuda_stream]
+        assert eh._stream(None) == side.cuda_stream
+    assert eh._stream(side) == side.cuda_stream and eh._stream(7) == 7
+    with pytest.raises(TypeError):
+        eh._dev(torch.zeros(3, dtype=torch.float32, device="cuda"), "float64")
+    with pytest.raises(TypeError):
+        eh._dev(torch.zeros(4, 4, dtype=torch.float64, device="cuda")[:, 1], "float64")
+    with pytest.raises(TypeError):
+        eh._dev(torch.zeros(3, dtype=torch.float64), "float64")
