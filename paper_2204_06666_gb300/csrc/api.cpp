@@ -190,6 +190,70 @@ WideLists wide_lists(int32_t nparts, const std::vector<int32_t>& slice_ptr, cons
   return L;
 }
 
+// Slots per staged column from which staging pays, measured (FP32 / BF16 product, gathers -> staged): elasticity 45^3,
+// 15.7 slots a column, 29.2 -> 26.6 / 23.1 -> 15.9 us; scalar hexahedra 60^3, about 6.5, 10.5 -> 11.0; tets, 4.2, even.
+static constexpr int64_t kSlotsPerHaloColumn = 10;
+
+bool low_halo(const HostPlan& H, int64_t max_stage, int threads, LowHalo& out) {
+  const int T = planner_threads(threads);
+  const int64_t slots = (int64_t)H.er_scol_low.size();
+  out = LowHalo();
+  if (slots == 0 || (int64_t)H.ell_col_low.size() > 10 * slots) return false;  // extra rows below about a tenth
+  std::vector<std::vector<int32_t>> cols((size_t)H.nparts);
+  auto range = [&](int32_t p, int64_t& k0, int64_t& k1) {
+    k0 = H.er_slice_pos[(size_t)H.slice_ptr[(size_t)p]];
+    k1 = H.er_slice_pos[(size_t)H.slice_ptr[(size_t)p + 1]];
+  };
+  parallel_for(H.nparts, T, [&](int64_t lo, int64_t hi) {
+    std::vector<int32_t> seen((size_t)H.n, -1);
+    for (int64_t p = lo; p < hi; ++p) {
+      int64_t k0, k1;
+      range((int32_t)p, k0, k1);
+      std::vector<int32_t>& c = cols[(size_t)p];
+      for (int64_t k = k0; k < k1; ++k) {
+        const int32_t v = H.er_scol_low[(size_t)k];
+        if (seen[(size_t)v] != (int32_t)p) {
+          seen[(size_t)v] = (int32_t)p;
+          c.push_back(v);
+        }
+      }
+      std::sort(c.begin(), c.end());
+    }
+  }, 1);
+  out.ptr.assign((size_t)H.nparts + 1, 0);
+  for (int32_t p = 0; p < H.nparts; ++p) {
+    const int64_t m = (int64_t)cols[(size_t)p].size();
+    const int64_t rows = H.part_ptr[(size_t)p + 1] - H.part_ptr[(size_t)p];
+    out.ptr[(size_t)p + 1] = out.ptr[(size_t)p] + m;
+    out.max_cols = (int32_t)std::max<int64_t>(out.max_cols, m);
+    out.max_stage = (int32_t)std::max<int64_t>(out.max_stage, rows + m);
+  }
+  const int64_t total = out.ptr[(size_t)H.nparts];
+  if (out.max_stage > max_stage || out.max_cols > 65536 || slots < kSlotsPerHaloColumn * total) {
+    out = LowHalo();
+    return false;
+  }
+  out.col_new.resize((size_t)total);
+  out.col_old.resize((size_t)total);
+  out.hcol.resize((size_t)slots);
+  parallel_for(H.nparts, T, [&](int64_t lo, int64_t hi) {
+    std::vector<int32_t> rank((size_t)H.n, 0);
+    for (int64_t p = lo; p < hi; ++p) {
+      int64_t k0, k1;
+      range((int32_t)p, k0, k1);
+      const std::vector<int32_t>& c = cols[(size_t)p];
+      const int64_t o = out.ptr[(size_t)p];
+      for (size_t t = 0; t < c.size(); ++t) {
+        rank[(size_t)c[t]] = (int32_t)t;
+        out.col_new[(size_t)o + t] = c[t];
+        out.col_old[(size_t)o + t] = H.new_to_old[(size_t)c[t]];
+      }
+      for (int64_t k = k0; k < k1; ++k) out.hcol[(size_t)k] = (uint16_t)rank[(size_t)H.er_scol_low[(size_t)k]];
+    }
+  }, 1);
+  return true;
+}
+
 const DevPlan* plan_device_view(ehyb_plan_t plan, int* device) {
   if (!plan || plan->host_only) return nullptr;
   if (device) *device = plan->device;
@@ -481,6 +545,24 @@ ehyb_status_t plan_finalize(std::unique_ptr<ehyb_plan_s>& P, const ehyb_options_
     const size_t o_hp = A.add<int64_t>(H.halo_ptr.size());
     const size_t o_hn = A.add<int32_t>(H.halo_new.size());
     const size_t o_ho = A.add<int32_t>(H.halo_old.size());
+    LowHalo LH;
+    if (opt.lowp && H.er_layout == 0 && H.lowp_group == 4 && W.parts == 0) {
+      int optin = 0;
+      cudaError_t e0 = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, d.dev);
+      if (e0 != cudaSuccess) return cuda_fail(e0, "cudaDeviceGetAttribute");
+      try {  // FP32 elements of x, and the alignment slack
+        if (low_halo(H, ((int64_t)optin - 1024) / 4 - 8, opt.host_threads, LH)) {
+          D.max_low_halo = LH.max_cols;
+          D.low_stage_rows = LH.max_stage;
+        }
+      } catch (const std::bad_alloc&) {
+        return EHYB_ERR_OOM;
+      }
+    }
+    const size_t o_lhp = A.add<int64_t>(LH.ptr.size());
+    const size_t o_lhn = A.add<int32_t>(LH.col_new.size());
+    const size_t o_lho = A.add<int32_t>(LH.col_old.size());
+    const size_t o_lhc = A.add<uint16_t>(LH.hcol.size());
     const bool halo_wide = W.parts > 0 && H.er_layout == 2;
     const size_t o_sw = A.add<int32_t>(W.slice_wide.size());
     const size_t o_up = A.add<int32_t>(W.unit_ptr.size());
@@ -510,6 +592,7 @@ ehyb_status_t plan_finalize(std::unique_ptr<ehyb_plan_s>& P, const ehyb_options_
     UP(o_erv16, H.er_val_bf16) UP(o_esp, H.er_slice_pos) UP(o_so, H.slice_order) UP(o_esc, H.er_scol) UP(o_eso, H.er_scol_old) UP(o_esv, H.er_sval)
     UP(o_esv32, H.er_sval_f32) UP(o_esv16, H.er_sval_bf16) UP(o_ecl, H.ell_col_low) UP(o_escl, H.er_scol_low)
     UP(o_esol, H.er_scol_old_low) UP(o_hp, H.halo_ptr) UP(o_hn, H.halo_new) UP(o_ho, H.halo_old)
+    UP(o_lhp, LH.ptr) UP(o_lhn, LH.col_new) UP(o_lho, LH.col_old) UP(o_lhc, LH.hcol)
     UP(o_sw, W.slice_wide) UP(o_up, W.unit_ptr) UP(o_un, W.units) UP(o_wp, W.wide_ptr) UP(o_ws, W.wides)
     if (halo_wide) {
       UP(o_rc, H.row_ell_count) UP(o_re, H.row_er_count)
@@ -549,6 +632,12 @@ ehyb_status_t plan_finalize(std::unique_ptr<ehyb_plan_s>& P, const ehyb_options_
     D.halo_ptr = (const int64_t*)(base + o_hp);
     D.halo_new = (const int32_t*)(base + o_hn);
     D.halo_old = (const int32_t*)(base + o_ho);
+    if (!LH.hcol.empty()) {
+      D.low_halo_ptr = (const int64_t*)(base + o_lhp);
+      D.low_halo_new = (const int32_t*)(base + o_lhn);
+      D.low_halo_old = (const int32_t*)(base + o_lho);
+      D.er_hcol_low = (const uint16_t*)(base + o_lhc);
+    }
     if (W.parts > 0) {
       D.slice_wide = (const int32_t*)(base + o_sw);
       D.unit_ptr = (const int32_t*)(base + o_up);

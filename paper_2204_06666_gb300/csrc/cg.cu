@@ -390,43 +390,43 @@ __device__ __noinline__ void cg_step_pq(CgBlock<V, X>& sh, int round) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   X* const ps = reinterpret_cast<X*>(smem_raw);
   const int bd = blockDim.x;
-      double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
-      {
-        const X* const q = sh.q;
-        const int rows = sh.prod.rows;
-        double acc = 0.0;
-        const int tid = threadIdx.x;
-        for (int i0 = tid; i0 < rows; i0 += U * bd) {
-          X qv[U], pv[U];
+  double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
+  {
+    const X* const q = sh.q;
+    const int rows = sh.prod.rows;
+    double acc = 0.0;
+    const int tid = threadIdx.x;
+    for (int i0 = tid; i0 < rows; i0 += U * bd) {
+      X qv[U], pv[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * bd;
-            qv[u] = i < rows ? q[i] : X(0);
-            pv[u] = i < rows ? ps[i] : X(0);
-          }
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * bd;
+        qv[u] = i < rows ? q[i] : X(0);
+        pv[u] = i < rows ? ps[i] : X(0);
+      }
 #pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (i0 + u * bd < rows) acc = fma((double)qv[u], (double)pv[u], acc);
-        }
-        red[tid] = acc;
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * bd < rows) acc = fma((double)qv[u], (double)pv[u], acc);
+    }
+    red[tid] = acc;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round, red);
+  if (threadIdx.x < 32) {
+    double pq;
+    const bool ok = persist::gather_sum<false>(sh.sync, round, &pq);
+    if (threadIdx.x == 0) {
+      sh.prod.counter = bd >> 5;  // for the next product
+    const double rr = sh.rr, alpha = ok && pq > 0.0 ? rr / pq : 0.0;
+      if (!ok) {
+        sh.stop = 1;
+      } else if (!(alpha > 0.0) && rr > 0.0) {  // A is not positive definite along p: nothing is updated
+        sh.breakdown = sh.done = sh.stop = 1;
       }
-      __syncthreads();
-      if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round, red);
-      if (threadIdx.x < 32) {
-        double pq;
-        const bool ok = persist::gather_sum<false>(sh.sync, round, &pq);
-        if (threadIdx.x == 0) {
-          sh.prod.counter = bd >> 5;  // for the next product
-        const double rr = sh.rr, alpha = ok && pq > 0.0 ? rr / pq : 0.0;
-          if (!ok) {
-            sh.stop = 1;
-          } else if (!(alpha > 0.0) && rr > 0.0) {  // A is not positive definite along p: nothing is updated
-            sh.breakdown = sh.done = sh.stop = 1;
-          }
-          sh.alpha = alpha;
-        }
-      }
-      __syncthreads();
+      sh.alpha = alpha;
+    }
+  }
+  __syncthreads();
 }
 
 template <typename V, typename X>
@@ -436,73 +436,73 @@ __device__ __noinline__ void cg_step_update(CgBlock<V, X>& sh, int round) {
   X* const ps = reinterpret_cast<X*>(smem_raw);
   const int bd = blockDim.x;
   double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
-      // r -= alpha q, r.r; then x += alpha p while the sum is on its way
-      {
-        const X al = (X)sh.alpha;
-        const X* const q = sh.q;
-        X* const r = sh.r;
-        const int rows = sh.prod.rows;
-        double acc = 0.0;
-        const int tid = threadIdx.x;
-        for (int i0 = tid; i0 < rows; i0 += U * bd) {
-          X qv[U], rv[U];
+  // r -= alpha q, r.r; then x += alpha p while the sum is on its way
+  {
+    const X al = (X)sh.alpha;
+    const X* const q = sh.q;
+    X* const r = sh.r;
+    const int rows = sh.prod.rows;
+    double acc = 0.0;
+    const int tid = threadIdx.x;
+    for (int i0 = tid; i0 < rows; i0 += U * bd) {
+      X qv[U], rv[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * bd;
-            qv[u] = i < rows ? q[i] : X(0);
-            rv[u] = i < rows ? r[i] : X(0);
-          }
-#pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (i0 + u * bd < rows) {
-              rv[u] = fma(-al, qv[u], rv[u]);
-              r[i0 + u * bd] = rv[u];
-              acc = fma((double)rv[u], (double)rv[u], acc);
-            }
-        }
-        red[tid] = acc;
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * bd;
+        qv[u] = i < rows ? q[i] : X(0);
+        rv[u] = i < rows ? r[i] : X(0);
       }
-      __syncthreads();
-      if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round + 1, red);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * bd < rows) {
+          rv[u] = fma(-al, qv[u], rv[u]);
+          r[i0 + u * bd] = rv[u];
+          acc = fma((double)rv[u], (double)rv[u], acc);
+        }
+    }
+    red[tid] = acc;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round + 1, red);
   __syncthreads();  // the update of x would delay the sum: both need the FP64 unit
-      if (threadIdx.x >= 32 || bd == 32) {
-        const int tid = threadIdx.x;
-        const X al = (X)sh.alpha;
-        X* const x = sh.x;
-        const int rows = sh.prod.rows, ts = bd == 32 ? 32 : bd - 32;
-        for (int i0 = bd == 32 ? tid : tid - 32; i0 < rows; i0 += U * ts) {
-          X xv[U], pv[U];
+  if (threadIdx.x >= 32 || bd == 32) {
+    const int tid = threadIdx.x;
+    const X al = (X)sh.alpha;
+    X* const x = sh.x;
+    const int rows = sh.prod.rows, ts = bd == 32 ? 32 : bd - 32;
+    for (int i0 = bd == 32 ? tid : tid - 32; i0 < rows; i0 += U * ts) {
+      X xv[U], pv[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * ts;
-            xv[u] = i < rows ? x[i] : X(0);
-            pv[u] = i < rows ? ps[i] : X(0);
-          }
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * ts;
+        xv[u] = i < rows ? x[i] : X(0);
+        pv[u] = i < rows ? ps[i] : X(0);
+      }
 #pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (i0 + u * ts < rows) x[i0 + u * ts] = fma(al, pv[u], xv[u]);
-        }
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * ts < rows) x[i0 + u * ts] = fma(al, pv[u], xv[u]);
+    }
+  }
+  if (threadIdx.x < 32) {
+    double rrn;
+    const bool ok = persist::gather_sum<false>(sh.sync, round + 1, &rrn);
+    if (threadIdx.x == 0) {
+      if (!ok) {
+        sh.stop = 1;
+      } else {
+        const int it = sh.it + 1;
+        if (blockIdx.x == 0) sh.hist[it] = rrn;
+        sh.beta = rrn / sh.rr;
+        sh.rr = rrn;
+        sh.it = it;
+        if (rrn <= sh.tol2) sh.converged = sh.stop = 1;
+        else if (!(rrn <= sh.grow_limit)) sh.breakdown = sh.stop = 1;  // non-finite or diverging
+        else if (it >= sh.max_iter) sh.stop = 1;
+        sh.done = sh.stop;
       }
-      if (threadIdx.x < 32) {
-        double rrn;
-        const bool ok = persist::gather_sum<false>(sh.sync, round + 1, &rrn);
-        if (threadIdx.x == 0) {
-          if (!ok) {
-            sh.stop = 1;
-          } else {
-            const int it = sh.it + 1;
-            if (blockIdx.x == 0) sh.hist[it] = rrn;
-            sh.beta = rrn / sh.rr;
-            sh.rr = rrn;
-            sh.it = it;
-            if (rrn <= sh.tol2) sh.converged = sh.stop = 1;
-            else if (!(rrn <= sh.grow_limit)) sh.breakdown = sh.stop = 1;  // non-finite or diverging
-            else if (it >= sh.max_iter) sh.stop = 1;
-            sh.done = sh.stop;
-          }
-        }
-      }
-      __syncthreads();
+    }
+  }
+  __syncthreads();
 }
 
 template <typename V, typename X>
@@ -511,32 +511,32 @@ __device__ __noinline__ void cg_step_direction(CgBlock<V, X>& sh) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   X* const ps = reinterpret_cast<X*>(smem_raw);
   const int bd = blockDim.x;
-      // p = r + beta p
-      {
-        const X be = (X)sh.beta;
-        const X* const r = sh.r;
-        X* const p = sh.p;
-        const int rows = sh.prod.rows;
-        const int tid = threadIdx.x;
-        for (int i0 = tid; i0 < rows; i0 += U * bd) {
-          X pv[U], rv[U];
+  // p = r + beta p
+  {
+    const X be = (X)sh.beta;
+    const X* const r = sh.r;
+    X* const p = sh.p;
+    const int rows = sh.prod.rows;
+    const int tid = threadIdx.x;
+    for (int i0 = tid; i0 < rows; i0 += U * bd) {
+      X pv[U], rv[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * bd;
-            pv[u] = i < rows ? ps[i] : X(0);
-            rv[u] = i < rows ? r[i] : X(0);
-          }
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * bd;
+        pv[u] = i < rows ? ps[i] : X(0);
+        rv[u] = i < rows ? r[i] : X(0);
+      }
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * bd;
-            if (i < rows) {
-              const X pi = fma(be, pv[u], rv[u]);
-              ps[i] = pi;
-              p[i] = pi;
-            }
-          }
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * bd;
+        if (i < rows) {
+          const X pi = fma(be, pv[u], rv[u]);
+          ps[i] = pi;
+          p[i] = pi;
         }
       }
+    }
+  }
 }
 
 // MAXT 512 for blocks that are no larger: 128 registers a thread, and with them deeper batches (KB)

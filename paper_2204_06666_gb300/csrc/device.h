@@ -74,6 +74,14 @@ struct DevPlan {
   double* wide_ws = nullptr;
   const int32_t* row_cin = nullptr;
   const int32_t* row_cer = nullptr;
+  // staged extra rows of the FP32 / BF16 copies in runs (er_hcol_low; low_halo in plan_internal.h): per partition the
+  // distinct columns of its sliced extra rows, and 16-bit columns into them in the copies' slot layout
+  const uint16_t* er_hcol_low = nullptr;
+  const int64_t* low_halo_ptr = nullptr;
+  const int32_t* low_halo_new = nullptr;
+  const int32_t* low_halo_old = nullptr;
+  int32_t max_low_halo = 0;    // most columns of one partition
+  int32_t low_stage_rows = 0;  // most rows + columns of one partition
   int32_t* status = nullptr;  // device status word (first fault wins)
   uint64_t wait_timeout_ns = 1000000000ull;
   int32_t inject_wait_fault = 0;

@@ -489,6 +489,7 @@ struct KArgs {
   int32_t wide_parts;     // parts in the workspace (checked build only)
   const int32_t* row_cin;   // er_layout 2 with one lane per row: slab / extra entries of each row (else null)
   const int32_t* row_cer;
+  const uint16_t* er_hcol;  // staged extra rows (HER kernels; halo_* lists their columns): 16-bit columns, else null
   int32_t meta_off;       // byte offset of the partition's slice table in dynamic shared memory (0: none)
   int32_t meta_cap;       //   ... and its capacity in entries (checked build only)
 };
@@ -572,13 +573,15 @@ struct BlockState {
 // TABLE: the launch may provide the partition's slice table (a.meta_off); without it only the global path is
 // compiled (the persistent batch kernel, whose blocks run many partitions one after the other).
 // WIDE: the plan has wide slices.
+// HER: the extra rows' x is staged too (a.halo_*, a.er_hcol) and their slots run like the slab's: same order, same bits.
 // sub, nsub: the block takes every nsub-th slice of the processing order, from the sub-th on (nsub > 1: several
 // blocks share a partition of a batch; not with WIDE, whose partial sums are combined by one block).
 // PDL: the kernel was launched with programmatic stream serialization and has not yet waited for the previous
 // grid: the slice table, which reads plan arrays only, is filled first, then griddepcontrol.wait, then every
 // read of x (and of the solver's skip flag) and every write of y.
 template <typename V, typename X, bool SCATTER, bool ER_SLICED, bool DOT = false, bool GATHER = false,
-          int KB = kBatch, bool RUNS = false, bool TABLE = false, bool PDL = false, bool WIDE = false>
+          int KB = kBatch, bool RUNS = false, bool TABLE = false, bool PDL = false, bool WIDE = false,
+          bool HER = false>
 __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restrict__ ell_val,
                                                const V* __restrict__ er_val, const X* __restrict__ xp,
                                                X* __restrict__ y, const int p, X* xs, BlockState& bs,
@@ -788,7 +791,9 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
       part = -1;
     } else if constexpr (RUNS) {  // the copy in runs of four slots (its own column arrays are in a.ell_col / a.er_scol*)
       acc = slab_dot_runs<V, X, KB>(ell_val + pos, a.ell_col + pos, lane, w, xsl, X(0), pe - pb + nh, a.status);
-      if (ER_SLICED)
+      if constexpr (HER)
+        acc = slab_dot_runs<V, X, KB>(er_val + epos, a.er_hcol + epos, lane, we, xsl + (pe - pb), acc, nh, a.status);
+      else if (ER_SLICED)
         acc = er_dot_runs<V, X>(er_val + epos, (GATHER ? a.er_scol_old : a.er_scol) + epos, lane, we, xp, acc, a.n_x,
                                 a.status);
     } else {
@@ -1076,6 +1081,7 @@ inline KArgs make_kargs(const DevPlan& P) {
   a.wide_parts = P.wide_parts;
   a.row_cin = P.row_cin;
   a.row_cer = P.row_cer;
+  a.er_hcol = nullptr;
   a.meta_off = 0;
   a.meta_cap = 0;
   return a;

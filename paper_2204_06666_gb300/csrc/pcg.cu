@@ -398,6 +398,7 @@ struct PcgPersist {
   XG *rg, *t, *z;                             // rg: r in XG's type (r itself when the types agree)
   int32_t gs_off, q_off, r_off, t_off, x_off;  // byte offsets in dynamic shared memory; -1: in global memory
   int32_t red_off;
+  int32_t h_off;                              // r, then t, staged for the extra rows of G and G^T (-1: gathered)
   int32_t tbl_off[3];
   int32_t max_steps;
   double rr_limit;
@@ -429,38 +430,38 @@ __device__ __noinline__ void pcg_step_pq(PcgBlock<VA, XA, VG, XG>& sh, int round
   XA* const ps = reinterpret_cast<XA*>(smem_raw);
   double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
   const int bd = blockDim.x;
-      {
-        const XA* const q = sh.q;
-        const int rows = sh.a.rows;
-        double acc = 0.0;
-        const int tid = threadIdx.x;
-        for (int i0 = tid; i0 < rows; i0 += U * bd) {
-          XA qv[U], pv[U];
+  {
+    const XA* const q = sh.q;
+    const int rows = sh.a.rows;
+    double acc = 0.0;
+    const int tid = threadIdx.x;
+    for (int i0 = tid; i0 < rows; i0 += U * bd) {
+      XA qv[U], pv[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * bd;
-            qv[u] = i < rows ? q[i] : XA(0);
-            pv[u] = i < rows ? ps[i] : XA(0);
-          }
-#pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (i0 + u * bd < rows) acc = fma((double)qv[u], (double)pv[u], acc);
-        }
-        red[tid] = acc;
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * bd;
+        qv[u] = i < rows ? q[i] : XA(0);
+        pv[u] = i < rows ? ps[i] : XA(0);
       }
-      __syncthreads();
-      if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round, red);
-      if (threadIdx.x < 32) {
-        double pq;
-        const bool ok = persist::gather_sum<false>(sh.sync, round, &pq);
-        if (threadIdx.x == 0) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * bd < rows) acc = fma((double)qv[u], (double)pv[u], acc);
+    }
+    red[tid] = acc;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round, red);
+  if (threadIdx.x < 32) {
+    double pq;
+    const bool ok = persist::gather_sum<false>(sh.sync, round, &pq);
+    if (threadIdx.x == 0) {
       sh.a.counter = sh.h.counter = bd >> 5;  // for the next products of A and G^T
-          if (!ok) sh.stop = 1;
-          else if (!(pq > 0.0)) sh.breakdown = sh.done = sh.stop = 1;  // not positive definite along p (or p vanished)
-          else sh.alpha = sh.rz / pq;
-        }
-      }
-      __syncthreads();
+      if (!ok) sh.stop = 1;
+      else if (!(pq > 0.0)) sh.breakdown = sh.done = sh.stop = 1;  // not positive definite along p (or p vanished)
+      else sh.alpha = sh.rz / pq;
+    }
+  }
+  __syncthreads();
 }
 
 template <typename VA, typename XA, typename VG, typename XG>
@@ -472,84 +473,84 @@ __device__ __noinline__ void pcg_step_update(PcgBlock<VA, XA, VG, XG>& sh, int r
   XG* const gs = reinterpret_cast<XG*>(smem_raw + sh.gs_off);
   double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
   const int bd = blockDim.x;
-      // K2: r -= alpha q (and r for the other blocks' extra rows), r.r; then x += alpha p while the sum is on its way
-      {
-        const XA al = (XA)sh.alpha;
-        const XA* const q = sh.q;
-        XA* const r = sh.r;
-        XG* const rg = sh.rg;
-        const int rows = sh.a.rows;
-        double acc = 0.0;
-        const int tid = threadIdx.x;
-        for (int i0 = tid; i0 < rows; i0 += U * bd) {
-          XA qv[U], rv[U];
+  // K2: r -= alpha q (and r for the other blocks' extra rows), r.r; then x += alpha p while the sum is on its way
+  {
+    const XA al = (XA)sh.alpha;
+    const XA* const q = sh.q;
+    XA* const r = sh.r;
+    XG* const rg = sh.rg;
+    const int rows = sh.a.rows;
+    double acc = 0.0;
+    const int tid = threadIdx.x;
+    for (int i0 = tid; i0 < rows; i0 += U * bd) {
+      XA qv[U], rv[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * bd;
-            qv[u] = i < rows ? q[i] : XA(0);
-            rv[u] = i < rows ? r[i] : XA(0);
-          }
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * bd;
-            if (i < rows) {
-              rv[u] = fma(-al, qv[u], rv[u]);
-              r[i] = rv[u];
-              rg[i] = (XG)rv[u];
-              acc = fma((double)rv[u], (double)rv[u], acc);
-            }
-          }
-        }
-        red[tid] = acc;
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * bd;
+        qv[u] = i < rows ? q[i] : XA(0);
+        rv[u] = i < rows ? r[i] : XA(0);
       }
-      __syncthreads();
-      if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<true>(sh.sync, round + 1, red);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * bd;
+        if (i < rows) {
+          rv[u] = fma(-al, qv[u], rv[u]);
+          r[i] = rv[u];
+          rg[i] = (XG)rv[u];
+          acc = fma((double)rv[u], (double)rv[u], acc);
+        }
+      }
+    }
+    red[tid] = acc;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<true>(sh.sync, round + 1, red);
   __syncthreads();  // the update of x would delay the sum: both need the FP64 unit
-      if (threadIdx.x >= 32 || bd == 32) {
-        const int tid = threadIdx.x;
-        const XA al = (XA)sh.alpha;
-        XA* const x = sh.x;
-        const XA* const r = sh.r;
-        const int32_t* const n2o = sh.g.n2o;
-        const int rows = sh.a.rows, pb = sh.a.pb, ts = bd == 32 ? 32 : bd - 32, t0 = bd == 32 ? tid : tid - 32;
-        for (int i0 = t0; i0 < rows; i0 += U * ts) {
-          XA xv[U], pv[U];
-          int m[U];
+  if (threadIdx.x >= 32 || bd == 32) {
+    const int tid = threadIdx.x;
+    const XA al = (XA)sh.alpha;
+    XA* const x = sh.x;
+    const XA* const r = sh.r;
+    const int32_t* const n2o = sh.g.n2o;
+    const int rows = sh.a.rows, pb = sh.a.pb, ts = bd == 32 ? 32 : bd - 32, t0 = bd == 32 ? tid : tid - 32;
+    for (int i0 = t0; i0 < rows; i0 += U * ts) {
+      XA xv[U], pv[U];
+      int m[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * ts;
-            m[u] = i < rows ? checked(n2o[i] - pb, rows, sh.a.status) : 0;
-            xv[u] = i < rows ? x[i] : XA(0);
-            pv[u] = i < rows ? ps[i] : XA(0);
-          }
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * ts;
+        m[u] = i < rows ? checked(n2o[i] - pb, rows, sh.a.status) : 0;
+        xv[u] = i < rows ? x[i] : XA(0);
+        pv[u] = i < rows ? ps[i] : XA(0);
+      }
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * ts;
-            if (i < rows) {
-              x[i] = fma(al, pv[u], xv[u]);
-              gs[checked(i, rows, sh.a.status)] = (XG)r[m[u]];  // K3's slice of r in G's row order
-            }
-          }
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * ts;
+        if (i < rows) {
+          x[i] = fma(al, pv[u], xv[u]);
+          gs[checked(i, rows, sh.a.status)] = (XG)r[m[u]];  // K3's slice of r in G's row order
         }
       }
-      if (threadIdx.x < 32) {
-        double rr;
-        const bool ok = persist::gather_sum<true>(sh.sync, round + 1, &rr);
-        if (threadIdx.x == 0) {
-          if (!ok) {
-            sh.stop = 1;
-          } else {
-            const int it = sh.it + 1;
-            sh.it = it;
-            if (blockIdx.x == 0) sh.hist[it] = rr;
-            sh.rz_old = sh.rz;
-            if (rr <= sh.tol2) sh.converged = sh.stop = 1;
-            else if (!(rr < sh.rr_limit) || it >= sh.max_iter) sh.stop = 1;
-            sh.done = sh.stop;
-          }
-        }
+    }
+  }
+  if (threadIdx.x < 32) {
+    double rr;
+    const bool ok = persist::gather_sum<true>(sh.sync, round + 1, &rr);
+    if (threadIdx.x == 0) {
+      if (!ok) {
+        sh.stop = 1;
+      } else {
+        const int it = sh.it + 1;
+        sh.it = it;
+        if (blockIdx.x == 0) sh.hist[it] = rr;
+        sh.rz_old = sh.rz;
+        if (rr <= sh.tol2) sh.converged = sh.stop = 1;
+        else if (!(rr < sh.rr_limit) || it >= sh.max_iter) sh.stop = 1;
+        sh.done = sh.stop;
       }
-      __syncthreads();
+    }
+  }
+  __syncthreads();
 }
 
 // t.t, published, and K4's slice of t
@@ -561,30 +562,30 @@ __device__ __noinline__ void pcg_step_tt(PcgBlock<VA, XA, VG, XG>& sh, int round
   XG* const gs = reinterpret_cast<XG*>(smem_raw + sh.gs_off);
   double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
   const int bd = blockDim.x;
-      {
-        const XG* const t = sh.t;
-        const int32_t* const n2o = sh.h.n2o;
-        const int rows = sh.a.rows, pb = sh.a.pb;
-        double acc = 0.0;
-        const int tid = threadIdx.x;
-        for (int i0 = tid; i0 < rows; i0 += U * bd) {
-          int m[U];
+  {
+    const XG* const t = sh.t;
+    const int32_t* const n2o = sh.h.n2o;
+    const int rows = sh.a.rows, pb = sh.a.pb;
+    double acc = 0.0;
+    const int tid = threadIdx.x;
+    for (int i0 = tid; i0 < rows; i0 += U * bd) {
+      int m[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) m[u] = i0 + u * bd < rows ? checked(n2o[i0 + u * bd] - pb, rows, sh.a.status) : 0;
+      for (int u = 0; u < U; ++u) m[u] = i0 + u * bd < rows ? checked(n2o[i0 + u * bd] - pb, rows, sh.a.status) : 0;
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * bd;
-            if (i < rows) {
-              const XG v = t[m[u]];
-              gs[checked(i, rows, sh.a.status)] = v;  // K4's slice of t in G^T's row order
-              acc = fma((double)v, (double)v, acc);
-            }
-          }
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * bd;
+        if (i < rows) {
+          const XG v = t[m[u]];
+          gs[checked(i, rows, sh.a.status)] = v;  // K4's slice of t in G^T's row order
+          acc = fma((double)v, (double)v, acc);
         }
-        red[tid] = acc;
       }
-      __syncthreads();
-      if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round + 2, red);
+    }
+    red[tid] = acc;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round + 2, red);
 }
 
 // beta from t.t, then the direction
@@ -594,46 +595,47 @@ __device__ __noinline__ void pcg_step_direction(PcgBlock<VA, XA, VG, XG>& sh, in
   extern __shared__ __align__(16) unsigned char smem_raw[];
   XA* const ps = reinterpret_cast<XA*>(smem_raw);
   const int bd = blockDim.x;
-      if (threadIdx.x < 32) {
-        double tt;
-        const bool ok = persist::gather_sum<false>(sh.sync, round + 2, &tt);
-        if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {
+    double tt;
+    const bool ok = persist::gather_sum<false>(sh.sync, round + 2, &tt);
+    if (threadIdx.x == 0) {
       sh.g.counter = bd >> 5;
-          if (!ok) {
-            sh.stop = 1;
-          } else {
-            sh.rz = tt;
-            sh.beta = tt / sh.rz_old;
-          }
+      if (!ok) {
+        sh.stop = 1;
+      } else {
+        sh.rz = tt;
+        sh.beta = tt / sh.rz_old;
+      }
+    }
+  }
+  __syncthreads();
+  if (sh.stop) return;
+  // K5: p = z + beta p
+  {
+    const XA be = (XA)sh.beta;
+    const XG* const z = sh.z;
+    XA* const p = sh.p;
+    const int rows = sh.a.rows;
+    const int tid = threadIdx.x;
+    for (int i0 = tid; i0 < rows; i0 += U * bd) {
+      XA pv[U], zv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * bd;
+        pv[u] = i < rows ? ps[i] : XA(0);
+        zv[u] = i < rows ? (XA)z[i] : XA(0);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * bd;
+        if (i < rows) {
+          const XA pi = fma(be, pv[u], zv[u]);
+          ps[i] = pi;
+          p[i] = pi;
         }
       }
-      __syncthreads();
-      // K5: p = z + beta p
-      {
-        const XA be = (XA)sh.beta;
-        const XG* const z = sh.z;
-        XA* const p = sh.p;
-        const int rows = sh.a.rows;
-        const int tid = threadIdx.x;
-        for (int i0 = tid; i0 < rows; i0 += U * bd) {
-          XA pv[U], zv[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * bd;
-            pv[u] = i < rows ? ps[i] : XA(0);
-            zv[u] = i < rows ? (XA)z[i] : XA(0);
-          }
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * bd;
-            if (i < rows) {
-              const XA pi = fma(be, pv[u], zv[u]);
-              ps[i] = pi;
-              p[i] = pi;
-            }
-          }
-        }
-      }
+    }
+  }
 }
 
 // MAXT 512 for blocks that are no larger: 128 registers a thread, and with them deeper batches
@@ -693,6 +695,8 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_persist_kernel(core::KArgs a, con
       sh.h.xg = c.t;
       sh.h.out = sh.z;
       sh.h.n2o = h.new_to_old + pb;
+      persist::use_halo(&sh.g, g, g.halo_old, blk, c.h_off);
+      persist::use_halo(&sh.h, h, h.halo_old, blk, c.h_off);
       sh.a.stop = sh.g.stop = sh.h.stop = &sh.stop;
       sh.a.seen = sh.g.seen = sh.h.seen = &sh.seen;
     }
@@ -714,11 +718,13 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_persist_kernel(core::KArgs a, con
     pcg_step_update(sh, round);
     if (sh.stop) break;
     // K3: t = G r, t.t = r.z
+    persist::stage_halo(&sh.g, &sh.sync, 0);
     persist::run_slices<VG, XG, KG, kRunsG>(&sh.g, &sh.sync, 0);  // r of all blocks: ordered by the sum above
     __syncthreads();
     if (threadIdx.x == 0) persist::arrive(sh.sync);  // t: round 2 step + 1
     pcg_step_tt(sh, round);
     // K4: z = G^T t
+    persist::stage_halo(&sh.h, &sh.sync, 2 * step + 1);
     persist::run_slices<VG, XG, KG, kRunsG>(&sh.h, &sh.sync, 2 * step + 1);
     pcg_step_direction(sh, round);
     if (sh.stop) break;
@@ -867,6 +873,11 @@ ehyb_status_t launch_persist(ehyb_precond_t M, const VA* av, const VA* aev, cons
       a.ell_col = P.ell_col_low;
       a.er_scol = P.er_scol_low;
       a.er_scol_old = P.er_scol_old_low;
+      if (P.er_hcol_low) {
+        a.er_hcol = P.er_hcol_low;
+        a.halo_ptr = P.low_halo_ptr;
+        a.halo_old = P.low_halo_old;
+      }
     }
     a.meta_cap = P.max_part_slices;
     return a;
@@ -897,6 +908,12 @@ ehyb_status_t launch_persist(ehyb_precond_t M, const VA* av, const VA* aev, cons
   c.tbl_off[0] = place((size_t)D.max_part_slices * sizeof(core::SliceMeta));
   c.tbl_off[1] = place((size_t)G.max_part_slices * sizeof(core::SliceMeta));
   c.tbl_off[2] = place((size_t)H.max_part_slices * sizeof(core::SliceMeta));
+  {
+    int32_t most = 0;
+    if (g.er_hcol) most = std::max(most, G.max_low_halo);
+    if (h.er_hcol) most = std::max(most, H.max_low_halo);
+    c.h_off = most > 0 ? place((size_t)most * sizeof(float)) : -1;
+  }
   c.x_off = place(va);
   CKP(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
   CKP(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, D.threads, smem));
@@ -950,17 +967,17 @@ ehyb_status_t run_persist(ehyb_precond_t M, PcgWork* w, cudaStream_t s, bool inn
                 : with_g(va, av, aev, c, integral_constant<int, 16>(), t1024);
   };
   if (inner32) {
-    const PcgPersist<float, float> c{w->d32, w->r32, w->p32, w->q32, w->r32, w->t32, w->z32, -1, -1, -1, -1, -1, -1,
+    const PcgPersist<float, float> c{w->d32, w->r32, w->p32, w->q32, w->r32, w->t32, w->z32, -1, -1, -1, -1, -1, -1, -1,
                                      {-1, -1, -1}, kPersistSteps, 1e30, w->st, w->hist, sync};
     return P->lowp == 1 ? fp32(float(), D.ell_val_f32, D.er_sval_f32, c)
                         : fp32(uint16_t(), D.ell_val_bf16, D.er_sval_bf16, c);
   }
   if (M->lowp) {
-    const PcgPersist<double, float> c{w->xp, w->r, w->p, w->q, w->r32, w->t32, w->z32, -1, -1, -1, -1, -1, -1,
+    const PcgPersist<double, float> c{w->xp, w->r, w->p, w->q, w->r32, w->t32, w->z32, -1, -1, -1, -1, -1, -1, -1,
                                       {-1, -1, -1}, kPersistSteps, 1e300, w->st, w->hist, sync};
     return fp64(c);
   }
-  const PcgPersist<double, double> c{w->xp, w->r, w->p, w->q, w->r, w->t, w->z, -1, -1, -1, -1, -1, -1,
+  const PcgPersist<double, double> c{w->xp, w->r, w->p, w->q, w->r, w->t, w->z, -1, -1, -1, -1, -1, -1, -1,
                                      {-1, -1, -1}, kPersistSteps, 1e300, w->st, w->hist, sync};
   return fp64(c);
 }

@@ -191,10 +191,13 @@ struct Product {
   const X* xg;              // x in memory, for the extra rows
   X *out, *mirror;          // out[m] = sum of the row; mirror (optional): the same in memory
   const int32_t* n2o;       // m = n2o[row] - pb (optional: m = row)
+  const uint16_t* er_hcol;  // staged extra rows (else null): 16-bit columns into x staged at `halo`
+  const int32_t* halo;
   const SliceMeta* tbl;     // slice table, or null: the metadata is read from memory
   int32_t *status, *stop, *seen;
   int64_t n_x;
   int32_t xs_off, lim;      // x in shared memory: byte offset of the slice (by local column), its elements
+  int32_t xh_off, nh;       // staged extra rows: byte offset, columns
   int32_t rows, s0, s1, tpr_log2, pb, meta_cap, counter;
 };
 
@@ -213,6 +216,8 @@ __device__ __forceinline__ void init_product(Product<V, X>* pr, const KArgs& a, 
     pr->er_slice_pos = a.er_slice_pos;
     pr->mirror = nullptr;
     pr->n2o = nullptr;
+    pr->er_hcol = nullptr;
+    pr->nh = 0;
     pr->tbl = tbl;
     pr->status = a.status;
     pr->n_x = a.n_x;
@@ -235,6 +240,42 @@ __device__ __forceinline__ void init_product(Product<V, X>* pr, const KArgs& a, 
     m.pad = 0;
     tbl[checked(t, a.meta_cap, a.status)] = m;
   }
+}
+
+// thread 0: pr reads its extra rows from x staged at the partition's columns (plan of D, numbering `cols`), at `off`
+template <typename V, typename X>
+__device__ __forceinline__ void use_halo(Product<V, X>* pr, const KArgs& a, const int32_t* cols, int p, int32_t off) {
+  if (!a.er_hcol || off < 0) return;
+  pr->er_hcol = a.er_hcol;
+  pr->halo = cols + a.halo_ptr[p];
+  pr->nh = (int)(a.halo_ptr[p + 1] - a.halo_ptr[p]);
+  pr->xh_off = off;
+}
+
+// (G and G^T of the preconditioner.  Not the matrix's product: staging waits for the other blocks' direction at once,
+// which the slabs otherwise hide; elasticity 40^3, mixed-precision solve: 2.80 ms gathered, 2.84 with G and G^T
+// staged, 3.05 with A too; 60^3: 5.46, 5.32, 5.31.)
+// stage x at the columns of the product's extra rows (when it does so), by all threads, before run_slices; the
+// caller's next __syncthreads is inside
+template <typename V, typename X>
+__device__ __noinline__ void stage_halo(Product<V, X>* pr, const SyncArgs* sync, int round) {
+  if (!pr->er_hcol) return;  // uniform over the block
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  X* const xh = reinterpret_cast<X*>(smem_raw + pr->xh_off);
+  if (!wait_round(*sync, round, pr->seen)) *pr->stop = 1;
+  const int nh = pr->nh, bd = blockDim.x;
+  for (int j0 = threadIdx.x; j0 < nh; j0 += 4 * bd) {
+    int c[4];
+    X v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) c[u] = j0 + u * bd < nh ? (int)checked((int64_t)pr->halo[j0 + u * bd], pr->n_x, pr->status) : 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = j0 + u * bd < nh ? load_x(pr->xg + c[u]) : X(0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j0 + u * bd < nh) xh[j0 + u * bd] = v[u];
+  }
+  __syncthreads();
 }
 
 // All slices of the block's partition, claimed dynamically from pr->counter (blockDim.x / 32 on entry).  Before its
@@ -286,9 +327,17 @@ __device__ __noinline__ void run_slices(Product<V, X>* pr, const SyncArgs* sync,
         return;
       }
       const int32_t* ecol = pr->er_col;
+      if constexpr (RUNS) {
+        if (const uint16_t* hcol = pr->er_hcol) {
+          const X* const xh = reinterpret_cast<const X*>(smem_raw + pr->xh_off);
+          acc = slab_dot_runs<V, X, 16>(er_val + epos, hcol + epos, lane, we, xh, acc, pr->nh, status);
+          goto summed;
+        }
+      }
       if constexpr (RUNS) acc = er_dot_runs<V, X>(er_val + epos, ecol + epos, lane, we, pr->xg, acc, pr->n_x, status);
       else acc = er_dot<V, X, KB>(er_val + epos + lane, ecol + epos + lane, we, pr->xg, acc, pr->n_x, status);
     }
+  summed:
     const int lg = pr->tpr_log2, tpr = 1 << lg;
     for (int off = tpr >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(FULL, acc, off);
     const int row = (s - s0) * (32 >> lg) + (lane >> lg);

@@ -36,6 +36,19 @@ struct WideLists {
   std::vector<WideSlice> wides;
   int32_t max_items = 0;  // most slices + units of one partition
 };
+// Staged extra rows of the FP32 / BF16 copies (er_layout 0, copies in runs).  A low-precision product is bound by the
+// wavefronts of its gathers of x from memory (up to 32 a slot and warp), not by arithmetic; where a partition's
+// extra rows name the same columns many times over (the three unknowns of a node, the rows around it), the
+// block stages x at those columns once and reads it from shared memory, through 16-bit columns.
+struct LowHalo {
+  std::vector<int64_t> ptr;
+  std::vector<int32_t> col_new, col_old;  // ascending plan numbering; the same in the caller's
+  UninitVec<uint16_t> hcol;               // per slot of er_scol_low: index into the partition's columns
+  int32_t max_cols = 0, max_stage = 0;
+};
+// false (and out empty): a partition's rows and columns exceed max_stage or 2^16, or too little is shared
+bool low_halo(const HostPlan& H, int64_t max_stage, int threads, LowHalo& out);
+
 WideLists wide_lists(int32_t nparts, const std::vector<int32_t>& slice_ptr, const std::vector<int64_t>& slice_pos,
                      const std::vector<int64_t>& er_slice_pos);
 }  // namespace ehyb

@@ -24,7 +24,7 @@ constexpr int run_batch() {
   return (sizeof(V) == 2 && !DOT) ? 32 : 16;
 }
 template <typename V, typename X, bool SCATTER, bool ER_SLICED, bool DOT, bool GATHER = false,
-          int KB = (sizeof(V) == 8 ? kBatch : kLowBatch), bool RUNS = false, bool WIDE = false>
+          int KB = (sizeof(V) == 8 ? kBatch : kLowBatch), bool RUNS = false, bool WIDE = false, bool HER = false>
 __global__ void __launch_bounds__(1024, 1) ehyb_kernel(KArgs a, const V* __restrict__ ell_val,
                                                     const V* __restrict__ er_val, const X* __restrict__ xp,
                                                     X* __restrict__ y) {
@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(1024, 1) ehyb_kernel(KArgs a, const V* __restr
     bs.bar_ready = 0;
     bs.phase = 0;
   }
-  partition_spmv<V, X, SCATTER, ER_SLICED, DOT, GATHER, KB, RUNS, true, true, WIDE>(
+  partition_spmv<V, X, SCATTER, ER_SLICED, DOT, GATHER, KB, RUNS, true, true, WIDE, HER>(
       a, ell_val, er_val, xp, y, blockIdx.x, reinterpret_cast<X*>(smem_raw), bs);
 }
 
@@ -106,7 +106,7 @@ constexpr int kWideBatch = 6;
 // the kernel of one launch form: the plan's batch depth, slot layout of the copies and wide slices choose among
 // its instantiations (`f` is called with the kernel)
 template <typename V, typename X, bool SCATTER, bool ER_SLICED, bool DOT, bool GATHER, typename F>
-static cudaError_t pick_kernel(bool deep, bool runs, bool wide, F&& f) {
+static cudaError_t pick_kernel(bool deep, bool runs, bool wide, bool her, F&& f) {
   constexpr int KB = sizeof(V) == 8 ? kBatch : kLowBatch, R = run_batch<V, DOT>();
   if constexpr (ER_SLICED && sizeof(V) == 8) {
     if (wide) return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, KB, false, true>);
@@ -114,6 +114,7 @@ static cudaError_t pick_kernel(bool deep, bool runs, bool wide, F&& f) {
   } else if constexpr (ER_SLICED) {
     if (wide && runs) return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, 16, true, true>);
     if (wide) return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, KB, false, true>);
+    if (runs && her) return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, R, true, false, true>);
     if (runs) return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, R, true>);
   }
   return f(ehyb_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER, KB>);
@@ -123,16 +124,16 @@ static cudaError_t pick_kernel(bool deep, bool runs, bool wide, F&& f) {
 template <typename V, typename X>
 static cudaError_t set_smem(int bytes) {
   auto set = [&](auto k) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
-  for (int v = 0; v < 8; ++v) {
-    const bool deep = v & 1, runs = v & 2, wide = v & 4;
+  for (int v = 0; v < 16; ++v) {
+    const bool deep = v & 1, runs = v & 2, wide = v & 4, her = v & 8;
     cudaError_t e;
-    if ((e = pick_kernel<V, X, true, true, false, false>(deep, runs, wide, set))) return e;
-    if ((e = pick_kernel<V, X, true, false, false, false>(deep, runs, wide, set))) return e;
-    if ((e = pick_kernel<V, X, false, true, false, false>(deep, runs, wide, set))) return e;
-    if ((e = pick_kernel<V, X, false, false, false, false>(deep, runs, wide, set))) return e;
-    if ((e = pick_kernel<V, X, true, true, false, true>(deep, runs, wide, set))) return e;
-    if ((e = pick_kernel<V, X, true, true, true, true>(deep, runs, wide, set))) return e;
-    if ((e = pick_kernel<V, X, false, true, true, false>(deep, runs, wide, set))) return e;
+    if ((e = pick_kernel<V, X, true, true, false, false>(deep, runs, wide, her, set))) return e;
+    if ((e = pick_kernel<V, X, true, false, false, false>(deep, runs, wide, her, set))) return e;
+    if ((e = pick_kernel<V, X, false, true, false, false>(deep, runs, wide, her, set))) return e;
+    if ((e = pick_kernel<V, X, false, false, false, false>(deep, runs, wide, her, set))) return e;
+    if ((e = pick_kernel<V, X, true, true, false, true>(deep, runs, wide, her, set))) return e;
+    if ((e = pick_kernel<V, X, true, true, true, true>(deep, runs, wide, her, set))) return e;
+    if ((e = pick_kernel<V, X, false, true, true, false>(deep, runs, wide, her, set))) return e;
   }
   return cudaSuccess;
 }
@@ -183,7 +184,14 @@ static void launch_pdl(const DevPlan& P, size_t smem, cudaStream_t s, const KArg
     ar.er_scol = P.er_scol_low;
     ar.er_scol_old = P.er_scol_old_low;
   }
-  pick_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER>(P.kbatch != kWideBatch, runs, ER_SLICED && P.wide_parts > 0,
+  const bool her = runs && P.er_hcol_low != nullptr;
+  if (her) {
+    ar.er_hcol = P.er_hcol_low;
+    ar.halo_ptr = P.low_halo_ptr;
+    ar.halo_new = P.low_halo_new;
+    ar.halo_old = P.low_halo_old;
+  }
+  pick_kernel<V, X, SCATTER, ER_SLICED, DOT, GATHER>(P.kbatch != kWideBatch, runs, ER_SLICED && P.wide_parts > 0, her,
                                                      [&](auto k) { return cudaLaunchKernelEx(&cfg, k, ar, ev, erv, xp, y); });
 }
 
@@ -227,8 +235,9 @@ static void launch_typed(const DevPlan& P, const V* ev, const V* erv_csr, const 
   KArgs a = make_kargs(P);
   a.smem_elems = (int64_t)(smem / sizeof(X));
   if (P.small_threads > 0 && !dot && !skip && scatter != 1 && !P.inject_wait_fault) {
-    if (scatter == 2) launch_small<V, X, true>(P, smem, s, a, ev, erv_sl, xp, y);
-    else launch_small<V, X, false>(P, smem, s, a, ev, erv_sl, xp, y);
+    const size_t sm = ehyb_smem_bytes(P, (int)sizeof(X));
+    if (scatter == 2) launch_small<V, X, true>(P, sm, s, a, ev, erv_sl, xp, y);
+    else launch_small<V, X, false>(P, sm, s, a, ev, erv_sl, xp, y);
     return;
   }
   // the partition's slice table after the staged x, when both fit the block's shared memory
@@ -273,7 +282,9 @@ cudaError_t launch_ehyb_f64(const DevPlan& P, const double* xp, double* y, int s
 cudaError_t launch_ehyb_lowp(const DevPlan& P, int lowp, const float* xp, float* y, int scatter, cudaStream_t s,
                              const DotOut* dot, const int32_t* skip) {
   if (P.nparts == 0) return cudaSuccess;
-  const size_t smem = ehyb_smem_bytes(P, 4);
+  size_t smem = ehyb_smem_bytes(P, 4);
+  if (P.er_hcol_low && P.lowp_group == 4)  // the staged extra rows' columns after the slice
+    smem = ((size_t)(P.low_stage_rows + 4) * sizeof(float) + 15) & ~(size_t)15;
   if (lowp == 1)
     launch_typed<float, float>(P, P.ell_val_f32, P.er_val_f32, P.er_sval_f32, xp, y, scatter, smem, s, dot, skip);
   else
