@@ -151,7 +151,6 @@ ehyb_status_t device_query(int* dev, int* sms, int* smem_optin) {
 }
 ehyb_status_t device_alloc(void** p, size_t bytes) { return dev_alloc(p, bytes); }
 
-// device view of a plan for entry points defined in other translation units
 WideLists wide_lists(int32_t nparts, const std::vector<int32_t>& slice_ptr, const std::vector<int64_t>& slice_pos,
                      const std::vector<int64_t>& er_slice_pos) {
   WideLists L;
@@ -191,11 +190,12 @@ WideLists wide_lists(int32_t nparts, const std::vector<int32_t>& slice_ptr, cons
 }
 
 // Slots per staged column from which staging pays, measured (FP32 / BF16 product, gathers -> staged): elasticity 45^3,
-// 15.7 slots a column, 29.2 -> 26.6 / 23.1 -> 15.9 us; scalar hexahedra 60^3, about 6.5, 10.5 -> 11.0; tets, 4.2, even.
+// 15.7 slots a column, 29.2 -> 26.6 / 23.1 -> 20.2 us; scalar hexahedra 60^3, about 6.5, 10.5 -> 11.0; tets, 4.2, even.
 static constexpr int64_t kSlotsPerHaloColumn = 10;
 
 bool low_halo(const HostPlan& H, int64_t max_stage, int threads, LowHalo& out) {
-  const int T = planner_threads(threads);
+  const int T = std::min(planner_threads(threads), 16);  // each holds n integers
+  std::atomic<bool> oom{false};                           // a worker must not throw: that would end the process
   const int64_t slots = (int64_t)H.er_scol_low.size();
   out = LowHalo();
   if (slots == 0 || (int64_t)H.ell_col_low.size() > 10 * slots) return false;  // extra rows below about a tenth
@@ -204,7 +204,17 @@ bool low_halo(const HostPlan& H, int64_t max_stage, int threads, LowHalo& out) {
     k0 = H.er_slice_pos[(size_t)H.slice_ptr[(size_t)p]];
     k1 = H.er_slice_pos[(size_t)H.slice_ptr[(size_t)p + 1]];
   };
-  parallel_for(H.nparts, T, [&](int64_t lo, int64_t hi) {
+  auto each = [&](auto f) {
+    parallel_for(H.nparts, T, [&](int64_t lo, int64_t hi) {
+      try {
+        f(lo, hi);
+      } catch (const std::bad_alloc&) {
+        oom = true;
+      }
+    }, 1);
+    if (oom) throw std::bad_alloc();
+  };
+  each([&](int64_t lo, int64_t hi) {
     std::vector<int32_t> seen((size_t)H.n, -1);
     for (int64_t p = lo; p < hi; ++p) {
       int64_t k0, k1;
@@ -219,7 +229,7 @@ bool low_halo(const HostPlan& H, int64_t max_stage, int threads, LowHalo& out) {
       }
       std::sort(c.begin(), c.end());
     }
-  }, 1);
+  });
   out.ptr.assign((size_t)H.nparts + 1, 0);
   for (int32_t p = 0; p < H.nparts; ++p) {
     const int64_t m = (int64_t)cols[(size_t)p].size();
@@ -236,7 +246,7 @@ bool low_halo(const HostPlan& H, int64_t max_stage, int threads, LowHalo& out) {
   out.col_new.resize((size_t)total);
   out.col_old.resize((size_t)total);
   out.hcol.resize((size_t)slots);
-  parallel_for(H.nparts, T, [&](int64_t lo, int64_t hi) {
+  each([&](int64_t lo, int64_t hi) {
     std::vector<int32_t> rank((size_t)H.n, 0);
     for (int64_t p = lo; p < hi; ++p) {
       int64_t k0, k1;
@@ -250,10 +260,11 @@ bool low_halo(const HostPlan& H, int64_t max_stage, int threads, LowHalo& out) {
       }
       for (int64_t k = k0; k < k1; ++k) out.hcol[(size_t)k] = (uint16_t)rank[(size_t)H.er_scol_low[(size_t)k]];
     }
-  }, 1);
+  });
   return true;
 }
 
+// device view of a plan for entry points defined in other translation units
 const DevPlan* plan_device_view(ehyb_plan_t plan, int* device) {
   if (!plan || plan->host_only) return nullptr;
   if (device) *device = plan->device;

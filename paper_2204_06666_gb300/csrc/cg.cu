@@ -417,7 +417,7 @@ __device__ __noinline__ void cg_step_pq(CgBlock<V, X>& sh, int round) {
     const bool ok = persist::gather_sum<false>(sh.sync, round, &pq);
     if (threadIdx.x == 0) {
       sh.prod.counter = bd >> 5;  // for the next product
-    const double rr = sh.rr, alpha = ok && pq > 0.0 ? rr / pq : 0.0;
+      const double rr = sh.rr, alpha = ok && pq > 0.0 ? rr / pq : 0.0;
       if (!ok) {
         sh.stop = 1;
       } else if (!(alpha > 0.0) && rr > 0.0) {  // A is not positive definite along p: nothing is updated
