@@ -783,7 +783,7 @@ def _event_time(fn, reps, stream):
 
 def run_batch(args):
     """64 generated FEM matrices (n log-uniform in [5k, 300k], four element kinds): one persistent batch
-    launch (graph replay) vs the same 64 SpMVs issued one by one."""
+    launch vs the same 64 SpMVs issued one by one."""
     import torch
     import gen
     import paper_2204_06666_gb300 as eh
@@ -806,7 +806,7 @@ def run_batch(args):
     t_seq = _event_time(one_by_one, max(3, args.steps // 4), stream)
     nnz = sum(A.nnz for A in mats)
     byts = sum(P.info()["bytes_effective"] for P in plans)
-    line = {"metric": "batched EHYB SpMV GFLOP/s (64 FEM matrices, one persistent graph-captured launch)",
+    line = {"metric": "batched EHYB SpMV GFLOP/s (64 FEM matrices, one persistent launch)",
             "unit": "GFLOP/s", "value": 2 * nnz / t_batch / 1e6, "higher_is_better": True, "n_gpus": 1,
             "steps": args.steps, "warmup": args.warmup, "dtype": "f64", "data": "synthetic",
             "config": {"workload": f"fem_batch_{args.batch_count}", "matrices": len(mats),

@@ -421,8 +421,10 @@ ehyb_status_t ehyb_precond_destroy(ehyb_precond_t M); /* NULL is fine; synchroni
  * Preconditioned CG on `plan` with M (built for this plan): x (device, caller's numbering) holds x0 on
  * entry and the solution on return; b likewise.  Stops when the recursive residual ||r_k|| <= rtol ||b||
  * or after max_iter iterations; info->relres is the true FP64 residual ||b - A x|| / ||b|| of the returned
- * x.  Five launches per iteration (A p with p.q, the update, G r with r.z, G^T t, the direction), replayed
- * from CUDA graphs of 16 iterations; alpha and beta stay on the device.  Synchronous.
+ * x.  The iterations (A p with p.q, the update, G r with r.z, G^T t, the direction) run inside one cooperative
+ * kernel when the plan's partitions are all resident at once (sliced ER layout, no very long rows, at most one
+ * partition per SM), else as five launches each, replayed from CUDA graphs of 16 iterations; alpha and beta
+ * stay on the device.  Synchronous.
  * EHYB_ERR_NOT_CONVERGED at the iteration limit or when p.A p <= 0; EHYB_ERR_INVALID_ARG when M belongs
  * to another plan.
  */

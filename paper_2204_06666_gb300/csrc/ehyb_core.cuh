@@ -19,12 +19,16 @@
 //        - sliced (er_layout 0, default): the ER entries of the slice's own rows are stored in
 //          the same lane -> row arrangement right behind it (the paper stores its ER part as
 //          stride-32 slices too, Alg. 2); the warp continues with them, gathering x from global
-//          memory, and writes y once -- no block barrier, no read-modify-write, no FP64 shuffle;
+//          memory, and writes y once -- no block barrier, no read-modify-write, no FP64 shuffle.
+//          FP32 / BF16 products whose extra rows name each column many times (low_halo in
+//          plan_internal.h) stage x at those columns behind the slice and run them like the slab;
 //        - CSR lines (er_layout 1): after a block barrier, er_tpr lanes per ER line with a
 //          shuffle reduction, y[yIdxER] += sum;
 //        - halo (er_layout 2): step 1 also stages x at the partition's halo (the distinct columns
 //          of its ER entries outside it) behind the slice, and a row's ER entries follow its own
 //          in the slab slots with 16-bit columns into [slice | halo]: step 3 covers them.
+//   Slices with very long rows are summed in chunks (WIDE below); plans with one slice per warp take a
+//   kernel of their own (small_partition_spmv).
 //   In every layout the rows a block updates are its own, so the paper's second pass over ER
 //   slices from a global counter is not needed: no atomics on y, deterministic results.
 #pragma once
