@@ -38,7 +38,11 @@ struct BatchPlan {
 // kStageCost slots a row, from L2).  With whole partitions as units, a batch with fewer large partitions than
 // resident blocks took as long as its largest one: 24 matrices of 5k to 100k rows on 304 blocks, about 50 partitions
 // of up to 640k entries, 272 us; 91 us in shares (launched directly under the previous grid's tail).  Plans with wide slices are not split (one block combines their partial sums).
+// Nothing is split where the largest partition is less than kWhole of an SM's share: then the order alone balances the
+// units, and the extra staging would only cost (64 matrices of 5k to 300k rows, 0.52 of a share: whole 315 us, in
+// shares 337; the first 56 of them, 0.67 of a share: 280 and 263).
 constexpr double kShare = 2.0;
+constexpr double kWhole = 0.6;
 constexpr int kStageCost = 2;
 
 constexpr int kMaxThreads = 1024;  // block size: 512 when two or more blocks fit an SM, else 1024
@@ -191,11 +195,16 @@ extern "C" ehyb_status_t ehyb_batch_create(int32_t count, const ehyb_plan_t* pla
   std::vector<int64_t> cost;
   {
     int64_t total = 0;
-    for (const Tile& t : parts) total += t.slots;
+    int64_t largest = 0;
+    for (const Tile& t : parts) {
+      total += t.slots;
+      largest = std::max(largest, t.slots);
+    }
+    const bool whole = (double)largest * sms < kWhole * (double)total;
     const double target = std::max(1.0, (double)total / ((double)b->grid * kShare));
     for (const Tile& t : parts) {
       const int64_t most = std::max<int64_t>(1, t.slices / (b->threads / 32));
-      const int nsub = t.wide ? 1 : (int)std::min<int64_t>(most, (int64_t)((double)t.slots / target + 0.999));
+      const int nsub = t.wide || whole ? 1 : (int)std::min<int64_t>(most, (int64_t)((double)t.slots / target + 0.999));
       for (int k = 0; k < std::max(nsub, 1); ++k) {
         tiles.push_back(make_int4(t.plan, t.part, k, std::max(nsub, 1)));
         cost.push_back(t.slots / std::max(nsub, 1) + kStageCost * (int64_t)t.rows);

@@ -858,8 +858,8 @@ ehyb_status_t enqueue_chunk32(ehyb_precond_t M, PcgWork* w, cudaStream_t s) {
 }
 
 // One persistent launch of at most kPersistSteps iterations; *ran = false (and nothing launched) where the separate
-// launches are needed: more partitions than SMs, a wide slice, copies not in runs of four, vectors that do not
-// fit a block's shared memory, the staging-fault test hook.
+// launches are needed: more partitions than SMs, a wide slice, copies not in runs of four, more shared
+// memory than persist::shared_budget grants, the staging-fault test hook.
 constexpr int kPersistSteps = 2000;  // bounds one launch to a fraction of a second
 
 template <typename VA, typename XA, int KA, typename VG, typename XG, int MAXT>
@@ -886,17 +886,18 @@ ehyb_status_t launch_persist(ehyb_precond_t M, const VA* av, const VA* aev, cons
   int optin = 0, resident = 0, sms = 0;
   CKP(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, M->plan->device));
   CKP(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, M->plan->device));
-  const size_t budget = (size_t)optin - 1024;
   auto al = [](size_t b) { return (b + 15) & ~(size_t)15; };
   size_t smem = ehyb_smem_bytes(D, (int)sizeof(XA));
   a.smem_elems = (int64_t)(smem / sizeof(XA));
+  const size_t va = (size_t)D.max_part_rows * sizeof(XA), vg = (size_t)D.max_part_rows * sizeof(XG);
+  const size_t budget =
+      std::min((size_t)optin - 1024, persist::shared_budget(smem + al(vg) + (size_t)D.threads * sizeof(double)));
   auto place = [&](size_t bytes) -> int32_t {
     if (smem + al(bytes) > budget) return -1;
     const size_t o = smem;
     smem += al(bytes);
     return (int32_t)o;
   };
-  const size_t va = (size_t)D.max_part_rows * sizeof(XA), vg = (size_t)D.max_part_rows * sizeof(XG);
   *ran = false;
   c.gs_off = place(vg);
   c.red_off = place((size_t)D.threads * sizeof(double));

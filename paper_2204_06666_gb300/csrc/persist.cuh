@@ -8,9 +8,11 @@
 // its partition's slices of the vectors in shared memory from one iteration to the next, as many of them as fit,
 // and the iteration's inner products double as the barriers that the data dependences need.  Scalars (a division
 // is a dozen dependent FP64 operations, and FP64 operations of 32 warps queue for one unit) are one thread's work.
-// 100 CG iterations with the solve's set-up, separate launches -> persistent: tet 80^3 4.40 -> 3.25 ms (41 -> 30 us an
-// iteration), tet 30^3 2.14 -> 1.28, tet 126^3 9.70 -> 8.87, elasticity 48^3 8.2 -> 7.8; 30^3 (81k rows, bound by 17
-// slices on four quarters of an SM) 3.97 both.  A third of the tet 80^3 iteration is still outside the product: FP64
+// Whole solves of (A + 0.1 mean diagonal) x = b to 1e-10, separate launches -> persistent, FP64 CG (40 to 66
+// iterations): tet 20^3 0.96 -> 0.61 ms, 40^3 1.11 -> 0.76, 80^3 2.06 -> 1.56, 126^3 4.55 -> 4.19, elasticity 24^3 1.86 ->
+// 1.34, 48^3 5.19 -> 4.90, 70^3 10.87 -> 10.75; elasticity 30^3 (81k rows, bound by 17 slices on four quarters of an SM)
+// 2.54 both.  Mixed-precision PCG: tet 80^3 2.13 -> 1.53, 126^3 3.92 -> 3.72, elasticity 40^3 3.56 -> 2.90, 70^3 8.33 ->
+// 7.70; FP64 PCG: tet 80^3 1.76 -> 1.25, elasticity 70^3 11.69 -> 11.45.  A third of the tet 80^3 iteration is still outside the product: FP64
 // vector arithmetic (five FMAs a row, 4.4 us at the pipe's rate) and the three meetings.
 #pragma once
 #include "ehyb_core.cuh"
@@ -43,6 +45,19 @@ struct SyncArgs {
   int32_t* done;              // set to kAborted with it, so that the host stops launching
   uint64_t limit_ns;
 };
+
+// Shared memory of a persistent block, out of the SM's 256 KB that the rest of L1 shares: the least of the sizes the
+// hardware can set aside that holds `must` bytes (what the kernel cannot do without), less what the system and the
+// kernel's own variables take; the vectors beyond it go there only as far as they fit.  The extra rows gather freshly
+// written vectors through L1, so a vector kept in shared memory at L1's cost loses more than it saves: at elasticity
+// 64^3 (41 KB a vector) the FP64 PCG took 23.1 ms a solve with five vectors in shared memory (215 KB), 9.5 with two
+// (separate launches 9.8); scalar hexahedra 80^3 with BF16 G 3.0 and 1.9 ms (2.4).  0: more than 196 KB, where
+// the separate launches are the faster form (tet 126^3, FP64 G, two vectors of 105 KB: 4.9 ms against 3.9).
+inline size_t shared_budget(size_t must) {
+  for (size_t kb : {100, 132, 164, 196})
+    if (must + 3072 <= kb * 1024) return kb * 1024 - 3072;
+  return 0;
+}
 
 __device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 

@@ -91,3 +91,29 @@ def test_pcg_forms(name):
                     xs.append(x.cpu().numpy())
                 assert len(xs) < 2 or np.array_equal(xs[0], xs[1])
         assert P.check() == 0
+
+
+@pytest.mark.parametrize("rows", (3900, 4100, 6000, 6300, 9500, 9800, 11900, 12300))
+def test_solvers_at_each_size_of_shared_memory(rows):
+    """Two FP64 vectors and the block sum on either side of 100, 132, 164 and 196 KB: what else stays in shared memory, and
+    whether the iterations run persistently at all, changes there; the residual history does not."""
+    import paper_2204_06666_gb300 as eh
+    A = gen.tet_lap3d(N=33)
+    b = torch.from_numpy(oracle.spmv(A, gen.uniform(A.n, 3))).cuda()
+    ref = oracle.cg(A, b.cpu().numpy())
+    P = eh.Plan(A, lowp=1, slice_rows=rows, block_threads=1024)
+    x = torch.zeros_like(b)
+    st, info = P.cg(b, x, rtol=1e-10)
+    assert st == 0 and abs(info["iterations"] - ref[2]) <= 1
+    _check(A, b, x, info)
+    for low in (0, 2):
+        M = eh.Fsai(P, A, lowp=low)
+        x = torch.zeros_like(b)
+        st, info = P.pcg(M, b, x, rtol=1e-10)
+        assert st == 0, (low, info)
+        _check(A, b, x, info)
+    x = torch.zeros_like(b)
+    st, info = P.pcg_refined(M, b, x, rtol=1e-9)
+    assert st == 0, info
+    _check(A, b, x, info, 1e-9)
+    assert P.check() == 0
