@@ -739,8 +739,8 @@ ehyb_status_t run_chunk(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s) {
 
 // One persistent launch of at most kPersistSteps iterations; *ran = false (and nothing launched) for a plan that
 // needs the separate launches: more partitions than SMs (a block owns one partition, all blocks resident), a
-// wide slice (its sums go through the plan's workspace), more shared memory than persist::shared_budget grants, BF16
-// values whose vectors do not fit, the staging-fault test hook.
+// wide slice (its sums go through the plan's workspace), more shared memory than persist::shared_budget grants, FP32
+// vectors of more than persist::kMaxRows32 rows a partition, the staging-fault test hook.
 constexpr int kPersistSteps = 2000;  // bounds one launch to a fraction of a second
 
 template <typename V, typename X, int KB, bool RUNS, int MAXT>
@@ -775,9 +775,6 @@ ehyb_status_t launch_persist(ehyb_plan_t P, const V* ev, const V* erv, CgPersist
   c.q_off = place(vec);
   c.r_off = place(vec);
   c.x_off = place(vec);
-  // BF16 values leave little but the vectors: with none of q, r and x in shared memory the separate launches' passes
-  // over them are faster (tet 126^3, refine 4: 6.24 ms a solve against 6.41; FP32 values 5.18 against 5.10)
-  if (sizeof(V) == 2 && c.q_off < 0) return EHYB_OK;
   CKC(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
   CKC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, D.threads, smem));
   *ran = D.nparts <= sms * resident && D.nparts <= persist::kMaxGrid;
@@ -800,6 +797,7 @@ ehyb_status_t run_persist(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s, bo
     return D.kbatch == 6 ? launch_persist<double, double, 6, false, 1024>(P, D.ell_val, D.er_sval, c, s, ran)
                          : launch_persist<double, double, 8, false, 1024>(P, D.ell_val, D.er_sval, c, s, ran);
   }
+  if (D.max_part_rows > persist::kMaxRows32) return EHYB_OK;
   const CgPersist<float> c{w->d32, w->r32, w->p32, w->q32, -1, -1, -1, -1, -1, kPersistSteps, w->st, w->hist, sync};
   const bool runs = D.lowp_group == 4, half = D.threads <= 512;
   if (lowp == 1)

@@ -859,7 +859,7 @@ ehyb_status_t enqueue_chunk32(ehyb_precond_t M, PcgWork* w, cudaStream_t s) {
 
 // One persistent launch of at most kPersistSteps iterations; *ran = false (and nothing launched) where the separate
 // launches are needed: more partitions than SMs, a wide slice, copies not in runs of four, more shared
-// memory than persist::shared_budget grants, the staging-fault test hook.
+// memory than persist::shared_budget grants, FP32 vectors of more than persist::kMaxRows32 rows a partition, the staging-fault test hook.
 constexpr int kPersistSteps = 2000;  // bounds one launch to a fraction of a second
 
 template <typename VA, typename XA, int KA, typename VG, typename XG, int MAXT>
@@ -937,7 +937,7 @@ ehyb_status_t run_persist(ehyb_precond_t M, PcgWork* w, cudaStream_t s, bool inn
   // the three plans own the same rows block by block
   if (M->g->host.part_ptr != P->host.part_ptr || M->gt->host.part_ptr != P->host.part_ptr) return EHYB_OK;
   if (M->lowp && (G.lowp_group != 4 || H.lowp_group != 4)) return EHYB_OK;
-  if (inner32 && D.lowp_group != 4) return EHYB_OK;
+  if (inner32 && (D.lowp_group != 4 || D.max_part_rows > persist::kMaxRows32)) return EHYB_OK;
   const persist::SyncArgs sync{w->meeting, D.status, &w->st->done, std::max(D.wait_timeout_ns, persist::kMinLimitNs)};
   const bool half = D.threads <= 512;
   auto with_g = [&](auto va, const auto* av, const auto* aev, auto c, auto ka, auto mt) -> ehyb_status_t {

@@ -11,8 +11,7 @@
 // Whole solves of (A + 0.1 mean diagonal) x = b to 1e-10, separate launches -> persistent, FP64 CG (40 to 66
 // iterations): tet 20^3 0.96 -> 0.61 ms, 40^3 1.11 -> 0.76, 80^3 2.06 -> 1.56, 126^3 4.55 -> 4.19, elasticity 24^3 1.86 ->
 // 1.34, 48^3 5.19 -> 4.90, 70^3 10.87 -> 10.75; elasticity 30^3 (81k rows, bound by 17 slices on four quarters of an SM)
-// 2.54 both.  Mixed-precision PCG: tet 80^3 2.13 -> 1.53, 126^3 3.92 -> 3.72, elasticity 40^3 3.56 -> 2.90, 70^3 8.33 ->
-// 7.70; FP64 PCG: tet 80^3 1.76 -> 1.25, elasticity 70^3 11.69 -> 11.45.  A third of the tet 80^3 iteration is still outside the product: FP64
+// 2.54 both.  Mixed-precision PCG: tet 80^3 2.13 -> 1.53, elasticity 40^3 3.56 -> 2.90, 70^3 8.33 -> 7.70; FP64 PCG: tet 80^3 1.76 -> 1.25, elasticity 70^3 11.69 -> 11.45.  A third of the tet 80^3 iteration is still outside the product: FP64
 // vector arithmetic (five FMAs a row, 4.4 us at the pipe's rate) and the three meetings.
 #pragma once
 #include "ehyb_core.cuh"
@@ -58,6 +57,12 @@ inline size_t shared_budget(size_t must) {
     if (must + 3072 <= kb * 1024) return kb * 1024 - 3072;
   return 0;
 }
+
+// Rows of a partition up to which FP32 iterations run persistently.  Beyond, the FP32 products are short of bytes rather
+// than of launches, and the vectors' passes of the separate launches are the faster ones (us an iteration, separate ->
+// persistent: tet 102^3, 6,982 rows, CG 42.8 -> 39.5, mixed PCG 85.4 -> 79.9; tet 114^3, 9,747 rows, 50.8 -> 52.1 and
+// 99.9 -> 106.8; tet 126^3 61.0 -> 65.3 and 127.1 -> 139.7; FP64 iterations gain there: CG 93.6 -> 85.4, PCG 203.7 -> 202.3).
+constexpr int kMaxRows32 = 8192;
 
 __device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 

@@ -117,3 +117,23 @@ def test_solvers_at_each_size_of_shared_memory(rows):
     assert st == 0, info
     _check(A, b, x, info, 1e-9)
     assert P.check() == 0
+
+
+@pytest.mark.parametrize("rows", (8192, 8193))
+def test_fp32_iterations_at_the_row_limit(rows):
+    """FP32 vectors run persistently up to 8,192 rows a partition: both forms reach the tolerance."""
+    import paper_2204_06666_gb300 as eh
+    A = gen.tet_lap3d(N=26)
+    b = torch.from_numpy(oracle.spmv(A, gen.uniform(A.n, 3))).cuda()
+    for low in (1, 2):
+        P = eh.Plan(A, lowp=low, slice_rows=rows)
+        M = eh.Fsai(P, A, lowp=low)
+        x = torch.zeros_like(b)
+        st, info = P.cg(b, x, rtol=1e-10, refine=2 + low)
+        assert st == 0, info
+        _check(A, b, x, info)
+        if low == 1:
+            x = torch.zeros_like(b)
+            st, info = P.pcg_refined(M, b, x, rtol=1e-9)
+            assert st == 0, info
+            _check(A, b, x, info, 1e-9)
