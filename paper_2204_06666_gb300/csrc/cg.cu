@@ -34,8 +34,7 @@ namespace ehyb {
 namespace {
 
 using core::FULL;
-constexpr int kVB = 608;  // vector-kernel blocks (4 per SM; 8 per SM measured slower)
-constexpr int kVT = 256;
+constexpr int kVB = persist::kVecBlocks, kVT = persist::kVecThreads;  // vector kernels
 constexpr int kChunk = 16;
 constexpr double kFcgInnerRtol = 0.1;  // default inner tolerance of the flexible CG's preconditioning solve
 
@@ -354,11 +353,12 @@ __global__ void fcg_update_kernel(int64_t n, double alpha, const double* __restr
 }
 
 // ---- persistent iterations: up to max_steps CG iterations (K1, K2, K3 of the launches above, the same arithmetic
-// per element) in one cooperative launch, block p owning partition p's rows.  p stays in shared memory (it is the
-// product's slice of x) and is mirrored to memory for the other blocks' extra rows; q, r and x stay there too as
-// far as they fit (in that order: q is written and read twice an iteration, r read and written, x likewise but by
-// one pass).  The blocks meet three times an iteration: for p.q, for r.r (x is updated while the sum travels)
-// and for the new p, which a warp waits for only when it comes to its first extra row.
+// per element and the same order of every sum) in one cooperative launch, block p owning partition p's rows.  p stays
+// in shared memory (it is the product's slice of x) and is mirrored to memory for the other blocks' extra rows; q, r
+// and x stay there too as far as they fit (in that order: q is written and read twice an iteration, r read and
+// written, x likewise but by one pass).  The blocks meet four times an iteration: for p.q, for the new r, which is
+// mirrored to memory too since r.r is summed in the order of K2's threads (x is updated while r travels), for r.r and
+// for the new p, which a warp waits for only when it comes to its first extra row.
 template <typename X>
 struct CgPersist {
   X *x, *r, *p, *q;                 // global vectors, plan numbering
@@ -377,73 +377,51 @@ struct CgBlock {
   int it, max_iter, converged, breakdown, done, stop, seen, nh;
   const int32_t* halo;
   X *q, *r, *x, *p;  // p: the block's rows of p in memory
+  X* rm;             // r's mirror in memory (null: r lies there)
+  const X* r_all;    // r of all blocks in memory
+  int n;
   persist::Product<V, X> prod;
   double* hist;
   int32_t red_off;
+  double sums[32];
   persist::SyncArgs sync;
 };
 
 // p.q and alpha
 template <typename V, typename X>
 __device__ __noinline__ void cg_step_pq(CgBlock<V, X>& sh, int round) {
-  constexpr int U = 4;  // elements a thread has in flight
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  X* const ps = reinterpret_cast<X*>(smem_raw);
-  const int bd = blockDim.x;
+  const X* const ps = reinterpret_cast<const X*>(smem_raw);
+  const int warps = blockDim.x >> 5;
   double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
   {
     const X* const q = sh.q;
-    const int rows = sh.prod.rows;
-    double acc = 0.0;
-    const int tid = threadIdx.x;
-    for (int i0 = tid; i0 < rows; i0 += U * bd) {
-      X qv[U], pv[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int i = i0 + u * bd;
-        qv[u] = i < rows ? q[i] : X(0);
-        pv[u] = i < rows ? ps[i] : X(0);
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (i0 + u * bd < rows) acc = fma((double)qv[u], (double)pv[u], acc);
-    }
-    red[tid] = acc;
+    persist::part_terms(sh.prod, warps, red, [&](int i) { return make_double2((double)q[i], (double)ps[i]); });
   }
   __syncthreads();
-  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round, red);
-  if (threadIdx.x < 32) {
-    double pq;
-    const bool ok = persist::gather_sum<false>(sh.sync, round, &pq);
-    if (threadIdx.x == 0) {
-      sh.prod.counter = bd >> 5;  // for the next product
-      const double rr = sh.rr, alpha = ok && pq > 0.0 ? rr / pq : 0.0;
-      if (!ok) {
-        sh.stop = 1;
-      } else if (!(alpha > 0.0) && rr > 0.0) {  // A is not positive definite along p: nothing is updated
-        sh.breakdown = sh.done = sh.stop = 1;
-      }
-      sh.alpha = alpha;
-    }
+  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_part(sh.sync, round, 0, red, warps, sh.sums);
+  double pq;
+  const bool ok = persist::gather_sum(sh.sync, round, sh.sync.m->part[0], gridDim.x, red, &sh.stop, &pq);
+  if (threadIdx.x == 0) {
+    sh.prod.counter = warps;  // for the next product
+    const double rr = sh.rr, alpha = ok && pq > 0.0 ? rr / pq : 0.0;
+    // A is not positive definite along p: nothing is updated
+    if (ok && !(alpha > 0.0) && rr > 0.0) sh.breakdown = sh.done = sh.stop = 1;
+    sh.alpha = alpha;
   }
   __syncthreads();
 }
 
 template <typename V, typename X>
-__device__ __noinline__ void cg_step_update(CgBlock<V, X>& sh, int round) {
+__device__ __noinline__ void cg_step_update(CgBlock<V, X>& sh, int round, int r_round) {
   constexpr int U = 4;  // elements a thread has in flight
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  X* const ps = reinterpret_cast<X*>(smem_raw);
-  const int bd = blockDim.x;
-  double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
-  // r -= alpha q, r.r; then x += alpha p while the sum is on its way
-  {
-    const X al = (X)sh.alpha;
+  const X* const ps = reinterpret_cast<const X*>(smem_raw);
+  const int bd = blockDim.x, tid = threadIdx.x, rows = sh.prod.rows;
+  const X al = (X)sh.alpha;
+  {  // r -= alpha q
     const X* const q = sh.q;
-    X* const r = sh.r;
-    const int rows = sh.prod.rows;
-    double acc = 0.0;
-    const int tid = threadIdx.x;
+    X *const r = sh.r, *const rm = sh.rm;
     for (int i0 = tid; i0 < rows; i0 += U * bd) {
       X qv[U], rv[U];
 #pragma unroll
@@ -453,54 +431,50 @@ __device__ __noinline__ void cg_step_update(CgBlock<V, X>& sh, int round) {
         rv[u] = i < rows ? r[i] : X(0);
       }
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (i0 + u * bd < rows) {
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * bd;
+        if (i < rows) {
           rv[u] = fma(-al, qv[u], rv[u]);
-          r[i0 + u * bd] = rv[u];
-          acc = fma((double)rv[u], (double)rv[u], acc);
+          r[i] = rv[u];
+          if (rm) rm[i] = rv[u];
         }
+      }
     }
-    red[tid] = acc;
   }
   __syncthreads();
-  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round + 1, red);
-  __syncthreads();  // the update of x would delay the sum: both need the FP64 unit
-  if (threadIdx.x >= 32 || bd == 32) {
-    const int tid = threadIdx.x;
-    const X al = (X)sh.alpha;
+  if (tid == 0) persist::arrive(sh.sync);
+  {  // x += alpha p while r is on its way
     X* const x = sh.x;
-    const int rows = sh.prod.rows, ts = bd == 32 ? 32 : bd - 32;
-    for (int i0 = bd == 32 ? tid : tid - 32; i0 < rows; i0 += U * ts) {
+    for (int i0 = tid; i0 < rows; i0 += U * bd) {
       X xv[U], pv[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int i = i0 + u * ts;
+        const int i = i0 + u * bd;
         xv[u] = i < rows ? x[i] : X(0);
         pv[u] = i < rows ? ps[i] : X(0);
       }
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (i0 + u * ts < rows) x[i0 + u * ts] = fma(al, pv[u], xv[u]);
+        if (i0 + u * bd < rows) x[i0 + u * bd] = fma(al, pv[u], xv[u]);
     }
   }
-  if (threadIdx.x < 32) {
-    double rrn;
-    const bool ok = persist::gather_sum<false>(sh.sync, round + 1, &rrn);
-    if (threadIdx.x == 0) {
-      if (!ok) {
-        sh.stop = 1;
-      } else {
-        const int it = sh.it + 1;
-        if (blockIdx.x == 0) sh.hist[it] = rrn;
-        sh.beta = rrn / sh.rr;
-        sh.rr = rrn;
-        sh.it = it;
-        if (rrn <= sh.tol2) sh.converged = sh.stop = 1;
-        else if (!(rrn <= sh.grow_limit)) sh.breakdown = sh.stop = 1;  // non-finite or diverging
-        else if (it >= sh.max_iter) sh.stop = 1;
-        sh.done = sh.stop;
-      }
-    }
+  if (tid == 0 && !persist::wait_block(sh.sync, r_round, &sh.seen)) sh.stop = 1;
+  __syncthreads();
+  if (sh.stop) return;
+  double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
+  persist::publish_vec(sh.sync, round, sh.r_all, sh.n, red, sh.sums);
+  double rrn;
+  if (persist::gather_sum(sh.sync, round, sh.sync.m->vec, persist::vec_blocks<X>(sh.n), red, &sh.stop, &rrn) &&
+      tid == 0) {
+    const int it = sh.it + 1;
+    if (blockIdx.x == 0) sh.hist[it] = rrn;
+    sh.beta = rrn / sh.rr;
+    sh.rr = rrn;
+    sh.it = it;
+    if (rrn <= sh.tol2) sh.converged = sh.stop = 1;
+    else if (!(rrn <= sh.grow_limit)) sh.breakdown = sh.stop = 1;  // non-finite or diverging
+    else if (it >= sh.max_iter) sh.stop = 1;
+    sh.done = sh.stop;
   }
   __syncthreads();
 }
@@ -567,6 +541,9 @@ __global__ void __launch_bounds__(MAXT, 1) cg_persist_kernel(core::KArgs a, cons
       sh.r = r;
       sh.x = x;
       sh.p = c.p + pb;
+      sh.rm = c.r_off >= 0 ? c.r + pb : nullptr;
+      sh.r_all = c.r;
+      sh.n = (int)a.n;
       sh.hist = c.hist;
       sh.red_off = c.red_off;
       sh.sync = c.sync;
@@ -592,20 +569,21 @@ __global__ void __launch_bounds__(MAXT, 1) cg_persist_kernel(core::KArgs a, cons
   }
   __syncthreads();
   for (int step = 0; step < c.max_steps; ++step) {
-    const int round = 2 * step + 1;  // of the sums
-    // q = A p; p of the other blocks from round `step` on (their p at launch: nothing to wait for)
+    // rounds of the sums p.q and r.r, and rounds of arrivals with r and p: 2 step + 1 and 2 step + 2 each
+    const int round = 2 * step + 1;
+    // q = A p; p of the other blocks from round 2 step on (their p at launch: nothing to wait for)
     if (sh.nh > 0) {
-      if (!persist::wait_round(sh.sync, step, &sh.seen)) sh.stop = 1;
+      if (!persist::wait_round(sh.sync, 2 * step, &sh.seen)) sh.stop = 1;
       for (int j = threadIdx.x; j < sh.nh; j += bd)
         ps[checked(sh.prod.rows + j, a.smem_elems, a.status)] = load_x(c.p + checked(sh.halo[j], a.n, a.status));
       __syncthreads();
     }
-    persist::run_slices<V, X, KB, RUNS>(&sh.prod, &sh.sync, step);
+    persist::run_slices<V, X, KB, RUNS>(&sh.prod, &sh.sync, 2 * step);
     __syncthreads();
     if (sh.stop) break;
     cg_step_pq(sh, round);
     if (sh.stop) break;
-    cg_step_update(sh, round);
+    cg_step_update(sh, round + 1, round);
     if (sh.stop) break;
     cg_step_direction(sh);
     __syncthreads();
@@ -613,12 +591,10 @@ __global__ void __launch_bounds__(MAXT, 1) cg_persist_kernel(core::KArgs a, cons
   }
   __syncthreads();
   {
-    const X *const r = sh.r, *const x = sh.x;
+    const X* const x = sh.x;
     const int rows = sh.prod.rows, pb = sh.prod.pb;
-    for (int i = threadIdx.x; i < rows; i += bd) {
-      if (c.r_off >= 0) c.r[pb + i] = r[i];
-      if (c.x_off >= 0) c.x[pb + i] = x[i];
-    }
+    if (c.x_off >= 0)
+      for (int i = threadIdx.x; i < rows; i += bd) c.x[pb + i] = x[i];
   }
   // a launch that ran out of steps leaves with p updated; one that gave up has told the host already
   if (blockIdx.x == 0 && threadIdx.x == 0 && (sh.done || !sh.stop)) {
@@ -738,9 +714,10 @@ ehyb_status_t run_chunk(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s) {
 }
 
 // One persistent launch of at most kPersistSteps iterations; *ran = false (and nothing launched) for a plan that
-// needs the separate launches: more partitions than SMs (a block owns one partition, all blocks resident), a
-// wide slice (its sums go through the plan's workspace), more shared memory than persist::shared_budget grants, FP32
-// vectors of more than persist::kMaxRows32 rows a partition, the staging-fault test hook.
+// needs the separate launches: more partitions than SMs (a block owns one partition, all blocks resident), a wide
+// slice (its sums go through the plan's workspace), more shared memory than persist::shared_budget grants, more rows
+// a partition than persist::even_enough or, with FP32 vectors, kMaxRowsF32 / kMaxRowsBf16 allow, the staging-fault
+// test hook.
 constexpr int kPersistSteps = 2000;  // bounds one launch to a fraction of a second
 
 template <typename V, typename X, int KB, bool RUNS, int MAXT>
@@ -755,22 +732,23 @@ ehyb_status_t launch_persist(ehyb_plan_t P, const V* ev, const V* erv, CgPersist
   int optin = 0, resident = 0, sms = 0;
   CKC(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, P->device));
   CKC(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device));
+  if (!persist::even_enough(D.max_part_rows, D.n, sms, sizeof(X) == 8 ? persist::kSpare64 : persist::kSpare32))
+    return EHYB_OK;
   auto al = [](size_t b) { return (b + 15) & ~(size_t)15; };
   size_t smem = ehyb_smem_bytes(D, (int)sizeof(X));
   a.smem_elems = (int64_t)(smem / sizeof(X));
   const size_t tbl = al((size_t)D.max_part_slices * sizeof(core::SliceMeta));
   const size_t vec = al((size_t)D.max_part_rows * sizeof(X));
-  const size_t budget = std::min((size_t)optin - 1024, persist::shared_budget(smem + (size_t)D.threads * sizeof(double)));
+  const size_t budget = std::min((size_t)optin - 1024, persist::shared_budget(smem + persist::terms_bytes(D.threads)));
   auto place = [&](size_t bytes) -> int32_t {
     if (smem + bytes > budget) return -1;
     const size_t o = smem;
     smem += bytes;
     return (int32_t)o;
   };
-  c.red_off = place((size_t)D.threads * sizeof(double));
+  c.red_off = place(persist::terms_bytes(D.threads));
   c.tbl_off = place(tbl);
   a.meta_cap = D.max_part_slices;
-  *ran = false;
   if (c.red_off < 0) return EHYB_OK;
   c.q_off = place(vec);
   c.r_off = place(vec);
@@ -797,7 +775,7 @@ ehyb_status_t run_persist(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s, bo
     return D.kbatch == 6 ? launch_persist<double, double, 6, false, 1024>(P, D.ell_val, D.er_sval, c, s, ran)
                          : launch_persist<double, double, 8, false, 1024>(P, D.ell_val, D.er_sval, c, s, ran);
   }
-  if (D.max_part_rows > persist::kMaxRows32) return EHYB_OK;
+  if (D.max_part_rows > (lowp == 1 ? persist::kMaxRowsF32 : persist::kMaxRowsBf16)) return EHYB_OK;
   const CgPersist<float> c{w->d32, w->r32, w->p32, w->q32, -1, -1, -1, -1, -1, kPersistSteps, w->st, w->hist, sync};
   const bool runs = D.lowp_group == 4, half = D.threads <= 512;
   if (lowp == 1)

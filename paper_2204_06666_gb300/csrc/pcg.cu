@@ -40,8 +40,7 @@ namespace ehyb {
 namespace {
 
 using core::FULL;
-constexpr int kVB = 608;  // vector-kernel blocks (4 per SM; 8 per SM measured slower)
-constexpr int kVT = 256;
+constexpr int kVB = persist::kVecBlocks, kVT = persist::kVecThreads;  // vector kernels
 constexpr int kChunk = 16;
 
 }  // namespace
@@ -387,17 +386,18 @@ __global__ void pcg_pupdate32_force(int64_t n, const float* __restrict__ z, floa
 }
 
 // ---- persistent iterations (persist.cuh): up to max_steps iterations of K1 .. K5 in one cooperative launch, block p
-// owning partition p's rows, which are the same rows in A's, G's and G^T's plans.  XA is the type of x, p, q
-// and r, XG that of the preconditioner's vectors.  p, r, t, q (z after the update) and x stay in shared memory as
-// far as they fit; p, r and t are mirrored to memory for the other blocks' extra rows.  The blocks meet five times
-// an iteration: for the sums p.q, r.r (which orders r for K3) and t.t, and for t and the new p, which a warp waits
-// for only when it comes to its first extra row (t.t is not needed before K5: it travels during K4).
+// owning partition p's rows, which are the same rows in A's, G's and G^T's plans; every sum in the order of the
+// separate launches.  XA is the type of x, p, q and r, XG that of the preconditioner's vectors.  p, r, t, q (z after
+// the update) and x stay in shared memory as far as they fit; p, r and t are mirrored to memory for the other blocks'
+// extra rows (r for r.r too).  The blocks meet six times an iteration: for the sums p.q, r.r and t.t, and for r, t
+// and the new p, the last two of which a warp waits for only when it comes to its first extra row (t.t is not needed
+// before K5: it travels during K4).
 template <typename XA, typename XG>
 struct PcgPersist {
   XA *x, *r, *p, *q;
   XG *rg, *t, *z;                             // rg: r in XG's type (r itself when the types agree)
   int32_t gs_off, q_off, r_off, t_off, x_off;  // byte offsets in dynamic shared memory; -1: in global memory
-  int32_t red_off;
+  int32_t red_off, g_warps;                   // the sums' terms; warps of G's product
   int32_t h_off;                              // r, then t, staged for the extra rows of G and G^T (-1: gathered)
   int32_t tbl_off[3];
   int32_t max_steps;
@@ -414,74 +414,54 @@ struct PcgBlock {
   int it, max_iter, converged, breakdown, done, stop, seen;
   XA *q, *r, *x, *p;  // p: the block's rows of p in memory
   XG *z, *t, *rg;     // rg: its rows of r in memory, in XG's type
+  XA* rm;             // r's mirror in memory (null: r lies there, or rg is it)
+  const XA* r_all;    // r of all blocks in memory
+  int n;
   persist::Product<VA, XA> a;
   persist::Product<VG, XG> g, h;
   double* hist;
   double rr_limit;
-  int32_t red_off, gs_off;
+  int32_t red_off, gs_off, g_warps;
+  double sums[32];
   persist::SyncArgs sync;
 };
 
 // p.q and alpha
 template <typename VA, typename XA, typename VG, typename XG>
 __device__ __noinline__ void pcg_step_pq(PcgBlock<VA, XA, VG, XG>& sh, int round) {
-  constexpr int U = 4;  // elements a thread has in flight
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  XA* const ps = reinterpret_cast<XA*>(smem_raw);
+  const XA* const ps = reinterpret_cast<const XA*>(smem_raw);
   double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
-  const int bd = blockDim.x;
+  const int warps = blockDim.x >> 5;
   {
     const XA* const q = sh.q;
-    const int rows = sh.a.rows;
-    double acc = 0.0;
-    const int tid = threadIdx.x;
-    for (int i0 = tid; i0 < rows; i0 += U * bd) {
-      XA qv[U], pv[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int i = i0 + u * bd;
-        qv[u] = i < rows ? q[i] : XA(0);
-        pv[u] = i < rows ? ps[i] : XA(0);
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (i0 + u * bd < rows) acc = fma((double)qv[u], (double)pv[u], acc);
-    }
-    red[tid] = acc;
+    persist::part_terms(sh.a, warps, red, [&](int i) { return make_double2((double)q[i], (double)ps[i]); });
   }
   __syncthreads();
-  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round, red);
-  if (threadIdx.x < 32) {
-    double pq;
-    const bool ok = persist::gather_sum<false>(sh.sync, round, &pq);
-    if (threadIdx.x == 0) {
-      sh.a.counter = sh.h.counter = bd >> 5;  // for the next products of A and G^T
-      if (!ok) sh.stop = 1;
-      else if (!(pq > 0.0)) sh.breakdown = sh.done = sh.stop = 1;  // not positive definite along p (or p vanished)
-      else sh.alpha = sh.rz / pq;
-    }
+  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_part(sh.sync, round, 0, red, warps, sh.sums);
+  double pq;
+  const bool ok = persist::gather_sum(sh.sync, round, sh.sync.m->part[0], gridDim.x, red, &sh.stop, &pq);
+  if (threadIdx.x == 0) {
+    sh.a.counter = sh.h.counter = warps;  // for the next products of A and G^T
+    if (ok && !(pq > 0.0)) sh.breakdown = sh.done = sh.stop = 1;  // not positive definite along p (or p vanished)
+    else if (ok) sh.alpha = sh.rz / pq;
   }
   __syncthreads();
 }
 
 template <typename VA, typename XA, typename VG, typename XG>
-__device__ __noinline__ void pcg_step_update(PcgBlock<VA, XA, VG, XG>& sh, int round) {
+__device__ __noinline__ void pcg_step_update(PcgBlock<VA, XA, VG, XG>& sh, int round, int r_round) {
   using namespace core;
   constexpr int U = 4;  // elements a thread has in flight
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  XA* const ps = reinterpret_cast<XA*>(smem_raw);
+  const XA* const ps = reinterpret_cast<const XA*>(smem_raw);
   XG* const gs = reinterpret_cast<XG*>(smem_raw + sh.gs_off);
-  double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
-  const int bd = blockDim.x;
-  // K2: r -= alpha q (and r for the other blocks' extra rows), r.r; then x += alpha p while the sum is on its way
-  {
-    const XA al = (XA)sh.alpha;
+  const int bd = blockDim.x, tid = threadIdx.x, rows = sh.a.rows;
+  const XA al = (XA)sh.alpha;
+  {  // K2: r -= alpha q
     const XA* const q = sh.q;
-    XA* const r = sh.r;
+    XA *const r = sh.r, *const rm = sh.rm;
     XG* const rg = sh.rg;
-    const int rows = sh.a.rows;
-    double acc = 0.0;
-    const int tid = threadIdx.x;
     for (int i0 = tid; i0 < rows; i0 += U * bd) {
       XA qv[U], rv[U];
 #pragma unroll
@@ -497,35 +477,31 @@ __device__ __noinline__ void pcg_step_update(PcgBlock<VA, XA, VG, XG>& sh, int r
           rv[u] = fma(-al, qv[u], rv[u]);
           r[i] = rv[u];
           rg[i] = (XG)rv[u];
-          acc = fma((double)rv[u], (double)rv[u], acc);
+          if (rm) rm[i] = rv[u];
         }
       }
     }
-    red[tid] = acc;
   }
   __syncthreads();
-  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<true>(sh.sync, round + 1, red);
-  __syncthreads();  // the update of x would delay the sum: both need the FP64 unit
-  if (threadIdx.x >= 32 || bd == 32) {
-    const int tid = threadIdx.x;
-    const XA al = (XA)sh.alpha;
+  if (tid == 0) persist::arrive(sh.sync);
+  {  // x += alpha p while r is on its way
     XA* const x = sh.x;
     const XA* const r = sh.r;
     const int32_t* const n2o = sh.g.n2o;
-    const int rows = sh.a.rows, pb = sh.a.pb, ts = bd == 32 ? 32 : bd - 32, t0 = bd == 32 ? tid : tid - 32;
-    for (int i0 = t0; i0 < rows; i0 += U * ts) {
+    const int pb = sh.a.pb;
+    for (int i0 = tid; i0 < rows; i0 += U * bd) {
       XA xv[U], pv[U];
       int m[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int i = i0 + u * ts;
+        const int i = i0 + u * bd;
         m[u] = i < rows ? checked(n2o[i] - pb, rows, sh.a.status) : 0;
         xv[u] = i < rows ? x[i] : XA(0);
         pv[u] = i < rows ? ps[i] : XA(0);
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int i = i0 + u * ts;
+        const int i = i0 + u * bd;
         if (i < rows) {
           x[i] = fma(al, pv[u], xv[u]);
           gs[checked(i, rows, sh.a.status)] = (XG)r[m[u]];  // K3's slice of r in G's row order
@@ -533,22 +509,21 @@ __device__ __noinline__ void pcg_step_update(PcgBlock<VA, XA, VG, XG>& sh, int r
       }
     }
   }
-  if (threadIdx.x < 32) {
-    double rr;
-    const bool ok = persist::gather_sum<true>(sh.sync, round + 1, &rr);
-    if (threadIdx.x == 0) {
-      if (!ok) {
-        sh.stop = 1;
-      } else {
-        const int it = sh.it + 1;
-        sh.it = it;
-        if (blockIdx.x == 0) sh.hist[it] = rr;
-        sh.rz_old = sh.rz;
-        if (rr <= sh.tol2) sh.converged = sh.stop = 1;
-        else if (!(rr < sh.rr_limit) || it >= sh.max_iter) sh.stop = 1;
-        sh.done = sh.stop;
-      }
-    }
+  if (tid == 0 && !persist::wait_block(sh.sync, r_round, &sh.seen)) sh.stop = 1;
+  __syncthreads();
+  if (sh.stop) return;
+  double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
+  persist::publish_vec(sh.sync, round, sh.r_all, sh.n, red, sh.sums);
+  double rr;
+  if (persist::gather_sum(sh.sync, round, sh.sync.m->vec, persist::vec_blocks<XA>(sh.n), red, &sh.stop, &rr) &&
+      tid == 0) {
+    const int it = sh.it + 1;
+    sh.it = it;
+    if (blockIdx.x == 0) sh.hist[it] = rr;
+    sh.rz_old = sh.rz;
+    if (rr <= sh.tol2) sh.converged = sh.stop = 1;
+    else if (!(rr < sh.rr_limit) || it >= sh.max_iter) sh.stop = 1;
+    sh.done = sh.stop;
   }
   __syncthreads();
 }
@@ -561,31 +536,26 @@ __device__ __noinline__ void pcg_step_tt(PcgBlock<VA, XA, VG, XG>& sh, int round
   extern __shared__ __align__(16) unsigned char smem_raw[];
   XG* const gs = reinterpret_cast<XG*>(smem_raw + sh.gs_off);
   double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
-  const int bd = blockDim.x;
+  const int bd = blockDim.x, rows = sh.a.rows, pb = sh.a.pb;
+  const XG* const t = sh.t;
   {
-    const XG* const t = sh.t;
-    const int32_t* const n2o = sh.h.n2o;
-    const int rows = sh.a.rows, pb = sh.a.pb;
-    double acc = 0.0;
-    const int tid = threadIdx.x;
-    for (int i0 = tid; i0 < rows; i0 += U * bd) {
-      int m[U];
+    const int32_t* const n2o = sh.g.n2o;
+    persist::part_terms(sh.g, sh.g_warps, red, [&](int i) {
+      const double v = (double)t[checked(n2o[i] - pb, rows, sh.a.status)];
+      return make_double2(v, v);
+    });
+  }
+  const int32_t* const n2o = sh.h.n2o;
+  for (int i0 = threadIdx.x; i0 < rows; i0 += U * bd) {
+    int m[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) m[u] = i0 + u * bd < rows ? checked(n2o[i0 + u * bd] - pb, rows, sh.a.status) : 0;
+    for (int u = 0; u < U; ++u) m[u] = i0 + u * bd < rows ? checked(n2o[i0 + u * bd] - pb, rows, sh.a.status) : 0;
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int i = i0 + u * bd;
-        if (i < rows) {
-          const XG v = t[m[u]];
-          gs[checked(i, rows, sh.a.status)] = v;  // K4's slice of t in G^T's row order
-          acc = fma((double)v, (double)v, acc);
-        }
-      }
-    }
-    red[tid] = acc;
+    for (int u = 0; u < U; ++u)  // K4's slice of t in G^T's row order
+      if (i0 + u * bd < rows) gs[checked(i0 + u * bd, rows, sh.a.status)] = t[m[u]];
   }
   __syncthreads();
-  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_sum<false>(sh.sync, round + 2, red);
+  if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_part(sh.sync, round, 1, red, sh.g_warps, sh.sums);
 }
 
 // beta from t.t, then the direction
@@ -595,17 +565,14 @@ __device__ __noinline__ void pcg_step_direction(PcgBlock<VA, XA, VG, XG>& sh, in
   extern __shared__ __align__(16) unsigned char smem_raw[];
   XA* const ps = reinterpret_cast<XA*>(smem_raw);
   const int bd = blockDim.x;
-  if (threadIdx.x < 32) {
-    double tt;
-    const bool ok = persist::gather_sum<false>(sh.sync, round + 2, &tt);
-    if (threadIdx.x == 0) {
-      sh.g.counter = bd >> 5;
-      if (!ok) {
-        sh.stop = 1;
-      } else {
-        sh.rz = tt;
-        sh.beta = tt / sh.rz_old;
-      }
+  double tt;
+  const bool ok = persist::gather_sum(sh.sync, round, sh.sync.m->part[1], gridDim.x,
+                                      reinterpret_cast<double*>(smem_raw + sh.red_off), &sh.stop, &tt);
+  if (threadIdx.x == 0) {
+    sh.g.counter = bd >> 5;
+    if (ok) {
+      sh.rz = tt;
+      sh.beta = tt / sh.rz_old;
     }
   }
   __syncthreads();
@@ -672,6 +639,10 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_persist_kernel(core::KArgs a, con
       sh.x = x;
       sh.p = c.p + pb;
       sh.rg = c.rg + pb;
+      sh.rm = c.r_off >= 0 && !std::is_same<XA, XG>::value ? c.r + pb : nullptr;
+      sh.r_all = c.r;
+      sh.n = (int)a.n;
+      sh.g_warps = c.g_warps;
       sh.hist = c.hist;
       sh.rr_limit = c.rr_limit;
       sh.red_off = c.red_off;
@@ -708,37 +679,36 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_persist_kernel(core::KArgs a, con
   }
   __syncthreads();
   for (int step = 0; step < c.max_steps; ++step) {
-    const int round = 3 * step + 1;  // of the sums
-    // K1: q = A p (p of the other blocks from round 2 step on), p.q
-    persist::run_slices<VA, XA, KA, kRunsA>(&sh.a, &sh.sync, 2 * step);
+    // rounds of the sums p.q, r.r and t.t, and rounds of arrivals with r, t and p: 3 step + 1, + 2 and + 3 each
+    const int round = 3 * step + 1;
+    // K1: q = A p (p of the other blocks from round 3 step on), p.q
+    persist::run_slices<VA, XA, KA, kRunsA>(&sh.a, &sh.sync, 3 * step);
     __syncthreads();
     if (sh.stop) break;
     pcg_step_pq(sh, round);
     if (sh.stop) break;
-    pcg_step_update(sh, round);
+    pcg_step_update(sh, round + 1, round);
     if (sh.stop) break;
     // K3: t = G r, t.t = r.z
-    persist::stage_halo(&sh.g, &sh.sync, 0);
-    persist::run_slices<VG, XG, KG, kRunsG>(&sh.g, &sh.sync, 0);  // r of all blocks: ordered by the sum above
+    persist::stage_halo(&sh.g, &sh.sync, round);
+    persist::run_slices<VG, XG, KG, kRunsG>(&sh.g, &sh.sync, round);
     __syncthreads();
-    if (threadIdx.x == 0) persist::arrive(sh.sync);  // t: round 2 step + 1
-    pcg_step_tt(sh, round);
+    if (threadIdx.x == 0) persist::arrive(sh.sync);  // t
+    pcg_step_tt(sh, round + 2);
     // K4: z = G^T t
-    persist::stage_halo(&sh.h, &sh.sync, 2 * step + 1);
-    persist::run_slices<VG, XG, KG, kRunsG>(&sh.h, &sh.sync, 2 * step + 1);
-    pcg_step_direction(sh, round);
+    persist::stage_halo(&sh.h, &sh.sync, round + 1);
+    persist::run_slices<VG, XG, KG, kRunsG>(&sh.h, &sh.sync, round + 1);
+    pcg_step_direction(sh, round + 2);
     if (sh.stop) break;
     __syncthreads();
-    if (threadIdx.x == 0) persist::arrive(sh.sync);  // p: round 2 (step + 1)
+    if (threadIdx.x == 0) persist::arrive(sh.sync);  // p
   }
   __syncthreads();
   {
-    const XA *const r = sh.r, *const x = sh.x;
+    const XA* const x = sh.x;
     const int rows = sh.a.rows, pb = sh.a.pb;
-    for (int i = threadIdx.x; i < rows; i += bd) {
-      if (c.r_off >= 0) c.r[pb + i] = r[i];
-      if (c.x_off >= 0) c.x[pb + i] = x[i];
-    }
+    if (c.x_off >= 0)
+      for (int i = threadIdx.x; i < rows; i += bd) c.x[pb + i] = x[i];
   }
   // a launch that ran out of steps leaves with p updated; one that gave up has told the host already
   if (blockIdx.x == 0 && threadIdx.x == 0 && (sh.done || !sh.stop)) {
@@ -858,8 +828,9 @@ ehyb_status_t enqueue_chunk32(ehyb_precond_t M, PcgWork* w, cudaStream_t s) {
 }
 
 // One persistent launch of at most kPersistSteps iterations; *ran = false (and nothing launched) where the separate
-// launches are needed: more partitions than SMs, a wide slice, copies not in runs of four, more shared
-// memory than persist::shared_budget grants, FP32 vectors of more than persist::kMaxRows32 rows a partition, the staging-fault test hook.
+// launches are needed: more partitions than SMs, a wide slice, copies not in runs of four, more shared memory than
+// persist::shared_budget grants, more rows a partition than persist::even_enough (FP64 vectors, low-precision G) or
+// kMaxRowsPcg32 (FP32 vectors) allow, the staging-fault test hook.
 constexpr int kPersistSteps = 2000;  // bounds one launch to a fraction of a second
 
 template <typename VA, typename XA, int KA, typename VG, typename XG, int MAXT>
@@ -886,21 +857,23 @@ ehyb_status_t launch_persist(ehyb_precond_t M, const VA* av, const VA* aev, cons
   int optin = 0, resident = 0, sms = 0;
   CKP(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, M->plan->device));
   CKP(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, M->plan->device));
+  if (sizeof(XG) < sizeof(XA) && !persist::even_enough(D.max_part_rows, D.n, sms, persist::kSparePcg)) return EHYB_OK;
   auto al = [](size_t b) { return (b + 15) & ~(size_t)15; };
   size_t smem = ehyb_smem_bytes(D, (int)sizeof(XA));
   a.smem_elems = (int64_t)(smem / sizeof(XA));
   const size_t va = (size_t)D.max_part_rows * sizeof(XA), vg = (size_t)D.max_part_rows * sizeof(XG);
+  const size_t terms = persist::terms_bytes(std::max(D.threads, G.threads));
+  c.g_warps = G.threads / 32;
   const size_t budget =
-      std::min((size_t)optin - 1024, persist::shared_budget(smem + al(vg) + (size_t)D.threads * sizeof(double)));
+      std::min((size_t)optin - 1024, persist::shared_budget(smem + al(vg) + terms));
   auto place = [&](size_t bytes) -> int32_t {
     if (smem + al(bytes) > budget) return -1;
     const size_t o = smem;
     smem += al(bytes);
     return (int32_t)o;
   };
-  *ran = false;
   c.gs_off = place(vg);
-  c.red_off = place((size_t)D.threads * sizeof(double));
+  c.red_off = place(terms);
   if (c.gs_off < 0 || c.red_off < 0) return EHYB_OK;
   g.smem_elems = h.smem_elems = D.max_part_rows;
   c.q_off = place(va);
@@ -937,7 +910,7 @@ ehyb_status_t run_persist(ehyb_precond_t M, PcgWork* w, cudaStream_t s, bool inn
   // the three plans own the same rows block by block
   if (M->g->host.part_ptr != P->host.part_ptr || M->gt->host.part_ptr != P->host.part_ptr) return EHYB_OK;
   if (M->lowp && (G.lowp_group != 4 || H.lowp_group != 4)) return EHYB_OK;
-  if (inner32 && (D.lowp_group != 4 || D.max_part_rows > persist::kMaxRows32)) return EHYB_OK;
+  if (inner32 && (D.lowp_group != 4 || D.max_part_rows > persist::kMaxRowsPcg32)) return EHYB_OK;
   const persist::SyncArgs sync{w->meeting, D.status, &w->st->done, std::max(D.wait_timeout_ns, persist::kMinLimitNs)};
   const bool half = D.threads <= 512;
   auto with_g = [&](auto va, const auto* av, const auto* aev, auto c, auto ka, auto mt) -> ehyb_status_t {
@@ -968,18 +941,18 @@ ehyb_status_t run_persist(ehyb_precond_t M, PcgWork* w, cudaStream_t s, bool inn
                 : with_g(va, av, aev, c, integral_constant<int, 16>(), t1024);
   };
   if (inner32) {
-    const PcgPersist<float, float> c{w->d32, w->r32, w->p32, w->q32, w->r32, w->t32, w->z32, -1, -1, -1, -1, -1, -1, -1,
-                                     {-1, -1, -1}, kPersistSteps, 1e30, w->st, w->hist, sync};
+    const PcgPersist<float, float> c{w->d32, w->r32, w->p32, w->q32, w->r32, w->t32, w->z32, -1, -1, -1, -1, -1, -1, 0,
+                                     -1, {-1, -1, -1}, kPersistSteps, 1e30, w->st, w->hist, sync};
     return P->lowp == 1 ? fp32(float(), D.ell_val_f32, D.er_sval_f32, c)
                         : fp32(uint16_t(), D.ell_val_bf16, D.er_sval_bf16, c);
   }
   if (M->lowp) {
-    const PcgPersist<double, float> c{w->xp, w->r, w->p, w->q, w->r32, w->t32, w->z32, -1, -1, -1, -1, -1, -1, -1,
-                                      {-1, -1, -1}, kPersistSteps, 1e300, w->st, w->hist, sync};
+    const PcgPersist<double, float> c{w->xp, w->r, w->p, w->q, w->r32, w->t32, w->z32, -1, -1, -1, -1, -1, -1, 0,
+                                      -1, {-1, -1, -1}, kPersistSteps, 1e300, w->st, w->hist, sync};
     return fp64(c);
   }
-  const PcgPersist<double, double> c{w->xp, w->r, w->p, w->q, w->r, w->t, w->z, -1, -1, -1, -1, -1, -1, -1,
-                                     {-1, -1, -1}, kPersistSteps, 1e300, w->st, w->hist, sync};
+  const PcgPersist<double, double> c{w->xp, w->r, w->p, w->q, w->r, w->t, w->z, -1, -1, -1, -1, -1, -1, 0,
+                                     -1, {-1, -1, -1}, kPersistSteps, 1e300, w->st, w->hist, sync};
   return fp64(c);
 }
 

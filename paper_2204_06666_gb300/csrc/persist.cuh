@@ -1,19 +1,24 @@
-// Device code of the persistent solver kernels (cg.cu, pcg.cu): a whole Krylov iteration, and then the next,
-// inside one cooperative launch with one block per partition.
+// Device code of the persistent solver kernels (cg.cu, pcg.cu): a whole Krylov iteration, and then the next, inside
+// one cooperative launch with one block per partition.
 //
-// A solver iteration as separate launches re-reads what the block that owns a partition has just had in hand:
-// the direction is staged into shared memory for every product, q and r go through memory between the product
-// and the updates, and every launch drains and refills the chip (tet 80^3, 512k rows: product 29 us, update 14
-// us, direction 5 us cold, 44 us an iteration back to back from a graph, for 74 MB of matrix).  Here a block keeps
-// its partition's slices of the vectors in shared memory from one iteration to the next, as many of them as fit,
-// and the iteration's inner products double as the barriers that the data dependences need.  Scalars (a division
-// is a dozen dependent FP64 operations, and FP64 operations of 32 warps queue for one unit) are one thread's work.
-// Whole solves of (A + 0.1 mean diagonal) x = b to 1e-10, separate launches -> persistent, FP64 CG (40 to 66
-// iterations): tet 20^3 0.96 -> 0.61 ms, 40^3 1.11 -> 0.76, 80^3 2.06 -> 1.56, 126^3 4.55 -> 4.19, elasticity 24^3 1.86 ->
-// 1.34, 48^3 5.19 -> 4.90, 70^3 10.87 -> 10.75; elasticity 30^3 (81k rows, bound by 17 slices on four quarters of an SM)
-// 2.54 both.  Mixed-precision PCG: tet 80^3 2.13 -> 1.53, elasticity 40^3 3.56 -> 2.90, 70^3 8.33 -> 7.70; FP64 PCG: tet 80^3 1.76 -> 1.25, elasticity 70^3 11.69 -> 11.45.  A third of the tet 80^3 iteration is still outside the product: FP64
-// vector arithmetic (five FMAs a row, 4.4 us at the pipe's rate) and the three meetings.
+// A solver iteration as separate launches re-reads what the block that owns a partition has just had in hand: the
+// direction is staged into shared memory for every product, q and r go through memory between the product and the
+// updates, and every launch drains and refills the chip (tet 80^3, 512k rows: product 29 us, update 14 us, direction
+// 5 us cold, 44 us an iteration back to back from a graph, for 74 MB of matrix).  Here a block keeps its partition's
+// slices of the vectors in shared memory from one iteration to the next, as many of them as fit, and the iteration's
+// inner products double as the barriers that the data dependences need.  Scalars (a division is a dozen dependent
+// FP64 operations, and FP64 operations of 32 warps queue for one unit) are one thread's work.
+//
+// The sums are added in the order of the separate launches, so both forms give the same bits; that costs a meeting
+// more an iteration (r.r, below) and a serial chain over the block's warps (p.q: 32 dependent FP64 additions, 1.6
+// us): 35.1 us an iteration at tet 80^3, 33.1 with sums in the blocks' own order, 42 in separate launches. Whole
+// solves of (A + 0.1 mean diagonal) x = b to 1e-10, separate launches -> persistent, FP64 CG (44 to 65 iterations):
+// tet 40^3 1.10 -> 0.82 ms, 80^3 2.10 -> 1.77, 126^3 4.62 -> 4.48, elasticity 24^3 2.14 -> 1.46, 40^3 3.87 -> 3.43,
+// 64^3 9.32 -> 8.80. Mixed-precision PCG (1e-9): tet 80^3 1.77 -> 1.33, elasticity 40^3 3.55 -> 2.93, 64^3 7.32 ->
+// 6.89; FP64 PCG: tet 80^3 1.74 -> 1.32, elasticity 64^3 9.88 -> 9.33.
 #pragma once
+#include <algorithm>
+
 #include "ehyb_core.cuh"
 
 namespace ehyb {
@@ -25,15 +30,23 @@ constexpr int kMaxGrid = 160;      // blocks of a persistent launch (five partia
 constexpr uint64_t kMinLimitNs = 2000000000ull;  // least time limit of a wait for the other blocks
 constexpr int kAborted = 2;
 
-// One block's partial sum: the halves of a double, each beside the number of its round in an 8-byte word of its own, so
-// that a reader sees for each half whether it is the one it waits for.
+// Grid of the vector kernels of the separate launches.  Their inner products add a vector's squares in the order of
+// these threads, blocks and partials, and the persistent kernels add them in the same one: a solve's bits do not
+// depend on the form its iterations take.
+constexpr int kVecBlocks = 608;  // 4 per SM; 8 per SM measured slower
+constexpr int kVecThreads = 256;
+constexpr int kVecWarps = kVecThreads / 32;
+
+// A partial sum: the halves of a double, each beside the number of its round in an 8-byte word of its own, so that a
+// reader sees for each half whether it is the one it waits for.
 struct __align__(16) Slot {
   unsigned long long lo, hi;
 };
 
 // The memory the blocks meet in, all zero at launch.
 struct Meeting {
-  Slot slot[2][kMaxGrid];    // partial sums of the even and the odd rounds of sums
+  Slot part[2][kMaxGrid];    // partitions' partial sums: p.q; t.t
+  Slot vec[kVecBlocks];      // vector blocks' partial sums: r.r
   int32_t summed, pad0[31];  // blocks that have published, over all rounds of sums
   int32_t arrived, pad1[31]; // arrivals at the plain rounds
 };
@@ -58,13 +71,23 @@ inline size_t shared_budget(size_t must) {
   return 0;
 }
 
-// Rows of a partition up to which FP32 iterations run persistently.  Beyond, the FP32 products are short of bytes rather
-// than of launches, and the vectors' passes of the separate launches are the faster ones (us an iteration, separate ->
-// persistent: tet 102^3, 6,982 rows, CG 42.8 -> 39.5, mixed PCG 85.4 -> 79.9; tet 114^3, 9,747 rows, 50.8 -> 52.1 and
-// 99.9 -> 106.8; tet 126^3 61.0 -> 65.3 and 127.1 -> 139.7; FP64 iterations gain there: CG 93.6 -> 85.4, PCG 203.7 -> 202.3).
-constexpr int kMaxRows32 = 8192;
+// Rows of a partition up to which iterations on FP32 vectors run persistently.  Beyond, the FP32 products are short
+// of bytes rather than of launches, and the vectors' passes of the separate launches are the faster ones.  CG, us an
+// iteration separate -> persistent, FP32 values: tet 90^3 (4,797 rows) 44.1 -> 43.3, 96^3 (5,821) 47.7 -> 48.1, 104^3
+// (7,401) 53.4 -> 54.1; BF16: tet 90^3 46.3 -> 46.8, 107^3 (8,060) 58.4 -> 61.1, elasticity 64^3 (5,174) 92.0 ->
+// 97.7.  Mixed PCG: tet 107^3 162 -> 144; 114^3 (9,747 rows) and 126^3 lost about a tenth before its sums took the
+// launches' order.
+constexpr int kMaxRowsF32 = 5500, kMaxRowsBf16 = 4500, kMaxRowsPcg32 = 8192;
 
-__device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+// Whether a plan's partitions are even enough with the SMs: a block passes over its partition's vectors alone, where
+// the separate launches spread them over the chip, so each row beyond the chip's share costs about 1.7 ns an
+// iteration of FP64 CG against the 5 us or so that the launches cost.  `spare`: the rows beyond n / SMs up to which
+// persistent iterations were the faster ones (ms a solve, separate -> persistent; FP64 CG: tet 37^3 in partitions of
+// 3,000 rows 1.57 -> 1.48, of 6,000 2.11 -> 2.23, tet 60^3 in 6,000 2.28 -> 2.36, tet 90^3 in 8,000 3.03 -> 2.94, in
+// 10,000 3.40 -> 3.55; FP32 CG: elasticity 24^3 in 3,000 4.12 -> 3.96, in 6,000 5.71 -> 6.18; FP64 PCG with BF16 G:
+// tet 60^3 in 6,000 1.78 -> 1.70, in 12,000 2.56 -> 2.87; the other PCG forms gained at every size).
+inline bool even_enough(int max_rows, int64_t n, int sms, int spare) { return max_rows - n / sms <= spare; }
+constexpr int kSpare64 = 3500, kSpare32 = 2500, kSparePcg = 4500;
 
 // a wait that has lasted: true when it must give up (its limit is over, or another block gave up)
 struct Patience {
@@ -100,85 +123,214 @@ __device__ __forceinline__ bool wait_at(const SyncArgs& g, const int32_t* counte
   }
 }
 
-// Sum over all threads of all blocks, which is a grid-wide barrier too, in two halves so that a block can work in
-// between.  Every thread has put its term into red[threadIdx.x] and passed a __syncthreads; then, for the launch's
-// sums number round = 1, 2, ...:
-//   publish_sum (the block's first four warps): the block's sum into its slot, then one more on the counter;
-//   gather_sum (warp 0): waits for the counter, then adds the slots, lane-strided, then an xor tree: every block
-//     gets the same bits.  False when a wait ran out (every wait is bounded).
-// With ORDER whatever a block wrote before it published is visible after the gather.  Without, no fence is paid
-// for (one costs half a microsecond to a microsecond behind a product): the counter is only the sign that
-// looking is worth while, the rounds in the slots tell whether a value is there.  Polling the one counter and
-// reading the slots once beats polling the slots (152 blocks, nothing else to do: 1.9 against 3.5 to 4.9 us;
-// many lines, written by stores and polled by all, against one atomic).  An FP64 instruction occupies its
-// quarter of the SM for 64 cycles however few lanes need it, so the block's sum is spread over one warp in each
-// quarter (eight adds, a tree, three adds), not a tree in every warp.  Two sets of slots take turns: a block
-// writes round + 2 only after all published round + 1, hence have read `round`.
+// Sums over the grid, each a grid-wide barrier too, in two halves so that a block can work in between.  The sums'
+// number in the launch is `round` = 1, 2, ...  A block's partial sums (one for its partition, or one for each vector
+// block it stands in for) go into slots with the round in them, and one more onto the counter; a gather waits for the
+// counter, then adds the slots, lane-strided, then an xor tree: every block gets the same bits.  No fence is paid for
+// (one costs half a microsecond to a microsecond behind a product): the counter is only the sign that looking is
+// worth while, the rounds in the slots tell whether a value is there.  Polling the one counter and reading the slots
+// once beats polling the slots (152 blocks, nothing else to do: 1.9 against 3.5 to 4.9 us; many lines, written by
+// stores and polled by all, against one atomic).  A slot is written again an iteration later, when a sum of another
+// kind has been gathered since, to which every block added after it had read the slot.
+//
+// An FP64 instruction occupies its quarter of the SM for 64 cycles however few lanes need it, so a block's lane trees
+// are not made by every warp (five adds each, eight warps a quarter) but by one warp in each quarter for eight warps'
+// terms at once (nine adds), from shared memory.  Terms lie there as they do in a warp, lane l of warp w at
+// term_at(w, l): four threads that read a row, and the four rows beside it, touch all banks.
 constexpr int kSumWarps = 4;
-template <bool ORDER>
-__device__ __forceinline__ void publish_sum(const SyncArgs& g, int round, double* red) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bd = blockDim.x;
-  const int sw = min(kSumWarps, bd >> 5);
-  double v = red[tid];
-  for (int i = tid + 32 * sw; i < bd; i += 32 * sw) v += red[i];
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
-  if (sw > 1) {  // every term has been read before the warps' sums take their place
-    asm volatile("bar.sync 1, %0;" ::"r"(32 * sw) : "memory");
-    if (lane == 0) red[warp] = v;
-    asm volatile("bar.sync 1, %0;" ::"r"(32 * sw) : "memory");
-    if (warp > 0) return;
-    v = red[0] + red[1];
-    if (sw > 2) v += sw > 3 ? red[2] + red[3] : red[2];
-  }
-  if (lane == 0) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(v), tag = (unsigned long long)round << 32;
-    if (ORDER) fence_acq_rel();
-    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(&g.m->slot[round & 1][blockIdx.x]),
-                 "l"(tag | (bits & 0xffffffffull)), "l"(tag | (bits >> 32))
-                 : "memory");
-    asm volatile("red.relaxed.gpu.global.add.s32 [%0], 1;" ::"l"(&g.m->summed) : "memory");
+__device__ __forceinline__ int term_at(int w, int l) { return 32 * w + ((l + 4 * w) & 31); }
+
+// sums[w] = the xor tree's sum of warp w's terms, w < count, by the block's first kSumWarps warps (all that there are)
+__device__ __forceinline__ void tree_sums(const double* red, int count, double* sums) {
+  const int tid = threadIdx.x, j = tid & 3, threads = min(32 * kSumWarps, (int)blockDim.x);
+  for (int w0 = 0; w0 < count; w0 += threads / 4) {
+    const int w = w0 + (tid >> 2);
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    if (w < count)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) a[k] = red[term_at(w, j + 4 * k)] + red[term_at(w, j + 4 * k + 16)];
+    double v = (a[0] + a[2]) + (a[1] + a[3]);
+    v += __shfl_xor_sync(FULL, v, 2);
+    v += __shfl_xor_sync(FULL, v, 1);
+    if (w < count && j == 0) sums[w] = v;
   }
 }
-template <bool ORDER>
-__device__ __forceinline__ bool gather_sum(const SyncArgs& g, int round, double* sum) {
-  const int lane = threadIdx.x, nb = gridDim.x;
-  const bool ok = lane > 0 || wait_at<false>(g, &g.m->summed, round);
-  if (!__all_sync(FULL, ok)) return false;
-  const Slot* slot = g.m->slot[round & 1];
-  unsigned long long lo[kMaxGrid / 32], hi[kMaxGrid / 32];
-  Patience wait;
-  for (;;) {
-    bool all = true;
-#pragma unroll
-    for (int k = 0; k < kMaxGrid / 32; ++k) {
-      lo[k] = hi[k] = 0;
-      if (lane + 32 * k < nb)
-        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];"
-                     : "=l"(lo[k]), "=l"(hi[k])
-                     : "l"(slot + lane + 32 * k)
-                     : "memory");
-    }
-#pragma unroll
-    for (int k = 0; k < kMaxGrid / 32; ++k)
-      if (lane + 32 * k < nb) all = all && (int)(lo[k] >> 32) == round && (int)(hi[k] >> 32) == round;
-    if (__all_sync(FULL, all)) break;
-    if (__any_sync(FULL, wait.over(g))) {
-      if (lane == 0) give_up(g);
-      return false;
+__device__ __forceinline__ void sum_warps_sync() {
+  const int threads = min(32 * kSumWarps, (int)blockDim.x);
+  asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+}
+__device__ __forceinline__ void put_slot(Slot* slot, int round, double v) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(v), tag = (unsigned long long)round << 32;
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(slot), "l"(tag | (bits & 0xffffffffull)),
+               "l"(tag | (bits >> 32))
+               : "memory");
+}
+__device__ __forceinline__ void count_published(const SyncArgs& g) {
+  asm volatile("red.relaxed.gpu.global.add.s32 [%0], 1;" ::"l"(&g.m->summed) : "memory");
+}
+
+// The block's partial of a partition's sum, by its first kSumWarps warps, after a __syncthreads behind the terms of
+// `warps` warps in red.  The order of the product's fused sum: a tree in each warp, then the warps one after the
+// other.
+static __device__ __noinline__ void publish_part(const SyncArgs& g, int round, int which, const double* red, int warps,
+                                                double* sums) {
+  tree_sums(red, warps, sums);
+  sum_warps_sync();
+  if (threadIdx.x == 0) {
+    double v = 0.0;
+    for (int w = 0; w < warps; ++w) v += sums[w];
+    put_slot(&g.m->part[which][blockIdx.x], round, v);
+    count_published(g);
+  }
+}
+
+// (The helpers from here on are functions of their own that need few registers.  Inlined, or with five slots a lane in
+// flight, they left the product's loop, which the same kernel calls, short of registers: 244 bytes of spills, 45.6 us
+// an iteration at tet 80^3 instead of 35.1.)
+//
+// Sum of `count` slots, by all threads, valid in warp 0.  One thread watches the counter; the slots are then read by
+// as many warps as there are, one slot a lane (vals: shared memory for them, the terms' place: the trees are done).
+// A wait that ran out raises *stop (down before) and gives false.
+static __device__ __noinline__ bool gather_sum(const SyncArgs& g, int round, const Slot* slot, int count, double* vals,
+                                               int* stop, double* sum) {
+  const int tid = threadIdx.x;
+  volatile int* const over = stop;
+  if (tid == 0 && !wait_at<false>(g, &g.m->summed, round)) *over = 1;
+  __syncthreads();
+  if (!*over) {
+#pragma unroll 1
+    for (int i = tid; i < count; i += blockDim.x) {
+      Patience wait;
+      unsigned long long lo, hi;
+      for (;;) {
+        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(slot + i) : "memory");
+        if ((int)(lo >> 32) == round && (int)(hi >> 32) == round) break;
+        if (wait.over(g)) {
+          give_up(g);
+          *over = 1;
+          break;
+        }
+      }
+      vals[i] = __longlong_as_double((long long)((hi << 32) | (lo & 0xffffffffull)));
     }
   }
-  if (ORDER) fence_acq_rel();
+  __syncthreads();
+  if (tid >= 32 || *over) return false;
   double s = 0.0;
-#pragma unroll
-  for (int k = 0; k < kMaxGrid / 32; ++k)
-    s += __longlong_as_double((long long)((hi[k] << 32) | (lo[k] & 0xffffffffull)));
+  for (int i = tid; i < count; i += 32) s += vals[i];
   for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(FULL, s, off);
   *sum = s;
   return true;
 }
 
-// Barrier without a value, in two halves: arrive (one thread, after a __syncthreads that follows the block's writes) and a
-// wait that each warp makes when it first needs the other blocks' writes, usually long after all have arrived.
+// Terms of a partition's sum, in the order of the product's fused sum with `warps` warps: warp w's lanes take the
+// rows of its slices w, w + warps, ... of the processing order.  load(row): the two factors.
+template <typename P, typename F>
+__device__ __forceinline__ void part_terms(const P& pr, int warps, double* red, F&& load) {
+  constexpr int U = 4;  // rows a lane has in flight
+  const int lane = threadIdx.x & 31, lg = pr.tpr_log2, s0 = pr.s0, ns = pr.s1 - s0, rows = pr.rows;
+  const bool lead = (lane & ((1 << lg) - 1)) == 0;
+  for (int w = threadIdx.x >> 5; w < warps; w += blockDim.x >> 5) {
+    double acc = 0.0;
+    for (int t0 = w; t0 < ns; t0 += U * warps) {
+      int row[U];
+      double2 v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int t = t0 + u * warps;
+        row[u] = rows;
+        if (t < ns && lead) {
+          const int sl = pr.tbl ? pr.tbl[checked(t, pr.meta_cap, pr.status)].s : pr.slice_order[s0 + t];
+          row[u] = (sl - s0) * (32 >> lg) + (lane >> lg);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = row[u] < rows ? load(row[u]) : make_double2(0.0, 0.0);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (row[u] < rows) acc = fma(v[u].x, v[u].y, acc);
+    }
+    red[term_at(w, lane)] = acc;
+  }
+}
+
+// 16 bytes of a vector that other blocks have written (ordered by a round), not through L1
+__device__ __forceinline__ void load_vec(const double* p, double (&v)[2]) {
+  asm volatile("ld.relaxed.gpu.global.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void load_vec(const float* p, float (&v)[4]) {
+  asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void load_one(const double* p, double& v) {
+  asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void load_one(const float* p, float& v) {
+  asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+}
+
+// shared memory of the terms, which a gather's values take too
+inline size_t terms_bytes(int threads) { return sizeof(double) * (size_t)std::max(threads, kVecBlocks); }
+
+// vector blocks whose terms are not all zero
+template <typename X>
+__host__ __device__ __forceinline__ int vec_blocks(int64_t n) {
+  const int64_t nv = n / (16 / (int)sizeof(X)), b = (nv + kVecThreads - 1) / kVecThreads;
+  return b < 1 ? 1 : b < kVecBlocks ? (int)b : kVecBlocks;
+}
+
+// The block's partials of r.r over the whole vector (16-byte aligned, in memory, written by all blocks and ordered by a
+// round): the block stands in for the vector blocks blockIdx.x, blockIdx.x + gridDim.x, ... of an update launch and
+// forms the sums that their threads, warps and blocks would.  All threads.
+template <typename X>
+__device__ __noinline__ void publish_vec(const SyncArgs& g, int round, const X* r, int n, double* red, double* sums) {
+  constexpr unsigned NV = 16 / (unsigned)sizeof(X), kStride = kVecBlocks * kVecThreads;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const int active = vec_blocks<X>(n), chunk = max(1, warps / kVecWarps);  // vector blocks at a time
+  const unsigned nv = (unsigned)n / NV;
+  for (int first = blockIdx.x; first < active; first += chunk * gridDim.x) {
+    for (int w = warp; w < chunk * kVecWarps; w += warps) {
+      const int vb = first + (w / kVecWarps) * gridDim.x;
+      double acc = 0.0;
+      if (vb < active) {
+        const unsigned v = (unsigned)vb * kVecThreads + 32 * (w % kVecWarps) + lane;
+#pragma unroll 1
+        for (unsigned j = v; j < nv; j += kStride) {
+          X x[NV];
+          load_vec(r + NV * (size_t)j, x);
+#pragma unroll
+          for (unsigned k = 0; k < NV; ++k) acc = fma((double)x[k], (double)x[k], acc);
+        }
+        if (v < (unsigned)n - nv * NV) {
+          X x;
+          load_one(r + (nv * NV + v), x);
+          acc = fma((double)x, (double)x, acc);
+        }
+      }
+      red[term_at(w, lane)] = acc;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32 * kSumWarps) {
+      tree_sums(red, chunk * kVecWarps, sums);
+      sum_warps_sync();
+      const int vb = first + threadIdx.x * gridDim.x;
+      if (threadIdx.x < chunk && vb < active) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < kVecWarps; ++k) s += sums[kVecWarps * threadIdx.x + k];
+        put_slot(&g.m->vec[vb], round, s);
+      }
+    }
+    if (first + chunk * gridDim.x < active) __syncthreads();  // the terms have been read
+  }
+  __syncwarp();
+  if (threadIdx.x == 0) count_published(g);
+}
+
+// Barrier without a value, in two halves: arrive (one thread, after a __syncthreads that follows the block's writes)
+// and a wait that each warp makes when it first needs the other blocks' writes, usually long after all have arrived.
 // round: 1, 2, ... within the launch.  seen: the last round this block knows to be complete, in shared memory.
 __device__ __forceinline__ void arrive(const SyncArgs& g) {
   asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(&g.m->arrived) : "memory");
@@ -195,6 +347,14 @@ __device__ __forceinline__ bool wait_round(const SyncArgs& g, int round, int* se
     asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_addr(seen)), "r"(now) : "memory");
   }
   __syncwarp();
+  return ok;
+}
+
+// the same by one thread for its whole block, which a __syncthreads has to follow
+__device__ __forceinline__ bool wait_block(const SyncArgs& g, int round, int* seen) {
+  const bool ok = wait_at<true>(g, &g.m->arrived, round);
+  const int now = ok ? round : -1;
+  asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_addr(seen)), "r"(now) : "memory");
   return ok;
 }
 
@@ -288,7 +448,8 @@ __device__ __noinline__ void stage_halo(Product<V, X>* pr, const SyncArgs* sync,
     int c[4];
     X v[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) c[u] = j0 + u * bd < nh ? (int)checked((int64_t)pr->halo[j0 + u * bd], pr->n_x, pr->status) : 0;
+    for (int u = 0; u < 4; ++u)
+      c[u] = j0 + u * bd < nh ? (int)checked((int64_t)pr->halo[j0 + u * bd], pr->n_x, pr->status) : 0;
 #pragma unroll
     for (int u = 0; u < 4; ++u) v[u] = j0 + u * bd < nh ? load_x(pr->xg + c[u]) : X(0);
 #pragma unroll
