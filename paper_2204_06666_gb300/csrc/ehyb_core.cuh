@@ -782,7 +782,9 @@ __device__ __forceinline__ bool partition_spmv(const KArgs& a, const V* __restri
     if (WIDE) {
       part = s < 0 ? -1 - s : a.slice_wide[s];
       halo_wide = part >= 0 && a.row_cin;
-      if (!halo_wide) {  // a slice's first chunks (a unit holds at most one chunk)
+      // a slice's first chunks (a unit holds at most one chunk).  In er_layout 2 a slice holds both parts of its rows: one
+      // without a wide part has up to two chunks of slots and is one chain over all of them
+      if (!a.row_cin) {
         w = min(w, kWideCap);
         we = min(we, kWideCap);
       }
