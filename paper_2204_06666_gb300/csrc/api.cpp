@@ -151,6 +151,16 @@ ehyb_status_t device_query(int* dev, int* sms, int* smem_optin) {
 }
 ehyb_status_t device_alloc(void** p, size_t bytes) { return dev_alloc(p, bytes); }
 
+bool uneven_rows(const HostPlan& H) {
+  int64_t longest = 0, entries = 0;
+  for (size_t r = 0; r < (size_t)H.n; ++r) {
+    const int64_t k = (int64_t)H.row_ell_count[r] + H.row_er_count[r];
+    longest = std::max(longest, k);
+    entries += k;
+  }
+  return longest * H.n >= kUneven * entries;
+}
+
 WideLists wide_lists(int32_t nparts, const std::vector<int32_t>& slice_ptr, const std::vector<int64_t>& slice_pos,
                      const std::vector<int64_t>& er_slice_pos) {
   WideLists L;
@@ -480,7 +490,9 @@ ehyb_status_t plan_finalize(std::unique_ptr<ehyb_plan_s>& P, const ehyb_options_
   D.er_tpr = P->er_tpr;
   WideLists W;
   try {
-    if (H.er_layout == 0) {
+    if (!uneven_rows(H)) {
+      // every slice stays one chain
+    } else if (H.er_layout == 0) {
       W = wide_lists(H.nparts, H.slice_ptr, H.slice_pos, H.er_slice_pos);
     } else if (H.er_layout == 2 && H.tpr == 1) {  // flags only: these slices hold both parts of a row in one
       for (int64_t r = 0; r < n; ++r)

@@ -6,8 +6,8 @@
 namespace ehyb {
 
 // Chunk of a lane's slots that one chain of FMAs sums, in the slab and in the extra rows of a slice alike
-// (ehyb_core.cuh, wide slices).  A multiple of 4, so that a chunk of the copies in runs of four starts on a run;
-// above 81, so that the rows of 3D elasticity stay one chain.
+// (ehyb_core.cuh, wide slices), in plans with uneven rows (uneven_rows in plan_internal.h).  A multiple of 4, so that a
+// chunk of the copies in runs of four starts on a run.
 constexpr int kWideCap = 96;
 struct WideUnit {  // one later chunk of a wide slice
   int64_t pos;     // its first slot in the slab (er 0) or extra-row (er 1) arrays
@@ -63,7 +63,7 @@ struct DevPlan {
   const uint16_t* ell_col_low = nullptr;
   const int32_t* er_scol_low = nullptr;
   const int32_t* er_scol_old_low = nullptr;
-  // wide slices (wide_parts > 0; wide_lists in plan.h): part of each slice or -1, units and wide slices by
+  // wide slices (wide_parts > 0; wide_lists in plan_internal.h): part of each slice or -1, units and wide slices by
   // partition, workspace of the partial sums.  er_layout 2: a flag per slice and the entry counts of each row
   int32_t wide_parts = 0;
   const int32_t* slice_wide = nullptr;

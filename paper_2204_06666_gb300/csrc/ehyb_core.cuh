@@ -442,16 +442,16 @@ __device__ __forceinline__ X er_dot_runs(const V* __restrict__ vb, const int32_t
   return acc;
 }
 
-// ---- wide slices.  A lane sums its slots one after the other, so a slice with a row of thousands of entries was
-// one chain of dependent loads and FMAs thousands of slots long while the other warps had nothing left to do
-// (power-law matrix, 200k rows, longest slice 3,299 slots a lane: 442 us for 2 M entries, 100 us now; what is left is
-// the block with the most padded slots, 7,706 a warp lane at about 20 cycles each).  The slots of a slice
-// are therefore summed in chunks of kWideCap a lane: acc0 = the first kWideCap slab slots, then the first
-// kWideCap extra-row slots, as one chain; every later chunk of the slab, then of the extra rows, is a chain of
-// its own (one unit of work, taken by any warp of the block); the row is acc0 + ((c1 + c2) + c3 ...).  A slice of
-// at most kWideCap slots in each part has no later chunk and keeps its single chain, so 81-entry elasticity
-// rows and narrower ones are summed as before.  Every path sums in this order (the products, the batch, SpMM,
-// the shards and er_layout 2), so their results stay equal bit for bit.
+// ---- wide slices.  A lane sums its slots one after the other, so a slice with a row of thousands of entries was one
+// chain of dependent loads and FMAs thousands of slots long while the other warps had nothing left to do (power-law
+// matrix, 200k rows, longest slice 3,299 slots a lane: 442 us for 2 M entries, 100 to 118 us now; what is left is the
+// block with the most padded slots, 7,706 a warp lane at about 20 cycles each).  Where a plan's rows are that uneven
+// (uneven_rows in plan_internal.h) the slots of a slice are summed in chunks of kWideCap a lane: acc0 = the first
+// kWideCap slab slots, then the first kWideCap extra-row slots, as one chain; every later chunk of the slab, then of
+// the extra rows, is a chain of its own (one unit of work, taken by any warp of the block); the row is
+// acc0 + ((c1 + c2) + c3 ...).  A slice of at most kWideCap slots in each part has no later chunk and keeps its single
+// chain, and so do all slices of a plan whose rows are alike.  Every path sums in this order (the products, the batch,
+// SpMM, the shards and er_layout 2), so their results stay equal bit for bit.
 
 struct KArgs {
   int32_t tpr_log2, er_tpr_log2;
@@ -482,7 +482,7 @@ struct KArgs {
   int32_t* dot_arrive;    // optional (with dot_part, one block per partition): arrival counter; the last
   double* dot_result;     //   block reduces the partials into *dot_result and resets the counter
   const int32_t* skip;    // optional: the launch does nothing while *skip != 0 (converged solver)
-  // wide slices (WIDE kernels; see wide_cap): a wide slice's part index or -1, the units and the wide slices of
+  // wide slices (WIDE kernels; see kWideCap): a wide slice's part index or -1, the units and the wide slices of
   // each partition, and the workspace of the parts' partial sums (32 lanes each, 8 bytes apart)
   const int32_t* slice_wide;
   const int32_t* unit_ptr;
@@ -490,7 +490,7 @@ struct KArgs {
   const int32_t* wide_ptr;
   const WideSlice* wides;
   double* wide_ws;
-  int32_t wide_parts;     // parts in the workspace (checked build only)
+  int32_t wide_parts;     // parts in the workspace; 0: every slice is one chain
   const int32_t* row_cin;   // er_layout 2 with one lane per row: slab / extra entries of each row (else null)
   const int32_t* row_cer;
   const uint16_t* er_hcol;  // staged extra rows (HER kernels; halo_* lists their columns): 16-bit columns, else null

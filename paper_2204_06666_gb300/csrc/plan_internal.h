@@ -27,8 +27,9 @@ ehyb_status_t device_alloc(void** p, size_t bytes);
 }  // namespace ehyb
 
 namespace ehyb {
-// Wide slices of a sliced layout (er_layout 0): slices with more than kWideCap slab or extra-row slots per lane,
-// their later chunks as units by partition (longest first), and the numbering of the parts' partial sums.
+// Wide slices of a sliced layout (er_layout 0) with uneven rows: slices with more than kWideCap slab or extra-row
+// slots per lane, their later chunks as units by partition (longest first), and the numbering of the parts' partial
+// sums.
 struct WideLists {
   int32_t parts = 0;
   std::vector<int32_t> slice_wide, unit_ptr, wide_ptr;
@@ -48,6 +49,18 @@ struct LowHalo {
 };
 // false (and out empty): a partition's rows and columns exceed max_stage or 2^16, or too little is shared
 bool low_halo(const HostPlan& H, int64_t max_stage, int threads, LowHalo& out);
+
+// Whether wide slices are summed in chunks at all: where the longest row has kUneven times the mean row's entries.
+// Chunks give the other warps of a block something to do while one slice's chain runs.  Where all rows are long
+// (quadratic elements, 243 entries a row) every warp has such a slice, and chunks only cost: the partial sums' way
+// through the workspace, and the deeper batches, staged extra rows, small-plan kernel, cooperative solvers and batch
+// shares that chunked plans go without (us, chunks -> one chain; 125-point stencil on 50^3 nodes: FP64 49.7 -> 37.2,
+// FP32 34.6 -> 22.1, BF16 32.6 -> 18.8; 375 entries a row, 24k rows: FP64 30.7 -> 34.8, k = 8 SpMM 355 -> 258,
+// er_layout 2 101 -> 44, three in a batch 428 -> 169, CG 1.25 -> 1.36 ms).  Grids and meshes have ratios of 1.1 to
+// 1.5, power-law matrices with a slice above 96 slots 18 to several hundred, so the line can lie anywhere between.
+// Rows, not slices, decide, so that both layouts of one matrix sum alike.
+constexpr int64_t kUneven = 4;
+bool uneven_rows(const HostPlan& H);
 
 WideLists wide_lists(int32_t nparts, const std::vector<int32_t>& slice_ptr, const std::vector<int64_t>& slice_pos,
                      const std::vector<int64_t>& er_slice_pos);

@@ -284,7 +284,8 @@ ehyb_status_t ehyb_shard_create(ehyb_plan_t plan, int32_t nranks, int32_t rank, 
   }
   WideLists W;
   try {
-    W = wide_lists(D.nparts, S->slice_ptr, S->slice_pos, S->er_slice_pos);
+    if (PD.wide_parts > 0)  // the plan's sums run in chunks: its slices here do too
+      W = wide_lists(D.nparts, S->slice_ptr, S->slice_pos, S->er_slice_pos);
   } catch (const std::bad_alloc&) {
     return EHYB_ERR_OOM;
   }

@@ -124,9 +124,10 @@ __global__ void __launch_bounds__(512) spmm_kernel(KArgs a, const double* __rest
         for (int j = 0; j < KC; ++j) q[j] = fma(v, xr.v[j], q[j]);
       }
     };
-    slab(0, min(w, kWideCap), acc);
-    extra(0, min(we, kWideCap), acc);
-    if (w > kWideCap || we > kWideCap) {  // a wide slice's later chunks, summed as the SpMV sums them
+    const int cap = a.wide_parts > 0 ? kWideCap : 0x7fffffff;
+    slab(0, min(w, cap), acc);
+    extra(0, min(we, cap), acc);
+    if (w > cap || we > cap) {  // a wide slice's later chunks, summed as the SpMV sums them
       double t[KC];
 #pragma unroll
       for (int j = 0; j < KC; ++j) t[j] = 0.0;
