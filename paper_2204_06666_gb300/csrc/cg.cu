@@ -520,6 +520,7 @@ __global__ void __launch_bounds__(MAXT, 1) cg_persist_kernel(core::KArgs a, cons
   using namespace core;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ CgBlock<V, X> sh;
+  static_assert(sizeof(sh) <= persist::kMaxStatic, "static shared memory");
   X* const ps = reinterpret_cast<X*>(smem_raw);
   const int bd = blockDim.x;
   if (c.st->done) return;  // uniform over the grid: nobody writes it before every block has met the others
@@ -739,7 +740,7 @@ ehyb_status_t launch_persist(ehyb_plan_t P, const V* ev, const V* erv, CgPersist
   a.smem_elems = (int64_t)(smem / sizeof(X));
   const size_t tbl = al((size_t)D.max_part_slices * sizeof(core::SliceMeta));
   const size_t vec = al((size_t)D.max_part_rows * sizeof(X));
-  const size_t budget = std::min((size_t)optin - 1024, persist::shared_budget(smem + persist::terms_bytes(D.threads)));
+  const size_t budget = std::min((size_t)(optin - persist::kMaxStatic), persist::shared_budget(smem + persist::terms_bytes(D.threads)));
   auto place = [&](size_t bytes) -> int32_t {
     if (smem + bytes > budget) return -1;
     const size_t o = smem;
@@ -753,7 +754,7 @@ ehyb_status_t launch_persist(ehyb_plan_t P, const V* ev, const V* erv, CgPersist
   c.q_off = place(vec);
   c.r_off = place(vec);
   c.x_off = place(vec);
-  CKC(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
+  CKC(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - persist::kMaxStatic));
   CKC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, D.threads, smem));
   *ran = D.nparts <= sms * resident && D.nparts <= persist::kMaxGrid;
   if (!*ran) return EHYB_OK;

@@ -617,6 +617,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_persist_kernel(core::KArgs a, con
   constexpr int KG = (kRunsG ? 16 : 8) * (1024 / MAXT);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ PcgBlock<VA, XA, VG, XG> sh;
+  static_assert(sizeof(sh) <= persist::kMaxStatic, "static shared memory");
   XA* const ps = reinterpret_cast<XA*>(smem_raw);
   const int bd = blockDim.x;
   if (c.st->done) return;  // uniform over the grid: nobody writes it before every block has met the others
@@ -865,7 +866,7 @@ ehyb_status_t launch_persist(ehyb_precond_t M, const VA* av, const VA* aev, cons
   const size_t terms = persist::terms_bytes(std::max(D.threads, G.threads));
   c.g_warps = G.threads / 32;
   const size_t budget =
-      std::min((size_t)optin - 1024, persist::shared_budget(smem + al(vg) + terms));
+      std::min((size_t)(optin - persist::kMaxStatic), persist::shared_budget(smem + al(vg) + terms));
   auto place = [&](size_t bytes) -> int32_t {
     if (smem + al(bytes) > budget) return -1;
     const size_t o = smem;
@@ -889,7 +890,7 @@ ehyb_status_t launch_persist(ehyb_precond_t M, const VA* av, const VA* aev, cons
     c.h_off = most > 0 ? place((size_t)most * sizeof(float)) : -1;
   }
   c.x_off = place(va);
-  CKP(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
+  CKP(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - persist::kMaxStatic));
   CKP(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, D.threads, smem));
   *ran = D.nparts <= sms * resident;
   if (!*ran) return EHYB_OK;

@@ -65,6 +65,11 @@ struct SyncArgs {
 // 64^3 (41 KB a vector) the FP64 PCG took 23.1 ms a solve with five vectors in shared memory (215 KB), 9.5 with two
 // (separate launches 9.8); scalar hexahedra 80^3 with BF16 G 3.0 and 1.9 ms (2.4).  0: more than 196 KB, where
 // the separate launches are the faster form (tet 126^3, FP64 G, two vectors of 105 KB: 4.9 ms against 3.9).
+//
+// The budget only decides what is placed.  What a kernel may be launched with is a property of its instantiation, shared
+// by every plan and host thread, so it is always set to the device's limit: a smaller plan's budget set there would
+// refuse the launch of a larger one that another thread is about to make.  (A launch's own size decides L1's share.)
+constexpr int kMaxStatic = 2048;  // static shared memory of a persistent kernel
 inline size_t shared_budget(size_t must) {
   for (size_t kb : {100, 132, 164, 196})
     if (must + 3072 <= kb * 1024) return kb * 1024 - 3072;
