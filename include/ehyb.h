@@ -82,8 +82,11 @@ typedef struct {
   int32_t num_sms;           /* P of Eq. 1 for host-only plans; 0 = query the current device */
   int32_t smem_budget;       /* SHM^max of Eq. 1 in bytes per block; 0 = device opt-in maximum - 1024 */
   const int32_t* part_vec;   /* optional PartVec (one partition id >= 0 per row); NULL = in-house partitioner */
-  int64_t wait_timeout_ns;   /* bound on each device-side wait; 0 = 1e9 (one second) */
-  int32_t inject_wait_fault; /* test hook: the staging wait waits for a copy that is never issued */
+  int64_t wait_timeout_ns;   /* bound on each device-side wait; 0 = 1e9 (one second).  Below 1e8 the solvers iterate
+                                in separate launches, which wait for no other block */
+  int32_t inject_wait_fault; /* test hook: 1 = the staging wait waits for a copy that is never issued; 2 / 3 = the
+                                blocks of a solver's cooperative kernel wait for one more at their sums / at the
+                                hand-over of a vector */
   int32_t keep_host;         /* keep host copies of the plan arrays (ehyb_plan_export without device reads) */
   uint64_t seed;             /* seed of the multilevel partitioner's matching order (partitioner 1); the plan is a
                                 deterministic function of the matrix, the options and this seed */

@@ -717,8 +717,8 @@ ehyb_status_t run_chunk(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s) {
 // One persistent launch of at most kPersistSteps iterations; *ran = false (and nothing launched) for a plan that
 // needs the separate launches: more partitions than SMs (a block owns one partition, all blocks resident), a wide
 // slice (its sums go through the plan's workspace), more shared memory than persist::shared_budget grants, more rows
-// a partition than persist::even_enough or, with FP32 vectors, kMaxRowsF32 / kMaxRowsBf16 allow, the staging-fault
-// test hook.
+// a partition than persist::even_enough or, with FP32 vectors, kMaxRowsF32 / kMaxRowsBf16 allow, a time
+// limit below kMinLimitNs, the staging-fault test hook.
 constexpr int kPersistSteps = 2000;  // bounds one launch to a fraction of a second
 
 template <typename V, typename X, int KB, bool RUNS, int MAXT>
@@ -758,7 +758,7 @@ ehyb_status_t launch_persist(ehyb_plan_t P, const V* ev, const V* erv, CgPersist
   CKC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, D.threads, smem));
   *ran = D.nparts <= sms * resident && D.nparts <= persist::kMaxGrid;
   if (!*ran) return EHYB_OK;
-  CKC(cudaMemsetAsync(c.sync.m, 0, sizeof(persist::Meeting), s));
+  CKC(persist::clear_meeting(c.sync.m, D.inject_wait_fault, s));
   void* args[] = {&a, (void*)&ev, (void*)&erv, &c};
   CKC(cudaLaunchCooperativeKernel((const void*)kernel, dim3((unsigned)D.nparts), dim3((unsigned)D.threads), args, smem,
                                   s));
@@ -768,8 +768,10 @@ ehyb_status_t launch_persist(ehyb_plan_t P, const V* ev, const V* erv, CgPersist
 ehyb_status_t run_persist(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s, bool* ran) {
   const DevPlan& D = P->dev;
   *ran = false;
-  if (D.wide_parts > 0 || D.inject_wait_fault || D.nparts > persist::kMaxGrid) return EHYB_OK;
-  const persist::SyncArgs sync{w->meeting, D.status, &w->st->done, std::max(D.wait_timeout_ns, persist::kMinLimitNs)};
+  if (D.wide_parts > 0 || D.inject_wait_fault == 1 || D.wait_timeout_ns < persist::kMinLimitNs ||
+      D.nparts > persist::kMaxGrid)
+    return EHYB_OK;
+  const persist::SyncArgs sync{w->meeting, D.status, &w->st->done, D.wait_timeout_ns};
   if (lowp == 0) {
     const CgPersist<double> c{w->xp, w->r, w->p, w->q, -1, -1, -1, -1, -1, kPersistSteps, w->st, w->hist, sync};
     if (D.threads <= 512) return launch_persist<double, double, 16, false, 512>(P, D.ell_val, D.er_sval, c, s, ran);

@@ -1072,7 +1072,7 @@ inline KArgs make_kargs(const DevPlan& P) {
   a.halo_old = halo ? P.halo_old : nullptr;
   a.status = P.status;
   a.timeout_ns = P.wait_timeout_ns;
-  a.inject = P.inject_wait_fault;
+  a.inject = P.inject_wait_fault == 1;
   a.dot_part = nullptr;
   a.dot_self = 0;
   a.dot_arrive = nullptr;

@@ -831,7 +831,7 @@ ehyb_status_t enqueue_chunk32(ehyb_precond_t M, PcgWork* w, cudaStream_t s) {
 // One persistent launch of at most kPersistSteps iterations; *ran = false (and nothing launched) where the separate
 // launches are needed: more partitions than SMs, a wide slice, copies not in runs of four, more shared memory than
 // persist::shared_budget grants, more rows a partition than persist::even_enough (FP64 vectors, low-precision G) or
-// kMaxRowsPcg32 (FP32 vectors) allow, the staging-fault test hook.
+// kMaxRowsPcg32 (FP32 vectors) allow, a time limit below kMinLimitNs, the staging-fault test hook.
 constexpr int kPersistSteps = 2000;  // bounds one launch to a fraction of a second
 
 template <typename VA, typename XA, int KA, typename VG, typename XG, int MAXT>
@@ -894,7 +894,7 @@ ehyb_status_t launch_persist(ehyb_precond_t M, const VA* av, const VA* aev, cons
   CKP(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, D.threads, smem));
   *ran = D.nparts <= sms * resident;
   if (!*ran) return EHYB_OK;
-  CKP(cudaMemsetAsync(c.sync.m, 0, sizeof(persist::Meeting), s));
+  CKP(persist::clear_meeting(c.sync.m, D.inject_wait_fault, s));
   void* args[] = {&a, (void*)&av, (void*)&aev, &g, (void*)&gv, (void*)&gev, &h, (void*)&hv, (void*)&hev, &c};
   CKP(cudaLaunchCooperativeKernel((const void*)kernel, dim3((unsigned)D.nparts), dim3((unsigned)D.threads), args, smem,
                                   s));
@@ -905,14 +905,15 @@ ehyb_status_t run_persist(ehyb_precond_t M, PcgWork* w, cudaStream_t s, bool inn
   const ehyb_plan_t P = M->plan;
   const DevPlan &D = P->dev, &G = M->g->dev, &H = M->gt->dev;
   *ran = false;
-  if (D.nparts > persist::kMaxGrid || D.wide_parts > 0 || G.wide_parts > 0 || H.wide_parts > 0 || D.inject_wait_fault ||
-      D.er_layout != 0 || G.er_layout != 0 || H.er_layout != 0)
+  if (D.nparts > persist::kMaxGrid || D.wide_parts > 0 || G.wide_parts > 0 || H.wide_parts > 0 ||
+      D.inject_wait_fault == 1 || D.wait_timeout_ns < persist::kMinLimitNs || D.er_layout != 0 ||
+      G.er_layout != 0 || H.er_layout != 0)
     return EHYB_OK;
   // the three plans own the same rows block by block
   if (M->g->host.part_ptr != P->host.part_ptr || M->gt->host.part_ptr != P->host.part_ptr) return EHYB_OK;
   if (M->lowp && (G.lowp_group != 4 || H.lowp_group != 4)) return EHYB_OK;
   if (inner32 && (D.lowp_group != 4 || D.max_part_rows > persist::kMaxRowsPcg32)) return EHYB_OK;
-  const persist::SyncArgs sync{w->meeting, D.status, &w->st->done, std::max(D.wait_timeout_ns, persist::kMinLimitNs)};
+  const persist::SyncArgs sync{w->meeting, D.status, &w->st->done, D.wait_timeout_ns};
   const bool half = D.threads <= 512;
   auto with_g = [&](auto va, const auto* av, const auto* aev, auto c, auto ka, auto mt) -> ehyb_status_t {
     using VA = decltype(va);

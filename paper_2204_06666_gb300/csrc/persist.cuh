@@ -27,7 +27,10 @@ namespace persist {
 using namespace core;
 
 constexpr int kMaxGrid = 160;      // blocks of a persistent launch (five partial sums per gathering lane)
-constexpr uint64_t kMinLimitNs = 2000000000ull;  // least time limit of a wait for the other blocks
+// Least time limit (wait_timeout_ns) with which solvers iterate persistently: the others' work, or another process's time
+// slice, may keep a block waiting for milliseconds.  Plans with a shorter one take the separate launches, which have no
+// such waits.
+constexpr uint64_t kMinLimitNs = 100000000ull;
 constexpr int kAborted = 2;
 
 // Grid of the vector kernels of the separate launches.  Their inner products add a vector's squares in the order of
@@ -54,7 +57,7 @@ struct Meeting {
 struct SyncArgs {
   Meeting* m;
   int32_t* status;            // the plan's status word: EHYB_ERR_TIMEOUT when a wait ran out
-  int32_t* done;              // set to kAborted with it, so that the host stops launching
+  int32_t* done;              // set to kAborted with it, so that the other blocks give up and the host stops launching
   uint64_t limit_ns;
 };
 
@@ -94,6 +97,15 @@ constexpr int kMaxRowsF32 = 5500, kMaxRowsBf16 = 4500, kMaxRowsPcg32 = 8192;
 inline bool even_enough(int max_rows, int64_t n, int sms, int spare) { return max_rows - n / sms <= spare; }
 constexpr int kSpare64 = 3500, kSpare32 = 2500, kSparePcg = 4500;
 
+// The meeting place of a launch, zeroed.  Test hook (inject_wait_fault 2 / 3): one arrival at the sums / the plain rounds
+// never happens, so that the first wait there runs out.
+inline cudaError_t clear_meeting(Meeting* m, int inject, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(m, 0, sizeof(Meeting), s);
+  if (e == cudaSuccess && inject >= 2)
+    e = cudaMemsetAsync(inject == 2 ? &m->summed : &m->arrived, 0xff, sizeof(int32_t), s);
+  return e;
+}
+
 // a wait that has lasted: true when it must give up (its limit is over, or another block gave up)
 struct Patience {
   uint64_t t0 = 0;
@@ -102,7 +114,7 @@ struct Patience {
     if ((++spins & 63) != 0) return false;
     const uint64_t t = globaltimer_ns();
     if (t0 == 0) t0 = t;
-    return t - t0 > g.limit_ns || *(volatile int32_t*)g.status == kTimeoutCode;
+    return t - t0 > g.limit_ns || *(volatile int32_t*)g.done == kAborted;
   }
 };
 __device__ __forceinline__ void give_up(const SyncArgs& g) {
