@@ -465,7 +465,8 @@ ehyb_status_t ehyb_batch_create(int32_t count, const ehyb_plan_t* plans, ehyb_ba
  * `stream`: ONE persistent launch whose blocks pull (plan, partition) tiles from a shared queue, each
  * tile gathering its slice of x through its plan's permutation as it stages it.  Results equal
  * ehyb_spmv on each plan bit for bit.  Uses the plans' workspaces: do not overlap with other calls on
- * the same plans.  xs / ys are host arrays of `count` device pointers.
+ * the same plans.  xs / ys are host arrays of `count` device pointers.  EHYB_ERR_CUDA on a stream that is being
+ * captured (the pointers go to the device beside the launch); the capture stays valid.
  */
 ehyb_status_t ehyb_batch_spmv(ehyb_batch_t batch, const double* const* xs, double* const* ys, void* stream);
 

@@ -245,6 +245,12 @@ extern "C" ehyb_status_t ehyb_batch_create(int32_t count, const ehyb_plan_t* pla
 extern "C" ehyb_status_t ehyb_batch_spmv(ehyb_batch_t b, const double* const* xs, double* const* ys, void* stream) {
   if (!b || !xs || !ys) return EHYB_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
+  // A captured call would only record the table's copy: later calls with the same pointers would launch without it, and
+  // a replay after a call with other pointers would use those.
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  CKB(cudaStreamIsCapturing(s, &capture));
+  if (capture != cudaStreamCaptureStatusNone)
+    return cuda_error_status(cudaErrorStreamCaptureUnsupported, "ehyb_batch_spmv on a capturing stream");
   bool changed = false;
   for (int i = 0; i < b->count; ++i) {
     if (b->table[(size_t)i].n > 0 && (!xs[i] || !ys[i] || (const void*)xs[i] == (const void*)ys[i]))
