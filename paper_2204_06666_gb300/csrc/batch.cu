@@ -114,6 +114,7 @@ struct ehyb_batch_s {
   int ntiles = 0, nunits = 0, grid = 0, threads = 512;  // partitions, work units
   size_t smem = 0;
   int64_t max_n = 0;
+  bool dirty = true;  // the pointers in `table` are not (known to be) on the device
 };
 
 #define CKB(call)                                                     \
@@ -245,26 +246,27 @@ extern "C" ehyb_status_t ehyb_batch_create(int32_t count, const ehyb_plan_t* pla
 extern "C" ehyb_status_t ehyb_batch_spmv(ehyb_batch_t b, const double* const* xs, double* const* ys, void* stream) {
   if (!b || !xs || !ys) return EHYB_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
+  for (int i = 0; i < b->count; ++i)
+    if (b->table[(size_t)i].n > 0 && (!xs[i] || !ys[i] || (const void*)xs[i] == (const void*)ys[i]))
+      return EHYB_ERR_INVALID_ARG;
   // A captured call would only record the table's copy: later calls with the same pointers would launch without it, and
   // a replay after a call with other pointers would use those.
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   CKB(cudaStreamIsCapturing(s, &capture));
   if (capture != cudaStreamCaptureStatusNone)
     return cuda_error_status(cudaErrorStreamCaptureUnsupported, "ehyb_batch_spmv on a capturing stream");
-  bool changed = false;
   for (int i = 0; i < b->count; ++i) {
-    if (b->table[(size_t)i].n > 0 && (!xs[i] || !ys[i] || (const void*)xs[i] == (const void*)ys[i]))
-      return EHYB_ERR_INVALID_ARG;
     if (xs[i] != b->xs[(size_t)i] || ys[i] != b->ys[(size_t)i]) {
       b->xs[(size_t)i] = xs[i];
       b->ys[(size_t)i] = ys[i];
       b->table[(size_t)i].x = xs[i];
       b->table[(size_t)i].y = ys[i];
-      changed = true;
+      b->dirty = true;
     }
   }
-  if (changed)
+  if (b->dirty)
     CKB(cudaMemcpyAsync(b->d_table, b->table.data(), (size_t)b->count * sizeof(BatchPlan), cudaMemcpyHostToDevice, s));
+  b->dirty = false;
   if (b->ntiles == 0) return EHYB_OK;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)b->grid);

@@ -1,4 +1,5 @@
-"""GPU: a batch refuses a stream that is being captured, leaves the capture as it was, and works afterwards."""
+"""GPU: a batch refuses a stream that is being captured, leaves the capture as it was, and works afterwards; a refused
+call leaves none of its pointers behind."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -33,3 +34,17 @@ def test_capture_is_refused(called_before):
     g.replay()
     assert torch.equal(other, refs[0])
 
+
+def test_refused_pointers_do_not_stay():
+    import paper_2204_06666_gb300 as eh
+    mats = [gen.tet_lap3d(N=n) for n in (8, 12)]
+    plans = [eh.Plan(A) for A in mats]
+    B = eh.Batch(plans)
+    xs = [torch.from_numpy(gen.uniform(A.n, 3 + i)).cuda() for i, A in enumerate(mats)]
+    ys = [torch.zeros_like(x) for x in xs]
+    B.spmv(xs, ys)
+    first = [torch.zeros_like(xs[0]), ys[1]]
+    with pytest.raises(eh.EhybError):
+        B.spmv(xs, [first[0], xs[1]])    # x and y of the second are one array
+    B.spmv(xs, first)
+    assert torch.equal(first[0], ys[0])
