@@ -33,27 +33,30 @@ struct BatchPlan {
   int32_t kbatch;   // the plan's batch depth (6 on wide slices, else 8)
 };
 
-// A partition worth more than 1 / kShare of a resident block's share of the batch is split into units that
-// each take every nsub-th slice of its processing order (and stage the whole slice of x again, which costs about
-// kStageCost slots a row, from L2).  With whole partitions as units, a batch with fewer large partitions than
-// resident blocks took as long as its largest one: 24 matrices of 5k to 100k rows on 304 blocks, about 50 partitions
-// of up to 640k entries, 272 us; 91 us in shares (launched directly under the previous grid's tail).  Plans with wide slices are not split (one block combines their partial sums).
-// Nothing is split where the largest partition is less than kWhole of an SM's share: then the order alone balances the
-// units, and the extra staging would only cost (64 matrices of 5k to 300k rows, 0.52 of a share: whole 315 us, in
-// shares 337; the first 56 of them, 0.67 of a share: 280 and 263).
+// A partition worth more than 1 / kShare of a resident block's share of the batch is split into units that each take
+// every nsub-th slice of its processing order (and stage the whole slice of x again, which costs about kStageCost
+// slots a row, from L2).  With whole partitions as units, a batch with fewer large partitions than resident blocks
+// took as long as its largest one: 24 matrices of 5k to 100k rows on 304 blocks, about 50 partitions of up to 640k
+// entries, 272 us; 91 us in shares (launched directly under the previous grid's tail).  Plans with wide slices are
+// not split (one block combines their partial sums). Nothing is split where the largest partition is less than kWhole
+// of an SM's share: then the order alone balances the units, and the extra staging would only cost (64 matrices of 5k
+// to 300k rows, 0.52 of a share: whole 315 us, in shares 337; the first 56 of them, 0.67 of a share: 280 and 263).
 constexpr double kShare = 2.0;
 constexpr double kWhole = 0.6;
 constexpr int kStageCost = 2;
 
 constexpr int kMaxThreads = 1024;  // block size: 512 when two or more blocks fit an SM, else 1024
 
-// plans with wide slices, out of line: their code costs the other plans no registers
+// plans with wide slices, out of line: their code costs the other plans of the batch no registers
 __device__ __noinline__ bool wide_partition(const BatchPlan& bp, int p, double* xs, BlockState& bs) {
   return partition_spmv<double, double, true, true, false, true, kBatch, false, false, false, true>(
       bp.a, bp.ell_val, bp.er_val, bp.x, bp.y, p, xs, bs);
 }
 
-// tiles: (plan, partition, share, shares)
+// tiles: (plan, partition, share, shares).  WIDE: a plan of the batch has wide slices.  Batches without go without
+// the call: it cost every batch a few registers' spills (64 matrices 317.9 -> 313.4 us, 32 of them 172 -> 160, 16 of
+// them 112 -> 110).
+template <bool WIDE>
 __global__ void __launch_bounds__(kMaxThreads, 1) batch_kernel(const BatchPlan* __restrict__ plans,
                                                               const int4* __restrict__ tiles, int ntiles,
                                                               int* counters) {
@@ -76,7 +79,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) batch_kernel(const BatchPlan* 
     const BatchPlan& bp = plans[tl.x];
     double* xs = reinterpret_cast<double*>(smem_raw);
     const bool ok =
-        bp.a.wide_parts > 0 ? wide_partition(bp, tl.y, xs, bs)
+        WIDE && bp.a.wide_parts > 0 ? wide_partition(bp, tl.y, xs, bs)
         : bp.kbatch == 6
             ? partition_spmv<double, double, true, true, false, true, 6>(bp.a, bp.ell_val, bp.er_val, bp.x, bp.y,
                                                                          tl.y, xs, bs, tl.z, tl.w)
@@ -114,6 +117,7 @@ struct ehyb_batch_s {
   int ntiles = 0, nunits = 0, grid = 0, threads = 512;  // partitions, work units
   size_t smem = 0;
   int64_t max_n = 0;
+  void (*kernel)(const BatchPlan*, const int4*, int, int*) = nullptr;
   bool dirty = true;  // the pointers in `table` are not (known to be) on the device
 };
 
@@ -178,15 +182,18 @@ extern "C" ehyb_status_t ehyb_batch_create(int32_t count, const ehyb_plan_t* pla
   int sms = 0, per_sm = 0, optin = 0;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device);
+  bool wide = false;
+  for (const Tile& t : parts) wide = wide || t.wide;
+  b->kernel = wide ? batch_kernel<true> : batch_kernel<false>;
   // the device's limit for every batch: a smaller one set for this batch would refuse the launches of another
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024);
+    e = cudaFuncSetAttribute(b->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024);
   // 512 threads while two blocks fit an SM (one block's staging overlaps the other's slices), otherwise
   // one block of 1024 threads per SM (32 warps keep enough loads in flight)
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, 512, b->smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b->kernel, 512, b->smem);
   if (e == cudaSuccess && per_sm < 2) {
     b->threads = kMaxThreads;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, kMaxThreads, b->smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b->kernel, kMaxThreads, b->smem);
   }
   if (e != cudaSuccess) { batch_free(b); return cuda_error_status(e, "batch launch setup"); }
   b->grid = sms * std::max(per_sm, 1);
@@ -222,9 +229,9 @@ extern "C" ehyb_status_t ehyb_batch_create(int32_t count, const ehyb_plan_t* pla
   const size_t t_bytes = ((size_t)count * sizeof(BatchPlan) + 255) & ~(size_t)255;
   const size_t l_bytes = ((size_t)std::max(b->nunits, 1) * sizeof(int4) + 255) & ~(size_t)255;
   // partial sums of the plans' wide slices: the batch's own, since a plan may be in it more than once
-  size_t wide = 0;
-  for (BatchPlan& bp : b->table) wide += (size_t)bp.a.wide_parts * 32 * sizeof(double);
-  ehyb_status_t st = device_alloc(&b->arena, t_bytes + l_bytes + 256 + wide);
+  size_t sums = 0;
+  for (BatchPlan& bp : b->table) sums += (size_t)bp.a.wide_parts * 32 * sizeof(double);
+  ehyb_status_t st = device_alloc(&b->arena, t_bytes + l_bytes + 256 + sums);
   if (st != EHYB_OK) { batch_free(b); return st; }
   b->d_table = (BatchPlan*)b->arena;
   b->d_tiles = (int4*)((char*)b->arena + t_bytes);
@@ -278,7 +285,7 @@ extern "C" ehyb_status_t ehyb_batch_spmv(ehyb_batch_t b, const double* const* xs
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  CKB(cudaLaunchKernelEx(&cfg, batch_kernel, (const BatchPlan*)b->d_table, (const int4*)b->d_tiles, b->nunits,
+  CKB(cudaLaunchKernelEx(&cfg, b->kernel, (const BatchPlan*)b->d_table, (const int4*)b->d_tiles, b->nunits,
                          b->d_counters));
   return EHYB_OK;
 }
