@@ -189,15 +189,18 @@ def _check(st: int, where: str):
         raise EhybError(st, where)
 
 
-_raw_stream = _device = None   # torch's own lookups of the current stream's handle and the current device
+# torch's own lookups of the current stream's handle and the current device: set at once, since another thread may be in
+# _stream at any moment
+_lookups: tuple | None = None
 
 
 def _stream(stream) -> int | None:
     if stream is None:
         # every product asks for the current stream: past the first call (which initialises CUDA) its handle is
         # read without building a Stream object (2.1 us of a 6.9 us call on the smallest matrices, with _dev)
-        if _raw_stream is not None:
-            return _raw_stream(_device())
+        if _lookups is not None:
+            raw, dev = _lookups
+            return raw(dev())
         return _first_stream()
     if isinstance(stream, int):
         return stream
@@ -205,12 +208,12 @@ def _stream(stream) -> int | None:
 
 
 def _first_stream() -> int:
-    global _raw_stream, _device
+    global _lookups
     import torch
     s = torch.cuda.current_stream().cuda_stream
     raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
     if raw is not None and dev is not None:
-        _raw_stream, _device = raw, dev
+        _lookups = raw, dev
     return s
 
 
