@@ -286,6 +286,14 @@ extern "C" ehyb_status_t ehyb_mlp_forward(const float* params, const float* X, i
                                           void* workspace, void* stream) {
   if (!params || !X || !out || batch < 0 || (batch > 0 && !workspace)) return EHYB_ERR_INVALID_ARG;
   if (batch == 0) return EHYB_OK;
+  // outputs in X's own memory: a block would write over samples that another has yet to read
+  const uintptr_t x0 = reinterpret_cast<uintptr_t>(X), o0 = reinterpret_cast<uintptr_t>(out);
+  const size_t xb = (size_t)batch * D0 * sizeof(float), ob = (size_t)batch * D3 * sizeof(float);
+  if (x0 < o0 + ob && o0 < x0 + xb) {
+    const cudaError_t e = cudaMemcpyAsync(workspace, X, xb, cudaMemcpyDeviceToDevice, (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_error_status(e, "mlp forward");
+    X = (const float*)workspace;
+  }
   const int per = (int)std::max<int64_t>(kTS, ((int64_t)batch + kMaxBlocks - 1) / kMaxBlocks);
   const int nb = (int)(((int64_t)batch + per - 1) / per);
   const cudaError_t e = launch(mlp_kernel<false>, nb, kMlpT, (cudaStream_t)stream, params, X, (const float*)nullptr,
