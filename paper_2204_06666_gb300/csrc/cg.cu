@@ -1,24 +1,25 @@
-// Conjugate gradients on an EHYB plan (the solver whose SpMV cost motivates the method, Sec. 6), and
-// FP64 iterative refinement around an inner CG whose matrix values are stored in FP32 or BF16.
+// Conjugate gradients on an EHYB plan (the solver whose SpMV cost motivates the method, Sec. 6), and FP64 iterative
+// refinement around an inner CG whose matrix values are stored in FP32 or BF16.
 //
-// All vectors live in the plan's numbering (b and x are permuted once in and once out).  One CG
-// iteration is three kernels:
+// All vectors live in the plan's numbering (b and x are permuted once in and once out).  One CG iteration is three
+// kernels:
 //   K1  q = A p on the EHYB kernel, with p . q accumulated in its epilogue (p_r is already in shared
 //       memory): one partial per partition, reduced into one scalar by the last block to finish;
 //   K2  alpha = (r.r) / (p.q) (once per block); x += alpha p; r -= alpha q; partial sums of the new r.r;
 //       the last block reduces them, stores r.r(new) in the history, computes beta = r.r(new) / r.r(old),
 //       advances the device iteration counter and raises `done` at convergence or at the limit;
 //   K3  p = r + beta p.
-// alpha and beta never leave the device.  Every reduction runs in a fixed order, so a solve is bit-
-// reproducible.  Once `done` is up the remaining kernels of a chunk return at once, so the iteration
-// count is exact although the host looks at the flag only once per chunk.  A chunk of kChunk
-// iterations is captured once into a CUDA graph and replayed.  A plan whose partitions are all resident at
-// once (Eq. 1's are, up to 4.4 M rows) runs its iterations inside one cooperative kernel instead
-// (cg_persist_kernel).
+// alpha and beta never leave the device.  Every reduction runs in a fixed order, so a solve is bit-reproducible.
+// Once `done` is up the remaining kernels of a chunk return at once, so the iteration count is exact although the
+// host looks at the flag only once per chunk.  A chunk of kChunk iterations is captured once into a CUDA graph and
+// replayed.  A plan whose partitions are all resident at once (at most one per SM) runs its iterations inside one
+// cooperative kernel instead (cg_persist_kernel), with the same bits, where that is the faster form: on Eq. 1's
+// partitions up to about 3.6 M rows in FP64 (two vectors' worth of shared memory), 840k with FP32 values, 690k with
+// BF16.
 //
-// Refinement (refine = 1: FP32 values, 2: BF16 values): outer FP64 residual r = b - A x on the FP64
-// plan, inner CG on the low-precision copy of the values with FP32 vectors, FP32 SpMV accumulation and
-// FP64 dot products / alpha / beta, started from d = 0 on r / ||r||; x += ||r|| d in FP64.
+// Refinement (refine = 1: FP32 values, 2: BF16 values): outer FP64 residual r = b - A x on the FP64 plan, inner CG on
+// the low-precision copy of the values with FP32 vectors, FP32 SpMV accumulation and FP64 dot products / alpha /
+// beta, started from d = 0 on r / ||r||; x += ||r|| d in FP64.
 #include <cuda_runtime.h>
 
 #include <chrono>
@@ -579,7 +580,7 @@ __global__ void __launch_bounds__(MAXT, 1) cg_persist_kernel(core::KArgs a, cons
         ps[checked(sh.prod.rows + j, a.smem_elems, a.status)] = load_x(c.p + checked(sh.halo[j], a.n, a.status));
       __syncthreads();
     }
-    persist::run_slices<V, X, KB, RUNS>(&sh.prod, &sh.sync, 2 * step);
+    persist::run_slices<V, X, KB, RUNS, false>(&sh.prod, &sh.sync, 2 * step);
     __syncthreads();
     if (sh.stop) break;
     cg_step_pq(sh, round);

@@ -1,8 +1,8 @@
-// Preconditioned conjugate gradients on an EHYB plan with the FSAI preconditioner M^-1 = G^T G (fsai.cpp):
-// the solver the paper's Sec. 6 motivates, its preconditioner applied as two further EHYB products.
+// Preconditioned conjugate gradients on an EHYB plan with the FSAI preconditioner M^-1 = G^T G (fsai.cpp): the solver
+// the paper's Sec. 6 motivates, its preconditioner applied as two further EHYB products.
 //
-// All vectors live in the matrix plan's numbering (b and x are permuted once in and once out).  One
-// iteration is four launches:
+// All vectors live in the matrix plan's numbering (b and x are permuted once in and once out).  One iteration is four
+// launches:
 //   K1  q = A p on the matrix plan, p . q fused into its epilogue (last block reduces);
 //   K2  alpha = (r.z) / (p.q); x += alpha p; r -= alpha q (FP32 copy of r when G is applied in FP32);
 //       partials of r.r, the last block stores r.r, keeps r.z as (r.z)_old, advances the iteration and
@@ -12,18 +12,19 @@
 //   K4  z = G^T t on G^T's plan;
 //   K5  p = z + beta p with beta = (r.z)_new / (r.z)_old (a coalesced pass: fusing it into K4's scattered
 //       stores measured slower).
-// alpha, beta and the inner products never leave the device; every reduction has a fixed order, so a
-// solve is bit-reproducible.  Chunks of kChunk iterations are captured once into a CUDA graph and
-// replayed; once `done` is up the remaining launches of a chunk return at once.  Plans whose partitions are all
-// resident at once (Eq. 1's are, up to 4.4 M rows) run their iterations inside one cooperative kernel instead
-// (pcg_persist_kernel), which also leaves at the iteration that met its threshold.
+// alpha, beta and the inner products never leave the device; every reduction has a fixed order, so a solve is
+// bit-reproducible.  Chunks of kChunk iterations are captured once into a CUDA graph and replayed; once `done` is up
+// the remaining launches of a chunk return at once.  Plans whose partitions are all resident at once (at most one per
+// SM) run their iterations inside one cooperative kernel instead (pcg_persist_kernel), with the same bits; it also
+// leaves at the iteration that met its threshold.  On Eq. 1's partitions up to about 1.8 M rows in FP64 (a slice of p
+// and one of r or t in shared memory; more with low-precision G), 1.25 M on FP32 vectors.
 //
-// Mixed precision (ehyb_pcg_refined): one PCG that runs on FP32 vectors -- A's FP32 / BF16 values, G's
-// FP32 / BF16 values, FP32 accumulation, FP64 inner products and alpha / beta -- with FP64 residual
-// replacement: the iteration works on d (A d = r / s for the residual r and scale s of the last
-// replacement); whenever its residual has dropped by the factor delta, x += s d in FP64, r = b - A x is
-// recomputed in FP64, the FP32 residual restarts from r / s' and the direction is kept, rescaled by s / s'
-// (and (r.z)_old by (s / s')^2), so the Krylov iteration is not restarted.  Stops when ||b - A x|| <= rtol ||b||.
+// Mixed precision (ehyb_pcg_refined): one PCG that runs on FP32 vectors -- A's FP32 / BF16 values, G's FP32 / BF16
+// values, FP32 accumulation, FP64 inner products and alpha / beta -- with FP64 residual replacement: the iteration
+// works on d (A d = r / s for the residual r and scale s of the last replacement); whenever its residual has dropped
+// by the factor delta, x += s d in FP64, r = b - A x is recomputed in FP64, the FP32 residual restarts from r / s'
+// and the direction is kept, rescaled by s / s' (and (r.z)_old by (s / s')^2), so the Krylov iteration is not
+// restarted.  Stops when ||b - A x|| <= rtol ||b||.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -683,7 +684,7 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_persist_kernel(core::KArgs a, con
     // rounds of the sums p.q, r.r and t.t, and rounds of arrivals with r, t and p: 3 step + 1, + 2 and + 3 each
     const int round = 3 * step + 1;
     // K1: q = A p (p of the other blocks from round 3 step on), p.q
-    persist::run_slices<VA, XA, KA, kRunsA>(&sh.a, &sh.sync, 3 * step);
+    persist::run_slices<VA, XA, KA, kRunsA, false>(&sh.a, &sh.sync, 3 * step);
     __syncthreads();
     if (sh.stop) break;
     pcg_step_pq(sh, round);
@@ -692,13 +693,13 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_persist_kernel(core::KArgs a, con
     if (sh.stop) break;
     // K3: t = G r, t.t = r.z
     persist::stage_halo(&sh.g, &sh.sync, round);
-    persist::run_slices<VG, XG, KG, kRunsG>(&sh.g, &sh.sync, round);
+    persist::run_slices<VG, XG, KG, kRunsG, true>(&sh.g, &sh.sync, round);
     __syncthreads();
     if (threadIdx.x == 0) persist::arrive(sh.sync);  // t
     pcg_step_tt(sh, round + 2);
     // K4: z = G^T t
     persist::stage_halo(&sh.h, &sh.sync, round + 1);
-    persist::run_slices<VG, XG, KG, kRunsG>(&sh.h, &sh.sync, round + 1);
+    persist::run_slices<VG, XG, KG, kRunsG, true>(&sh.h, &sh.sync, round + 1);
     pcg_step_direction(sh, round + 2);
     if (sh.stop) break;
     __syncthreads();
@@ -839,13 +840,13 @@ ehyb_status_t launch_persist(ehyb_precond_t M, const VA* av, const VA* aev, cons
                              const VG* hv, const VG* hev, PcgPersist<XA, XG> c, cudaStream_t s, bool* ran) {
   const DevPlan &D = M->plan->dev, &G = M->g->dev, &H = M->gt->dev;
   auto kernel = pcg_persist_kernel<VA, XA, KA, VG, XG, MAXT>;
-  auto args_of = [](const DevPlan& P, bool runs) {
+  auto args_of = [](const DevPlan& P, bool runs, bool staged) {
     core::KArgs a = core::make_kargs(P);
     if (runs) {
       a.ell_col = P.ell_col_low;
       a.er_scol = P.er_scol_low;
       a.er_scol_old = P.er_scol_old_low;
-      if (P.er_hcol_low) {
+      if (staged && P.er_hcol_low) {
         a.er_hcol = P.er_hcol_low;
         a.halo_ptr = P.low_halo_ptr;
         a.halo_old = P.low_halo_old;
@@ -854,7 +855,8 @@ ehyb_status_t launch_persist(ehyb_precond_t M, const VA* av, const VA* aev, cons
     a.meta_cap = P.max_part_slices;
     return a;
   };
-  core::KArgs a = args_of(D, sizeof(VA) < 8), g = args_of(G, sizeof(VG) < 8), h = args_of(H, sizeof(VG) < 8);
+  core::KArgs a = args_of(D, sizeof(VA) < 8, false), g = args_of(G, sizeof(VG) < 8, true),
+              h = args_of(H, sizeof(VG) < 8, true);
   int optin = 0, resident = 0, sms = 0;
   CKP(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, M->plan->device));
   CKP(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, M->plan->device));

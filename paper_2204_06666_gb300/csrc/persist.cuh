@@ -479,7 +479,8 @@ __device__ __noinline__ void stage_halo(Product<V, X>* pr, const SyncArgs* sync,
 // All slices of the block's partition, claimed dynamically from pr->counter (blockDim.x / 32 on entry).  Before its
 // first extra row a warp waits until round `round` of arrive() is complete (0: at once); a wait that ran out
 // raises *pr->stop and ends the pass.
-template <typename V, typename X, int KB, bool RUNS>
+// STAGED: the extra rows' x may be staged (pr->er_hcol).
+template <typename V, typename X, int KB, bool RUNS, bool STAGED>
 __device__ __noinline__ void run_slices(Product<V, X>* pr, const SyncArgs* sync, int round) {
   const int lane = threadIdx.x & 31;
   const V *ell_val = pr->ell_val, *er_val = pr->er_val;
@@ -525,7 +526,7 @@ __device__ __noinline__ void run_slices(Product<V, X>* pr, const SyncArgs* sync,
         return;
       }
       const int32_t* ecol = pr->er_col;
-      if constexpr (RUNS) {
+      if constexpr (RUNS && STAGED) {
         if (const uint16_t* hcol = pr->er_hcol) {
           const X* const xh = reinterpret_cast<const X*>(smem_raw + pr->xh_off);
           acc = slab_dot_runs<V, X, 16>(er_val + epos, hcol + epos, lane, we, xh, acc, pr->nh, status);
