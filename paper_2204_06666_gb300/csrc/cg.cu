@@ -741,7 +741,11 @@ ehyb_status_t launch_persist(ehyb_plan_t P, const V* ev, const V* erv, CgPersist
   a.smem_elems = (int64_t)(smem / sizeof(X));
   const size_t tbl = al((size_t)D.max_part_slices * sizeof(core::SliceMeta));
   const size_t vec = al((size_t)D.max_part_rows * sizeof(X));
-  const size_t budget = std::min((size_t)(optin - persist::kMaxStatic), persist::shared_budget(smem + persist::terms_bytes(D.threads)));
+  // with the slice table where that fits (ms a solve, separate launches -> without it -> with: tet 133^3 5.57, 5.62,
+  // 5.31; 140^3 6.18, 6.69, 6.25)
+  const size_t must = smem + persist::terms_bytes(D.threads), with_table = persist::shared_budget(must + tbl, 196);
+  const size_t budget = std::min((size_t)(optin - persist::kMaxStatic),
+                                 with_table ? with_table : persist::shared_budget(must, 196));
   auto place = [&](size_t bytes) -> int32_t {
     if (smem + bytes > budget) return -1;
     const size_t o = smem;

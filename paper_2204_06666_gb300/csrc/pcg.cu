@@ -16,8 +16,8 @@
 // bit-reproducible.  Chunks of kChunk iterations are captured once into a CUDA graph and replayed; once `done` is up
 // the remaining launches of a chunk return at once.  Plans whose partitions are all resident at once (at most one per
 // SM) run their iterations inside one cooperative kernel instead (pcg_persist_kernel), with the same bits; it also
-// leaves at the iteration that met its threshold.  On Eq. 1's partitions up to about 1.8 M rows in FP64 (a slice of p
-// and one of r or t in shared memory; more with low-precision G), 1.25 M on FP32 vectors.
+// leaves at the iteration that met its threshold.  On Eq. 1's partitions up to about 1.5 M rows in FP64 (a slice of p
+// and one of r or t in shared memory), 2 M with low-precision G, 1.25 M on FP32 vectors.
 //
 // Mixed precision (ehyb_pcg_refined): one PCG that runs on FP32 vectors -- A's FP32 / BF16 values, G's FP32 / BF16
 // values, FP32 accumulation, FP64 inner products and alpha / beta -- with FP64 residual replacement: the iteration
@@ -868,7 +868,7 @@ ehyb_status_t launch_persist(ehyb_precond_t M, const VA* av, const VA* aev, cons
   const size_t terms = persist::terms_bytes(std::max(D.threads, G.threads));
   c.g_warps = G.threads / 32;
   const size_t budget =
-      std::min((size_t)(optin - persist::kMaxStatic), persist::shared_budget(smem + al(vg) + terms));
+      std::min((size_t)(optin - persist::kMaxStatic), persist::shared_budget(smem + al(vg) + terms, 164));
   auto place = [&](size_t bytes) -> int32_t {
     if (smem + al(bytes) > budget) return -1;
     const size_t o = smem;

@@ -27,9 +27,9 @@ namespace persist {
 using namespace core;
 
 constexpr int kMaxGrid = 160;      // blocks of a persistent launch (five partial sums per gathering lane)
-// Least time limit (wait_timeout_ns) with which solvers iterate persistently: the others' work, or another process's time
-// slice, may keep a block waiting for milliseconds.  Plans with a shorter one take the separate launches, which have no
-// such waits.
+// Least time limit (wait_timeout_ns) with which solvers iterate persistently: the others' work, or another process's
+// time slice, may keep a block waiting for milliseconds.  Plans with a shorter one take the separate launches, which
+// have no such waits.
 constexpr uint64_t kMinLimitNs = 100000000ull;
 constexpr int kAborted = 2;
 
@@ -62,20 +62,23 @@ struct SyncArgs {
 };
 
 // Shared memory of a persistent block, out of the SM's 256 KB that the rest of L1 shares: the least of the sizes the
-// hardware can set aside that holds `must` bytes (what the kernel cannot do without), less what the system and the
-// kernel's own variables take; the vectors beyond it go there only as far as they fit.  The extra rows gather freshly
-// written vectors through L1, so a vector kept in shared memory at L1's cost loses more than it saves: at elasticity
-// 64^3 (41 KB a vector) the FP64 PCG took 23.1 ms a solve with five vectors in shared memory (215 KB), 9.5 with two
-// (separate launches 9.8); scalar hexahedra 80^3 with BF16 G 3.0 and 1.9 ms (2.4).  0: more than 196 KB, where
-// the separate launches are the faster form (tet 126^3, FP64 G, two vectors of 105 KB: 4.9 ms against 3.9).
+// hardware can set aside that holds `must` bytes (what the kernel should not do without), less what the system and
+// the kernel's own variables take; the vectors beyond it go there only as far as they fit.  The extra rows gather
+// freshly written vectors through L1, so a vector kept in shared memory at L1's cost loses more than it saves: at
+// elasticity 64^3 (41 KB a vector) the FP64 PCG took 23.1 ms a solve with five vectors in shared memory (215 KB), 9.5
+// with two (separate launches 9.8); scalar hexahedra 80^3 with BF16 G 3.0 and 1.9 ms (2.4).  0: more than `most` KB,
+// where the separate launches are the faster form: 196 for CG (ms a solve, separate -> persistent: tet 150^3 9.61 ->
+// 8.48), 164 for PCG, which gathers two more vectors (FP64 G: tet 111^3, 160 KB, 3.00 -> 2.80, scalar hexahedra
+// 115^3, 176 KB, 6.11 -> 6.89; FP32 G: tet 121^3, 156 KB, 3.25 -> 3.17, 126^3, 175 KB, 3.57 -> 3.61).
 //
-// The budget only decides what is placed.  What a kernel may be launched with is a property of its instantiation, shared
-// by every plan and host thread, so it is always set to the device's limit: a smaller plan's budget set there would
-// refuse the launch of a larger one that another thread is about to make.  (A launch's own size decides L1's share.)
+// The budget only decides what is placed.  What a kernel may be launched with is a property of its instantiation,
+// shared by every plan and host thread, so it is always set to the device's limit: a smaller plan's budget set there
+// would refuse the launch of a larger one that another thread is about to make.  (A launch's own size decides L1's
+// share.)
 constexpr int kMaxStatic = 2048;  // static shared memory of a persistent kernel
-inline size_t shared_budget(size_t must) {
+inline size_t shared_budget(size_t must, size_t most) {
   for (size_t kb : {100, 132, 164, 196})
-    if (must + 3072 <= kb * 1024) return kb * 1024 - 3072;
+    if (kb <= most && must + 3072 <= kb * 1024) return kb * 1024 - 3072;
   return 0;
 }
 
@@ -97,8 +100,8 @@ constexpr int kMaxRowsF32 = 5500, kMaxRowsBf16 = 4500, kMaxRowsPcg32 = 8192;
 inline bool even_enough(int max_rows, int64_t n, int sms, int spare) { return max_rows - n / sms <= spare; }
 constexpr int kSpare64 = 3500, kSpare32 = 2500, kSparePcg = 4500;
 
-// The meeting place of a launch, zeroed.  Test hook (inject_wait_fault 2 / 3): one arrival at the sums / the plain rounds
-// never happens, so that the first wait there runs out.
+// The meeting place of a launch, zeroed.  Test hook (inject_wait_fault 2 / 3): one arrival at the sums / the plain
+// rounds never happens, so that the first wait there runs out.
 inline cudaError_t clear_meeting(Meeting* m, int inject, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(m, 0, sizeof(Meeting), s);
   if (e == cudaSuccess && inject >= 2)
