@@ -567,18 +567,23 @@ struct BlockState {
   double ws[32];
 };
 
-// One partition p of a plan: stage its slice of x_p, run its slab (and ER) slices, write y. GATHER: x is given in the
-// caller's numbering and the permutation into the plan numbering is fused into the staging (xs[r - pb] =
-// x[new_to_old[r]], plain loads) and into the ER gathers (columns in the caller's numbering), so no permuted copy of
-// x is written or read; otherwise x is x_p and the slice is staged by one bulk asynchronous copy. Returns false
-// (uniformly across the block) when the staging wait ran out of time. TABLE: the launch may provide the partition's
-// slice table (a.meta_off); without it only the global path is compiled (the persistent batch kernel, whose blocks
-// run many partitions one after the other). WIDE: the plan has wide slices. HER: the extra rows' x is staged too
-// (a.halo_*, a.er_hcol) and their slots run like the slab's: same order, same bits. sub, nsub: the block takes every
-// nsub-th slice of the processing order, from the sub-th on (nsub > 1: several blocks share a partition of a batch;
-// not with WIDE, whose partial sums are combined by one block). PDL: the kernel was launched with programmatic stream
-// serialization and has not yet waited for the previous grid: the slice table, which reads plan arrays only, is
-// filled first, then griddepcontrol.wait, then every read of x (and of the solver's skip flag) and every write of y.
+// One partition p of a plan: stage its slice of x_p, run its slab (and ER) slices, write y.
+// GATHER: x is given in the caller's numbering and the permutation into the plan numbering is fused
+// into the staging (xs[r - pb] = x[new_to_old[r]], plain loads) and into the ER gathers (columns in the
+// caller's numbering), so no permuted copy of x is written or read; otherwise x is x_p and the slice is
+// staged by one bulk asynchronous copy.
+// Returns false (uniformly across the block) when the staging wait ran
+// out of time.
+// TABLE: the launch may provide the partition's slice table (a.meta_off); without it only the global path is
+// compiled (the persistent batch kernel, whose blocks run many partitions one after the other).
+// WIDE: the plan has wide slices.
+// HER: the extra rows' x is staged too (a.halo_*, a.er_hcol) and their slots run like the slab's: same order, same
+// bits.
+// sub, nsub: the block takes every nsub-th slice of the processing order, from the sub-th on (nsub > 1: several
+// blocks share a partition of a batch; not with WIDE, whose partial sums are combined by one block).
+// PDL: the kernel was launched with programmatic stream serialization and has not yet waited for the previous
+// grid: the slice table, which reads plan arrays only, is filled first, then griddepcontrol.wait, then every
+// read of x (and of the solver's skip flag) and every write of y.
 template <typename V, typename X, bool SCATTER, bool ER_SLICED, bool DOT = false, bool GATHER = false,
           int KB = kBatch, bool RUNS = false, bool TABLE = false, bool PDL = false, bool WIDE = false,
           bool HER = false>
