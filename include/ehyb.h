@@ -313,7 +313,7 @@ typedef struct {
  * filled) when the test was not met.  The solver workspace (5 FP64 + 4 FP32 vectors) is allocated on the first call.
  * The iterations (product with p.q, update with r.r, direction) run inside one cooperative kernel where the plan's
  * partitions are all resident at once and that is the faster form: at most one partition per SM, two vectors of a
- * partition in 196 KB of shared memory, no chunked long rows, at most 5,500 (FP32 values) or 4,500 (BF16) rows a
+ * partition in 196 KB of shared memory, no chunked long rows, at most 11,500 (FP32 values) or 9,000 (BF16) rows a
  * partition on FP32 vectors; else as three launches each, replayed from CUDA graphs of 16 iterations.  Both forms
  * return the same bits.
  */
@@ -431,7 +431,7 @@ ehyb_status_t ehyb_precond_destroy(ehyb_precond_t M); /* NULL is fine; synchroni
  * or after max_iter iterations; info->relres is the true FP64 residual ||b - A x|| / ||b|| of the returned
  * x.  The iterations (A p with p.q, the update, G r with r.z, G^T t, the direction) run inside one cooperative
  * kernel when the plan's partitions are all resident at once (sliced ER layout, no chunked long rows, at most one
- * partition per SM, a partition's slices of two vectors in 164 KB of shared memory, at most 8,192 rows a partition on
+ * partition per SM, a partition's slices of two vectors in 164 KB of shared memory, at most 11,500 rows a partition on
  * FP32 vectors), else as five launches each, replayed from CUDA graphs of 16 iterations, with the same bits; alpha and
  * beta stay on the device.  Synchronous.
  * EHYB_ERR_NOT_CONVERGED at the iteration limit or when p.A p <= 0; EHYB_ERR_INVALID_ARG when M belongs

@@ -14,7 +14,7 @@
 // host looks at the flag only once per chunk.  A chunk of kChunk iterations is captured once into a CUDA graph and
 // replayed.  A plan whose partitions are all resident at once (at most one per SM) runs its iterations inside one
 // cooperative kernel instead (cg_persist_kernel), with the same bits, where that is the faster form: on Eq. 1's
-// partitions up to about 3.6 M rows in FP64 (two vectors' worth of shared memory), 840k with FP32 values, 690k with
+// partitions up to about 3.6 M rows in FP64 (two vectors' worth of shared memory), 1.75 M with FP32 values, 1.37 M with
 // BF16.
 //
 // Refinement (refine = 1: FP32 values, 2: BF16 values): outer FP64 residual r = b - A x on the FP64 plan, inner CG on
@@ -389,17 +389,17 @@ struct CgBlock {
 };
 
 // p.q and alpha
-template <typename V, typename X>
+template <bool DOT, typename V, typename X>
 __device__ __noinline__ void cg_step_pq(CgBlock<V, X>& sh, int round) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const X* const ps = reinterpret_cast<const X*>(smem_raw);
   const int warps = blockDim.x >> 5;
   double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
-  {
+  if constexpr (!DOT) {
     const X* const q = sh.q;
     persist::part_terms(sh.prod, warps, red, [&](int i) { return make_double2((double)q[i], (double)ps[i]); });
+    __syncthreads();
   }
-  __syncthreads();
   if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_part(sh.sync, round, 0, red, warps, sh.sums);
   double pq;
   const bool ok = persist::gather_sum(sh.sync, round, sh.sync.m->part[0], gridDim.x, red, &sh.stop, &pq);
@@ -580,10 +580,11 @@ __global__ void __launch_bounds__(MAXT, 1) cg_persist_kernel(core::KArgs a, cons
         ps[checked(sh.prod.rows + j, a.smem_elems, a.status)] = load_x(c.p + checked(sh.halo[j], a.n, a.status));
       __syncthreads();
     }
-    persist::run_slices<V, X, KB, RUNS, false>(&sh.prod, &sh.sync, 2 * step);
+    persist::run_slices<V, X, KB, RUNS, false, persist::kDotInProduct<V, MAXT>>(
+        &sh.prod, &sh.sync, 2 * step, reinterpret_cast<double*>(smem_raw + sh.red_off));
     __syncthreads();
     if (sh.stop) break;
-    cg_step_pq(sh, round);
+    cg_step_pq<persist::kDotInProduct<V, MAXT>>(sh, round);
     if (sh.stop) break;
     cg_step_update(sh, round + 1, round);
     if (sh.stop) break;
@@ -718,7 +719,7 @@ ehyb_status_t run_chunk(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s) {
 // One persistent launch of at most kPersistSteps iterations; *ran = false (and nothing launched) for a plan that
 // needs the separate launches: more partitions than SMs (a block owns one partition, all blocks resident), a wide
 // slice (its sums go through the plan's workspace), more shared memory than persist::shared_budget grants, more rows
-// a partition than persist::even_enough or, with FP32 vectors, kMaxRowsF32 / kMaxRowsBf16 allow, a time
+// a partition than persist::even_enough or, with FP32 vectors, kMaxRowsF32 / kMaxRowsBf16(Staged) allow, a time
 // limit below kMinLimitNs, the staging-fault test hook.
 constexpr int kPersistSteps = 2000;  // bounds one launch to a fraction of a second
 
@@ -783,7 +784,10 @@ ehyb_status_t run_persist(ehyb_plan_t P, CgWork* w, int lowp, cudaStream_t s, bo
     return D.kbatch == 6 ? launch_persist<double, double, 6, false, 1024>(P, D.ell_val, D.er_sval, c, s, ran)
                          : launch_persist<double, double, 8, false, 1024>(P, D.ell_val, D.er_sval, c, s, ran);
   }
-  if (D.max_part_rows > (lowp == 1 ? persist::kMaxRowsF32 : persist::kMaxRowsBf16)) return EHYB_OK;
+  if (D.max_part_rows > (lowp == 1       ? persist::kMaxRowsF32
+                         : D.er_hcol_low ? persist::kMaxRowsBf16Staged
+                                         : persist::kMaxRowsBf16))
+    return EHYB_OK;
   const CgPersist<float> c{w->d32, w->r32, w->p32, w->q32, -1, -1, -1, -1, -1, kPersistSteps, w->st, w->hist, sync};
   const bool runs = D.lowp_group == 4, half = D.threads <= 512;
   if (lowp == 1)

@@ -17,7 +17,7 @@
 // the remaining launches of a chunk return at once.  Plans whose partitions are all resident at once (at most one per
 // SM) run their iterations inside one cooperative kernel instead (pcg_persist_kernel), with the same bits; it also
 // leaves at the iteration that met its threshold.  On Eq. 1's partitions up to about 1.5 M rows in FP64 (a slice of p
-// and one of r or t in shared memory), 2 M with low-precision G, 1.25 M on FP32 vectors.
+// and one of r or t in shared memory), 2 M with low-precision G, 1.75 M on FP32 vectors.
 //
 // Mixed precision (ehyb_pcg_refined): one PCG that runs on FP32 vectors -- A's FP32 / BF16 values, G's FP32 / BF16
 // values, FP32 accumulation, FP64 inner products and alpha / beta -- with FP64 residual replacement: the iteration
@@ -428,17 +428,17 @@ struct PcgBlock {
 };
 
 // p.q and alpha
-template <typename VA, typename XA, typename VG, typename XG>
+template <bool DOT, typename VA, typename XA, typename VG, typename XG>
 __device__ __noinline__ void pcg_step_pq(PcgBlock<VA, XA, VG, XG>& sh, int round) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const XA* const ps = reinterpret_cast<const XA*>(smem_raw);
   double* const red = reinterpret_cast<double*>(smem_raw + sh.red_off);
   const int warps = blockDim.x >> 5;
-  {
+  if constexpr (!DOT) {
     const XA* const q = sh.q;
     persist::part_terms(sh.a, warps, red, [&](int i) { return make_double2((double)q[i], (double)ps[i]); });
+    __syncthreads();
   }
-  __syncthreads();
   if (threadIdx.x < 32 * persist::kSumWarps) persist::publish_part(sh.sync, round, 0, red, warps, sh.sums);
   double pq;
   const bool ok = persist::gather_sum(sh.sync, round, sh.sync.m->part[0], gridDim.x, red, &sh.stop, &pq);
@@ -684,22 +684,23 @@ __global__ void __launch_bounds__(MAXT, 1) pcg_persist_kernel(core::KArgs a, con
     // rounds of the sums p.q, r.r and t.t, and rounds of arrivals with r, t and p: 3 step + 1, + 2 and + 3 each
     const int round = 3 * step + 1;
     // K1: q = A p (p of the other blocks from round 3 step on), p.q
-    persist::run_slices<VA, XA, KA, kRunsA, false>(&sh.a, &sh.sync, 3 * step);
+    persist::run_slices<VA, XA, KA, kRunsA, false, persist::kDotInProduct<VA, MAXT>>(
+        &sh.a, &sh.sync, 3 * step, reinterpret_cast<double*>(smem_raw + sh.red_off));
     __syncthreads();
     if (sh.stop) break;
-    pcg_step_pq(sh, round);
+    pcg_step_pq<persist::kDotInProduct<VA, MAXT>>(sh, round);
     if (sh.stop) break;
     pcg_step_update(sh, round + 1, round);
     if (sh.stop) break;
     // K3: t = G r, t.t = r.z
     persist::stage_halo(&sh.g, &sh.sync, round);
-    persist::run_slices<VG, XG, KG, kRunsG, true>(&sh.g, &sh.sync, round);
+    persist::run_slices<VG, XG, KG, kRunsG, true, false>(&sh.g, &sh.sync, round);
     __syncthreads();
     if (threadIdx.x == 0) persist::arrive(sh.sync);  // t
     pcg_step_tt(sh, round + 2);
     // K4: z = G^T t
     persist::stage_halo(&sh.h, &sh.sync, round + 1);
-    persist::run_slices<VG, XG, KG, kRunsG, true>(&sh.h, &sh.sync, round + 1);
+    persist::run_slices<VG, XG, KG, kRunsG, true, false>(&sh.h, &sh.sync, round + 1);
     pcg_step_direction(sh, round + 2);
     if (sh.stop) break;
     __syncthreads();

@@ -83,22 +83,24 @@ inline size_t shared_budget(size_t must, size_t most) {
 }
 
 // Rows of a partition up to which iterations on FP32 vectors run persistently.  Beyond, the FP32 products are short
-// of bytes rather than of launches, and the vectors' passes of the separate launches are the faster ones.  CG, us an
-// iteration separate -> persistent, FP32 values: tet 90^3 (4,797 rows) 44.1 -> 43.3, 96^3 (5,821) 47.7 -> 48.1, 104^3
-// (7,401) 53.4 -> 54.1; BF16: tet 90^3 46.3 -> 46.8, 107^3 (8,060) 58.4 -> 61.1, elasticity 64^3 (5,174) 92.0 ->
-// 97.7.  Mixed PCG: tet 107^3 162 -> 144; 114^3 (9,747 rows) and 126^3 lost about a tenth before its sums took the
-// launches' order.
-constexpr int kMaxRowsF32 = 5500, kMaxRowsBf16 = 4500, kMaxRowsPcg32 = 8192;
+// of bytes rather than of launches, and the vectors' passes of the separate launches are the faster ones.  Time of a
+// solve, separate over persistent: CG (refinement), FP32 values, tet 107^3 (8,060 rows) 1.10, 120^3 (11,369) 1.04,
+// scalar hexahedra 110^3 (8,757) 1.03, 120^3 0.99, elasticity 64^3 (5,174) 1.00, 76^3 (8,664) 1.09; BF16, tet 107^3
+// 1.07, 120^3 1.02, scalar hexahedra 110^3 1.00, 120^3 0.98.  Where the separate product stages its extra rows and
+// this one gathers them, BF16: elasticity 50^3 (2,468) 1.01, 54^3 (3,108) 1.00, 64^3 0.96.  Mixed PCG: tet 120^3
+// 1.09, scalar hexahedra 120^3 1.04, elasticity 58^3 1.03.
+constexpr int kMaxRowsF32 = 11500, kMaxRowsBf16 = 9000, kMaxRowsBf16Staged = 3000, kMaxRowsPcg32 = 11500;
 
 // Whether a plan's partitions are even enough with the SMs: a block passes over its partition's vectors alone, where
 // the separate launches spread them over the chip, so each row beyond the chip's share costs about 1.7 ns an
 // iteration of FP64 CG against the 5 us or so that the launches cost.  `spare`: the rows beyond n / SMs up to which
 // persistent iterations were the faster ones (ms a solve, separate -> persistent; FP64 CG: tet 37^3 in partitions of
 // 3,000 rows 1.57 -> 1.48, of 6,000 2.11 -> 2.23, tet 60^3 in 6,000 2.28 -> 2.36, tet 90^3 in 8,000 3.03 -> 2.94, in
-// 10,000 3.40 -> 3.55; FP32 CG: elasticity 24^3 in 3,000 4.12 -> 3.96, in 6,000 5.71 -> 6.18; FP64 PCG with BF16 G:
-// tet 60^3 in 6,000 1.78 -> 1.70, in 12,000 2.56 -> 2.87; the other PCG forms gained at every size).
+// 10,000 3.40 -> 3.55; FP32 CG: tet 37^3 in 4,500 2.36 -> 2.12, elasticity 24^3 in 3,000 3.45 -> 3.07, in 4,500 4.06
+// -> 4.10; FP64 PCG with BF16 G: tet 60^3 in 6,000 1.78 -> 1.70, in 12,000 2.56 -> 2.87; the other PCG forms gained
+// at every size).
 inline bool even_enough(int max_rows, int64_t n, int sms, int spare) { return max_rows - n / sms <= spare; }
-constexpr int kSpare64 = 3500, kSpare32 = 2500, kSparePcg = 4500;
+constexpr int kSpare64 = 3500, kSpare32 = 4000, kSparePcg = 4500;
 
 // The meeting place of a launch, zeroed.  Test hook (inject_wait_fault 2 / 3): one arrival at the sums / the plain
 // rounds never happens, so that the first wait there runs out.
@@ -378,6 +380,11 @@ __device__ __forceinline__ bool wait_block(const SyncArgs& g, int round, int* se
   return ok;
 }
 
+// Whether the product itself leaves the terms of p.q (run_slices, DOT): on low-precision values, and where a warp has
+// hardly more than one slice (MAXT 512: at most 16 warps, one for each slice of the average partition).
+template <typename V, int MAXT>
+constexpr bool kDotInProduct = sizeof(V) < 8 || MAXT <= 512;
+
 // One product of a block: what run_slices needs of the plan, the partition and the vectors.  It lies in shared memory,
 // and run_slices is a function of its own: a persistent kernel holds several loops that need every register, and
 // what the compiler keeps in registers across them (parameters, addresses) it would have to spill, to come back
@@ -480,11 +487,15 @@ __device__ __noinline__ void stage_halo(Product<V, X>* pr, const SyncArgs* sync,
 }
 
 // All slices of the block's partition, claimed dynamically from pr->counter (blockDim.x / 32 on entry).  Before its
-// first extra row a warp waits until round `round` of arrive() is complete (0: at once); a wait that ran out
-// raises *pr->stop and ends the pass.
+// first extra row a warp waits until round `round` of arrive() is complete (0: at once); a wait that ran out raises
+// *pr->stop and ends the pass.
 // STAGED: the extra rows' x may be staged (pr->er_hcol).
-template <typename V, typename X, int KB, bool RUNS, bool STAGED>
-__device__ __noinline__ void run_slices(Product<V, X>* pr, const SyncArgs* sync, int round) {
+// DOT: the terms of out.x go to red, in the order of part_terms; the warps then take their slices in turn instead of
+// claiming them.  Low-precision products gain by that (a pass over q and x less: elasticity 64^3 FP32 CG 102.9 ->
+// 97.7 us an iteration), FP64 ones need the balance more (elasticity 40^3 CG 54.5 us an iteration with claims, 59.4
+// without) unless a warp has one slice anyway (tet 40^3 FP64 CG 18.9 -> 18.2 us).
+template <typename V, typename X, int KB, bool RUNS, bool STAGED, bool DOT>
+__device__ __noinline__ void run_slices(Product<V, X>* pr, const SyncArgs* sync, int round, double* red = nullptr) {
   const int lane = threadIdx.x & 31;
   const V *ell_val = pr->ell_val, *er_val = pr->er_val;
   const uint16_t* ell_col = pr->ell_col;
@@ -512,10 +523,16 @@ __device__ __noinline__ void run_slices(Product<V, X>* pr, const SyncArgs* sync,
   int64_t pos = 0, epos = 0;
   int w = 0, we = 0;
   if (i < s1) meta(i, s, pos, w, epos, we);
+  double dacc = 0.0;
   while (i < s1) {
-    int t = 0;
-    if (lane == 0) t = atomicAdd(&pr->counter, 1);
-    const int inxt = s0 + __shfl_sync(FULL, t, 0);
+    int inxt;
+    if constexpr (DOT) {
+      inxt = i + (int)(blockDim.x >> 5);
+    } else {
+      int t = 0;
+      if (lane == 0) t = atomicAdd(&pr->counter, 1);
+      inxt = s0 + __shfl_sync(FULL, t, 0);
+    }
     int nxt = s1;
     int64_t npos = 0, nepos = 0;
     int nw = 0, nwe = 0;
@@ -546,7 +563,8 @@ __device__ __noinline__ void run_slices(Product<V, X>* pr, const SyncArgs* sync,
     if ((lane & (tpr - 1)) == 0 && row < pr->rows) {
       const int m = pr->n2o ? checked(pr->n2o[row] - pr->pb, pr->rows, status) : row;
       pr->out[m] = acc;
-      if (pr->mirror) pr->mirror[m] = acc;
+      if constexpr (DOT) dacc = fma((double)acc, (double)xsl[row], dacc);
+      else if (pr->mirror) pr->mirror[m] = acc;
     }
     i = inxt;
     s = nxt;
@@ -555,6 +573,7 @@ __device__ __noinline__ void run_slices(Product<V, X>* pr, const SyncArgs* sync,
     epos = nepos;
     we = nwe;
   }
+  if constexpr (DOT) red[term_at(threadIdx.x >> 5, lane)] = dacc;
 }
 
 }  // namespace persist
