@@ -10,12 +10,13 @@
 // FP64 operations, and FP64 operations of 32 warps queue for one unit) are one thread's work.
 //
 // The sums are added in the order of the separate launches, so both forms give the same bits; that costs a meeting
-// more an iteration (r.r, below) and a serial chain over the block's warps (p.q: 32 dependent FP64 additions, 1.6
-// us): 35.1 us an iteration at tet 80^3, 33.1 with sums in the blocks' own order, 42 in separate launches. Whole
-// solves of (A + 0.1 mean diagonal) x = b to 1e-10, separate launches -> persistent, FP64 CG (44 to 65 iterations):
-// tet 40^3 1.10 -> 0.82 ms, 80^3 2.10 -> 1.77, 126^3 4.62 -> 4.48, elasticity 24^3 2.14 -> 1.46, 40^3 3.87 -> 3.43,
-// 64^3 9.32 -> 8.80. Mixed-precision PCG (1e-9): tet 80^3 1.77 -> 1.33, elasticity 40^3 3.55 -> 2.93, 64^3 7.32 ->
-// 6.89; FP64 PCG: tet 80^3 1.74 -> 1.32, elasticity 64^3 9.88 -> 9.33.
+// more an iteration (r.r, below) and a serial chain over the block's warps (p.q: 32 dependent FP64 additions, 1.6 us):
+// 35.1 us an iteration at tet 80^3, 31 with sums in the blocks' own order, 43 in separate launches.
+// Whole solves of (A + 0.1 mean diagonal) x = b to 1e-10, separate launches -> persistent, FP64 CG (44 to 65
+// iterations): tet 40^3 1.12 -> 0.79 ms, 80^3 2.10 -> 1.76, 126^3 4.63 -> 4.48, elasticity 24^3 2.11 -> 1.50, 40^3 3.88 ->
+// 3.43, 64^3 9.32 -> 8.80.  FP32 CG (refinement): tet 40^3 1.61 -> 1.09, 101^3 3.25 -> 2.91, elasticity 64^3 7.88 -> 7.52.
+// Mixed-precision PCG (1e-9): tet 80^3 1.77 -> 1.33, elasticity 40^3 3.55 -> 2.94, 64^3 7.32 -> 6.71; FP64 PCG: tet 80^3
+// 1.74 -> 1.30, elasticity 64^3 9.88 -> 9.31.
 #pragma once
 #include <algorithm>
 
@@ -26,7 +27,7 @@ namespace persist {
 
 using namespace core;
 
-constexpr int kMaxGrid = 160;      // blocks of a persistent launch (five partial sums per gathering lane)
+constexpr int kMaxGrid = 160;  // blocks of a persistent launch
 // Least time limit (wait_timeout_ns) with which solvers iterate persistently: the others' work, or another process's
 // time slice, may keep a block waiting for milliseconds.  Plans with a shorter one take the separate launches, which
 // have no such waits.
