@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "ehyb_core.cuh"
 #include "plan_internal.h"
@@ -114,15 +115,42 @@ __global__ void __launch_bounds__(512) spmm_kernel(KArgs a, const double* __rest
         for (int j = 0; j < KC; ++j) q[j] = fma(v, xr[j], q[j]);
       }
     };
+    // N extra-row slots from kk on: their columns, then their rows of X, then the FMAs in slot order.  The loads of X
+    // keep their order (load_x), so slot by slot each waited for its column and its row in turn; a small plan's few
+    // warps cannot hide that, nor a long slice's chain (us, k = 2 / 3 / 8 / 16, slot by slot -> in batches: power-law
+    // 12k rows 476 / 650 / 920 / 1840 -> 314 / 463 / 582 / 1163, elasticity 20^3 34.6 / 72.7 / 64.1 / 127 -> 31.3 /
+    // 69.6 / 55.8 / 111, tet 40^3 13.1 / 25.8 / 22.0 / 44.5 -> 10.0 / 23.0 / 20.4 / 41.0).
+    auto batch = [&](auto count, int kk, double (&q)[KC]) {
+      constexpr int N = decltype(count)::value;
+      double v[N];
+      int64_t c[N];
+      RowCols<KC, VEC> xr[N];
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        v[u] = __ldcs(evp + 32 * (int64_t)(kk + u));
+        c[u] = (int64_t)checked(__ldcs(ecp + 32 * (int64_t)(kk + u)), a.n, a.status) * k;
+      }
+#pragma unroll
+      for (int u = 0; u < N; ++u) xr[u].ldg(Xc + c[u]);
+#pragma unroll
+      for (int u = 0; u < N; ++u)
+#pragma unroll
+        for (int j = 0; j < KC; ++j) q[j] = fma(v[u], xr[u].v[j], q[j]);
+    };
     // extra-row slots [k0, k1)
     auto extra = [&](int k0, int k1, double (&q)[KC]) {
-      for (int kk = k0; kk < k1; ++kk) {
-        const double v = __ldcs(evp + 32 * (int64_t)kk);
-        RowCols<KC, VEC> xr;
-        xr.ldg(Xc + (int64_t)checked(__ldcs(ecp + 32 * (int64_t)kk), a.n, a.status) * k);
-#pragma unroll
-        for (int j = 0; j < KC; ++j) q[j] = fma(v, xr.v[j], q[j]);
+      constexpr int N = KC == 8 ? 4 : KC == 4 ? 6 : KC == 2 ? 12 : 12;
+      int kk = k0;
+#pragma unroll 1
+      for (; kk + N <= k1; kk += N) batch(std::integral_constant<int, N>(), kk, q);
+      if constexpr (N > 4)
+#pragma unroll 1
+        for (; kk + 4 <= k1; kk += 4) batch(std::integral_constant<int, 4>(), kk, q);
+      if (kk + 2 <= k1) {
+        batch(std::integral_constant<int, 2>(), kk, q);
+        kk += 2;
       }
+      if (kk < k1) batch(std::integral_constant<int, 1>(), kk, q);
     };
     const int cap = a.wide_parts > 0 ? kWideCap : 0x7fffffff;
     slab(0, min(w, cap), acc);
