@@ -978,12 +978,19 @@ struct SlabHead<V, X, R, true> {
 // Partition p with one slice per warp (er_layout 0, no wide slices, blockDim.x >= the partition's rows); x and y as in
 // partition_spmv, gathered and scattered through new_to_old with GATHER, in the plan's numbering without.
 // R slab and 4 extra-row slots are held from before the wait; R is also the depth of the loops over the rest.
+// The next grid may come after the wait (FP64) or at once.  Let in at once it lets in the one after it too, and several
+// grids of waiting blocks share the SMs unevenly with the one at work (FP64, back to back, at once -> after the wait:
+// 2D 4,900 rows 3.84 -> 3.46 us, tets 10,648 rows 5.74 -> 4.52, elasticity 17k rows 10.3 -> 7.7; elsewhere within 0.2
+// us); on FP32 / BF16 values that was not seen, and the later start costs them up to a tenth.
+template <typename V>
+constexpr bool kLateTrigger = sizeof(V) == 8;
 template <typename V, typename X, bool GATHER, bool RUNS, int R>
 __device__ __forceinline__ void small_partition_spmv(const KArgs& a, const V* __restrict__ ell_val,
                                                      const V* __restrict__ er_val, const X* __restrict__ xp,
                                                      X* __restrict__ y, const int p, X* xs) {
   constexpr int E = 4;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if constexpr (!kLateTrigger<V>) pdl_launch_dependents();
   const int pb = a.part_ptr[p], rows = a.part_ptr[p + 1] - pb;
   const int s = a.slice_ptr[p] + warp;
   const bool on = s < a.slice_ptr[p + 1];
@@ -1021,6 +1028,7 @@ __device__ __forceinline__ void small_partition_spmv(const KArgs& a, const V* __
     }
   }
   pdl_wait();
+  if constexpr (kLateTrigger<V>) pdl_launch_dependents();
   X xe[E];
 #pragma unroll
   for (int u = 0; u < E; ++u) xe[u] = u < we ? load_x(xp + ec[u]) : X(0);

@@ -52,7 +52,6 @@ __global__ void __launch_bounds__(MAXT, 1) ehyb_small_kernel(KArgs a, const V* _
                                                           const V* __restrict__ er_val, const X* __restrict__ xp,
                                                           X* __restrict__ y) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_launch_dependents();
   small_partition_spmv<V, X, GATHER, RUNS, 8192 / MAXT>(a, ell_val, er_val, xp, y, blockIdx.x,
                                                                 reinterpret_cast<X*>(smem_raw));
 }
